@@ -203,6 +203,8 @@ struct rslb_handle {
   void* F[3];
   // tables in working precision
   void* t_mw;
+  void* t_m3;
+  void* t_pk;
   void* t_xi;
   void* t_wp;
   void* t_L1k;
@@ -237,6 +239,8 @@ template <typename T>
 SodTables<T> tables_of(const rslb_handle* h) {
   SodTables<T> tb;
   tb.mw = (const T*)h->t_mw;
+  tb.m3 = (const T*)h->t_m3;
+  tb.pk = (const T*)h->t_pk;
   tb.xi = (const T*)h->t_xi;
   tb.wp = (const T*)h->t_wp;
   tb.kidx = h->t_kidx;
@@ -263,7 +267,7 @@ SodTablesF64 tables64_of(const rslb_handle* h) {
 void free_handle(rslb_handle* h) {
   if (!h) return;
   if (h->graph) cudaGraphExecDestroy(h->graph);
-  void* ptrs[] = {h->F[0], h->F[1], h->F[2], h->t_mw, h->t_xi, h->t_wp, h->t_L1k, h->t_gL,
+  void* ptrs[] = {h->F[0], h->F[1], h->F[2], h->t_mw, h->t_m3, h->t_pk, h->t_xi, h->t_wp, h->t_L1k, h->t_gL,
                   h->t_gR, h->t_kidx, h->t_rowv, h->t_gl_t, h->t_gl_w, h->d_xi, h->d_p, h->d_wp,
                   h->d_L1k, h->d_mom, h->d_err, h->d_fields};
   for (void* p : ptrs)
@@ -355,7 +359,9 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   ce = sod_set_attributes();
   if (ce != cudaSuccess) return cuda_error(ce, "rslb_init: kernel attributes");
   const bool fp64 = c.precision == RSLB_F64;
-  SodLaunch L = sod_pick_launch(fp64, V, QL, nm, max_smem);
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  SodLaunch L = sod_pick_launch(fp64, V, QL, nm, max_smem, c.Z, nsm);
   if (c.tile_cells != 0) {
     // explicit tile width (tuning): must be one the kernels are built for
     const bool okB = fp64 ? (c.tile_cells == 16 || c.tile_cells == 8)
@@ -384,9 +390,6 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
     gq.V = V;
     gq.QL = QL;
     gq.nm = nm;
-    int nsm = 0;
-    ce = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (ce != cudaSuccess) return cuda_error(ce, "rslb_init: SM count");
     if (!sod32p_fits(gq, max_smem))
       return set_error(RSLB_ERR_ARG,
                        "rslb_init: the persistent packed kernel does not fit (V = %d, Z = %d)", V,
@@ -419,11 +422,12 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   g.inv_dz = 1.0 / dz;
   g.dt = c.dt;
   g.tau = c.tau;
+  g.dt_tau = c.tau_mode == RSLB_TAU_CONST ? c.dt / c.tau : 0.0;
   g.tau_AW0 = c.tau_AW0;
   g.lambda_ref = c.lambda_ref;
 
   // velocity tables (FP64 on the host)
-  std::vector<double> mw(5 * (size_t)V), xiv(V), pv(V), wp(kMaxM * (size_t)V, 0.0), L1k(QL);
+  std::vector<double> mw(5 * (size_t)V), m3(4 * (size_t)V, 0.0), xiv(V), pv(V), wp(kMaxM * (size_t)V, 0.0), L1k(QL);
   std::vector<int> kidx(V);
   for (int k = 0; k < QL; ++k) {
     L1k[k] = 3.0 - xk[k];
@@ -435,6 +439,9 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
       mw[2 * V + v] = p * (1.0 + x) * (1.0 + x);
       mw[3 * V + v] = p * (1.0 - x) * (1.0 - x);
       mw[4 * V + v] = p * (1.0 - x) * (1.0 + x);
+      m3[4 * (size_t)v] = (1.0 + x) * (1.0 + x);
+      m3[4 * (size_t)v + 1] = (1.0 - x) * (1.0 - x);
+      m3[4 * (size_t)v + 2] = (1.0 - x) * (1.0 + x);
       xiv[v] = x;
       pv[v] = p;
       kidx[v] = k;
@@ -455,6 +462,15 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
     return fp64 ? upload<double>(dst, src) : upload<float>(dst, src);
   };
   if (!rc) rc = up(&h->t_mw, mw);
+  if (!rc) rc = up(&h->t_m3, m3);
+  if (!rc) {
+    std::vector<double> pk(2 * (size_t)QL);  // p_k as hi + lo in the working precision
+    for (int k = 0; k < QL; ++k) {
+      pk[2 * k] = fp64 ? xk[k] : (double)(float)xk[k];
+      pk[2 * k + 1] = xk[k] - pk[2 * k];
+    }
+    rc = up(&h->t_pk, pk);
+  }
   if (!rc) rc = up(&h->t_xi, xiv);
   if (!rc) rc = up(&h->t_wp, wp);
   if (!rc) rc = up(&h->t_L1k, L1k);
@@ -743,7 +759,7 @@ extern "C" void rslb_destroy(rslb_handle* h) {
 // Batches of shock tubes
 // ---------------------------------------------------------------------------
 struct SodClass {
-  int V, nm, B, ctas_per_sm;
+  int V, QL, nm, B, ctas_per_sm;
   size_t smem;
   void* runs_dev;  // SodRunDesc<T>[nr]
   SodTask* tasks_dev;
@@ -792,7 +808,7 @@ cudaError_t batch_enqueue(rslb_sod_batch* b, int nsteps) {
       for (const SodClass& c : b->cls) {
         cudaError_t e = sod_batch_stage_launch<T>(
             c.B, c.smem, c.ctas_per_sm * b->nsm, (const SodRunDesc<T>*)c.runs_dev, c.tasks_dev,
-            c.ntasks, b->step_dev, stage, b->err, c.V, b->stream,
+            c.ntasks, b->step_dev, stage, b->err, c.V, c.QL, c.nm, b->stream,
             c.B == kSod32Cells ? c.maps_dev : nullptr);
         if (e != cudaSuccess) return e;
       }
@@ -835,8 +851,9 @@ int batch_build_classes(rslb_sod_batch* b, int autotune) {
     while (j < order.size() && b->h[order[j]]->V == V && b->h[order[j]]->nm == nm) ++j;
     SodClass c{};
     c.V = V;
+    c.QL = QL;
     c.nm = nm;
-    const SodLaunch L = sod_pick_launch(b->fp64, V, QL, nm, max_smem);
+    const SodLaunch L = sod_pick_launch(b->fp64, V, QL, nm, max_smem, 0, 0);
     if (L.B == 0)
       return set_error(RSLB_ERR_UNSUPPORTED, "rslb_sod_batch_init: V = %d does not fit a tile", V);
     c.B = L.B;
@@ -919,12 +936,12 @@ int batch_build_classes(rslb_sod_batch* b, int autotune) {
           cudaEventCreate(&e1);
           // stage 0 reads F0 and writes F1 only: safe to repeat
           sod_batch_stage_launch<T>(B, smem, k * b->nsm, (const SodRunDesc<T>*)c.runs_dev, td,
-                                    (int)tasks.size(), b->step_dev, 0, b->err, V, b->stream,
+                                    (int)tasks.size(), b->step_dev, 0, b->err, V, QL, nm, b->stream,
                                     B == kSod32Cells ? c.maps_dev : nullptr);
           cudaEventRecord(e0, b->stream);
           for (int rep = 0; rep < 3; ++rep)
             sod_batch_stage_launch<T>(B, smem, k * b->nsm, (const SodRunDesc<T>*)c.runs_dev, td,
-                                      (int)tasks.size(), b->step_dev, 0, b->err, V, b->stream,
+                                      (int)tasks.size(), b->step_dev, 0, b->err, V, QL, nm, b->stream,
                                       B == kSod32Cells ? c.maps_dev : nullptr);
           cudaEventRecord(e1, b->stream);
           cudaEventSynchronize(e1);

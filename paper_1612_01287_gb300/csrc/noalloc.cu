@@ -59,7 +59,7 @@ static int noalloc_scratch(void** out) {
 // nodes (the same tables rslb_init uploads; here nothing is allocated).
 template <typename T>
 __global__ void noalloc_tables_kernel(int Qx, int QL, int nm, const double* __restrict__ q,
-                                      T* mw, T* xi, T* wp, int* kidx, int* rowv, T* L1k,
+                                      bool packed, T* mw, T* m3, T* pk, T* xi, T* wp, int* kidx, int* rowv, T* L1k,
                                       double* dxi, double* dp, double* dwp, double* dL1k) {
   // q = [xi(Qx) | w_xi(Qx) | x_k(QL) | w_k(QL)]
   const int V = Qx * QL;
@@ -72,11 +72,18 @@ __global__ void noalloc_tables_kernel(int Qx, int QL, int nm, const double* __re
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
     const int k = v / Qx, j = v - k * Qx;
     const double x = xj[j], p = xk[k];
-    mw[0 * V + v] = T(1.0 + x);
-    mw[1 * V + v] = T(1.0 - x);
-    mw[2 * V + v] = T(p * (1.0 + x) * (1.0 + x));
-    mw[3 * V + v] = T(p * (1.0 - x) * (1.0 - x));
-    mw[4 * V + v] = T(p * (1.0 - x) * (1.0 + x));
+    if (packed) {
+      mw[0 * V + v] = T(1.0 + x);
+      mw[1 * V + v] = T(1.0 - x);
+      mw[2 * V + v] = T(p * (1.0 + x) * (1.0 + x));
+      mw[3 * V + v] = T(p * (1.0 - x) * (1.0 - x));
+      mw[4 * V + v] = T(p * (1.0 - x) * (1.0 + x));
+    } else {
+      m3[4 * v] = T((1.0 + x) * (1.0 + x));
+      m3[4 * v + 1] = T((1.0 - x) * (1.0 - x));
+      m3[4 * v + 2] = T((1.0 - x) * (1.0 + x));
+      m3[4 * v + 3] = T(0);
+    }
     xi[v] = T(x);
     kidx[v] = k;
     dxi[v] = x;
@@ -100,6 +107,8 @@ __global__ void noalloc_tables_kernel(int Qx, int QL, int nm, const double* __re
     rowv[r] = v;
     if (v < QL) {
       L1k[v] = T(3.0 - xk[v]);
+      pk[2 * v] = T(xk[v]);
+      pk[2 * v + 1] = T(xk[v] - double(T(xk[v])));
       dL1k[v] = 3.0 - xk[v];
     }
   }
@@ -119,8 +128,10 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
   };
   const size_t oF0 = take(es * (size_t)V * ldz), oF1 = take(es * (size_t)V * ldz),
                oF2 = take(es * (size_t)V * ldz);
-  const size_t omw = take(es * 5 * V), oxi = take(es * V), owp = take(es * kMaxM * V),
-               oL1 = take(es * kNoAllocMaxQL), ogL = take(es * V), ogR = take(es * V),
+  // one region holds the moment table of the kernel in use: mw [5][V] (packed) or
+  // m3 [V][4] (scalar)
+  const size_t omw = take(es * 5 * V), om3 = omw, oxi = take(es * V), owp = take(es * kMaxM * V),
+               oL1 = take(256), opk = oL1 + 128, ogL = take(es * V), ogR = take(es * V),
                okidx = take(sizeof(int) * V), orow = take(sizeof(int) * V),
                oglt = take(sizeof(double) * kAeqTable), oglw = take(sizeof(double) * kAeqTable),
                odxi = take(sizeof(double) * V), odp = take(sizeof(double) * V),
@@ -154,8 +165,10 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
   cudaError_t qe = cudaGetDevice(&dev);
   if (qe == cudaSuccess)
     qe = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  int nsm = 0;
+  if (qe == cudaSuccess) qe = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (qe != cudaSuccess) return cuda_error(qe, "rslb_sod_step_noalloc: device query");
-  const SodLaunch L = sod_pick_launch(sizeof(T) == 8, V, QL, nm, max_smem);
+  const SodLaunch L = sod_pick_launch(sizeof(T) == 8, V, QL, nm, max_smem, c.Z, nsm);
   if (L.B == 0)
     return set_error(RSLB_ERR_UNSUPPORTED, "rslb_sod_step_noalloc: V = %d does not fit a tile", V);
 
@@ -180,7 +193,8 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
   // tables must be in place before the pageable copies above are reused
   if (ok(cudaSuccess)) {
     noalloc_tables_kernel<T><<<(V + 255) / 256, 256, 0, st>>>(
-        Qx, QL, nm, (const double*)(S + oq), (T*)(S + omw), (T*)(S + oxi), (T*)(S + owp),
+        Qx, QL, nm, (const double*)(S + oq), L.B == kSod32Cells, (T*)(S + omw), (T*)(S + om3), (T*)(S + opk),
+        (T*)(S + oxi), (T*)(S + owp),
         (int*)(S + okidx), (int*)(S + orow), (T*)(S + oL1), (double*)(S + odxi),
         (double*)(S + odp), (double*)(S + odwp), (double*)(S + odL1));
     ok(cudaGetLastError());
@@ -197,6 +211,7 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
   g.inv_dz = 1.0 / dz;
   g.dt = c.dt;
   g.tau = c.tau;
+  g.dt_tau = c.tau_mode == RSLB_TAU_CONST ? c.dt / c.tau : 0.0;
   g.tau_AW0 = c.tau_AW0;
   g.lambda_ref = c.lambda_ref;
   SodTablesF64 t64;
@@ -225,6 +240,8 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
   }
   SodTables<T> tb;
   tb.mw = (const T*)(S + omw);
+  tb.m3 = (const T*)(S + om3);
+  tb.pk = (const T*)(S + opk);
   tb.xi = (const T*)(S + oxi);
   tb.wp = (const T*)(S + owp);
   tb.kidx = (const int*)(S + okidx);

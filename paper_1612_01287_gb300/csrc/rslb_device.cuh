@@ -1,7 +1,6 @@
 // rslb_device.cuh -- device building blocks of the R-SLB step (sm_103a).
 //
-// Landau matching, the WENO5 face flux and the f^eq expansion coefficients,
-// templated on the working precision.  Used by the Sod and Bjorken kernels.
+// Landau matching and the f^eq expansion coefficients, templated on the working precision.  Used by the Sod and Bjorken kernels.
 #pragma once
 
 #include <cfloat>
@@ -22,68 +21,17 @@ constexpr int kAeqTable = kAeqNodes + kAeqNodesF32;
 template <typename T> struct Prec;
 template <> struct Prec<float> {
   static __device__ __forceinline__ float tiny() { return FLT_MIN; }
-  static __device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
+  static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
 };
 template <> struct Prec<double> {
   static __device__ __forceinline__ double tiny() { return DBL_MIN; }
-  static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+  static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 };
 
 __device__ __forceinline__ float dev_exp(float x) { return expf(x); }
 __device__ __forceinline__ double dev_exp(double x) { return exp(x); }
 __device__ __forceinline__ float dev_expm1(float x) { return expm1f(x); }
 __device__ __forceinline__ double dev_expm1(double x) { return expm1(x); }
-
-// ---------------------------------------------------------------------------
-// WENO5 face flux (Sec. III F, Eqs. flux_weno, weno5_omega).
-// (a, b, c, d, e) are the five J = xi f values ordered upwind to downwind
-// around the face: (J_{s-2}, J_{s-1}, J_s, J_{s+1}, J_{s+2}) for xi > 0 and
-// the mirror (J_{s+3}, J_{s+2}, J_{s+1}, J_s, J_{s-1}) for xi < 0.
-// No epsilon: the limiting rules (i)-(iii) decide the weights when smoothness
-// indicators vanish.  The weights are scale-invariant, so sigma_q is divided
-// by max_q sigma_q first; a ratio whose square is below the smallest normal
-// number of T counts as a vanishing sigma_q.  Branch-free, one reciprocal
-// for the scale and one for the normalisation.
-// ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ T weno5_face(T a, T b, T c, T d, T e) {
-  const T c6 = T(1) / T(6);
-  const T F1 = (T(2) * a - T(7) * b + T(11) * c) * c6;
-  const T F2 = (-b + T(5) * c + T(2) * d) * c6;
-  const T F3 = (T(2) * c + T(5) * d - e) * c6;
-  const T k13 = T(13) / T(12);
-  const T d1 = a - T(2) * b + c, e1 = a - T(4) * b + T(3) * c;
-  const T d2 = b - T(2) * c + d, e2 = b - d;
-  const T d3 = c - T(2) * d + e, e3 = T(3) * c - T(4) * d + e;
-  const T s1 = k13 * d1 * d1 + T(0.25) * e1 * e1;
-  const T s2 = k13 * d2 * d2 + T(0.25) * e2 * e2;
-  const T s3 = k13 * d3 * d3 + T(0.25) * e3 * e3;
-  const T D1 = T(0.1), D2 = T(0.6), D3 = T(0.3);
-  const bool alleq = (s1 == s2) && (s2 == s3);
-  const T smax = fmax(s1, fmax(s2, s3));
-  const T inv = alleq ? T(0) : Prec<T>::rcp(smax);
-  const T r1 = s1 * inv, r2 = s2 * inv, r3 = s3 * inv;
-  const T t1 = r1 * r1, t2 = r2 * r2, t3 = r3 * r3;
-  const T tiny = Prec<T>::tiny();
-  const bool z1 = t1 < tiny, z2 = t2 < tiny, z3 = t3 < tiny;
-  const int nz = int(z1) + int(z2) + int(z3);
-  // general case: omega_q ~ delta_q / sigma_q^2, multiplied through by the
-  // product of all three t's
-  const T n1 = D1 * t2 * t3, n2 = D2 * t1 * t3, n3 = D3 * t1 * t2;
-  const T dz = (z1 ? D1 : T(0)) + (z2 ? D2 : T(0)) + (z3 ? D3 : T(0));
-  const T den = (nz == 0) ? (n1 + n2 + n3) : ((nz == 1) ? T(1) : dz);
-  const T rden = Prec<T>::rcp(den);
-  T w1, w2, w3;
-  if (nz == 0) {
-    w1 = n1 * rden; w2 = n2 * rden; w3 = n3 * rden;
-  } else if (nz == 1) {  // rule (iii)
-    w1 = z1 ? T(1) : T(0); w2 = z2 ? T(1) : T(0); w3 = z3 ? T(1) : T(0);
-  } else {  // rule (ii): the vanishing ones share delta_q / sum
-    w1 = z1 ? D1 * rden : T(0); w2 = z2 ? D2 * rden : T(0); w3 = z3 ? D3 * rden : T(0);
-  }
-  if (alleq) { w1 = D1; w2 = D2; w3 = D3; }  // rule (i)
-  return w1 * F1 + w2 * F2 + w3 * F3;
-}
 
 // ---------------------------------------------------------------------------
 // Landau frame of the 1-D stress tensor (Sec. II E, Eqs. E_landau, u_landau),
@@ -99,26 +47,43 @@ __device__ __forceinline__ T weno5_face(T a, T b, T c, T d, T e) {
 // ---------------------------------------------------------------------------
 struct LandauOut {
   double n, E, T, beta, gamma, u;  // u = gamma |beta|
+  double ub;                       // gamma beta (signed)
   bool ok;
 };
+
+// 1/x and 1/sqrt(x) in FP64 from the 20-bit hardware seeds and one step of
+// Householder's third-order iteration (e = 1 - x y or 1 - x y^2; the residual
+// is of order e^3 < 2^-57, so the result is within about an ulp).  GB300 issues
+// ~2 FP64 lane operations per SM and cycle, so these 3 and 5 operations
+// replace the ~10-20 of the IEEE division and square root.  x must be a
+// positive normal number; other inputs give inf or NaN, which the callers'
+// range checks reject.
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
 __device__ __forceinline__ LandauOut landau_factored(double Np, double Nm, double Ap,
                                                      double Am, double D) {
   LandauOut o;
-  const double a = sqrt(Ap), b = sqrt(Am);
-  const double ab = a * b, apb = a + b;
-  const double sab = sqrt(ab);
-  const double X = b * Np + a * Nm;
-  // one FP64 division (slow on this part) gives 1/(2 sqrt(ab)), 1/(a+b) and
-  // 1/X: r = 1/(sqrt(ab) (a+b) X)
-  const double r = 1.0 / (sab * apb * X);
-  const double h = 0.5 * apb * X * r;  // 1/(2 sqrt(ab))
-  o.E = 0.5 * (D + ab);
-  o.beta = (a - b) * sab * X * r;      // (a - b)/(a + b)
+  const double a = Ap * rsqrt64(Ap), b = Am * rsqrt64(Am);  // square roots
+  const double ab = a * b, apb = a + b, amb = a - b;
+  const double h = 0.5 * rsqrt64(ab);  // 1/(2 sqrt(ab))
+  o.E = fma(0.5, ab, 0.5 * D);
+  o.beta = amb * rcp64(apb);
   o.gamma = apb * h;
-  o.u = fabs(a - b) * h;
-  o.n = X * h;
-  o.T = (2.0 / 3.0) * o.E * ab * apb * r;  // E/(3n) = 2 E sqrt(ab)/(3X)
+  o.ub = amb * h;
+  o.u = fabs(o.ub);
+  o.n = fma(b, Np, a * Nm) * h;
+  o.T = o.E * rcp64(3.0 * o.n);
   o.ok = (Ap > 0.0) && (Am > 0.0) && (o.E > 0.0) && (o.n > 0.0) && isfinite(o.E) &&
          isfinite(o.n) && isfinite(o.beta) && (fabs(o.beta) < 1.0);
   return o;
@@ -157,6 +122,113 @@ __device__ __forceinline__ void aeq_node(T t, T wt, T A, T sh2, T uinv, bool at_
       p1 = p2;
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// The same integrals by recurrence over m (stage kernels).  With z = 1/|beta|,
+//   X3_m = (A/u) J3_m = int P_m(c) (u0 - u c)^{-3} dc,   X4_m likewise with -4,
+// are the second and third derivatives of the Legendre function Q_m(z) up to
+// a factor, i.e. the minimal solutions of
+//   (m+2) D_{m-1} = (2m+1) z D_m - (m-1) D_{m+1},
+//   (m+3) E_{m-1} = (2m+1) z E_m - (m-2) E_{m+1}
+// (associated Legendre recurrence), so the downward recurrence from a large
+// order (Miller's algorithm) is stable.  Writing D_m = beta^m S_m delta_m with
+// S_{m-1} = S_{m+1} (m-1)/(m+2) leaves
+//   delta_{m-1} = alpha_m delta_m - beta^2 delta_{m+1}
+// (two operations per order), regular at beta = 0, and the same form for E; the
+// norms are X3_0 = 2 u0 and X4_0 = 2 u0^2 + 2 u^2/3.  The starting order
+// follows from the decay rate rho = (1 + sqrt(1 - beta^2))/|beta| of D_{m+1}/D_m;
+// all m agree with the integrals to ~3e-16 of X_0 (FP64) up to |beta| = 0.99.
+// ~20 orders of 4 operations replace 32 (16) nodes with an exp, an expm1 and
+// 13 Legendre orders each.
+// ---------------------------------------------------------------------------
+constexpr int kAeqSteps = 128;  // largest starting order
+struct AeqTab {
+  double aD[kAeqSteps + 2], aE[kAeqSteps + 2];  // alpha_m of the two recurrences
+  double sD[kMaxM + 1], sE[kMaxM + 1];          // S_m
+  float aDf[kAeqSteps + 2], aEf[kAeqSteps + 2], sDf[kMaxM + 1], sEf[kMaxM + 1];
+};
+constexpr AeqTab make_aeq_tab() {
+  AeqTab t{};
+  double SD[kAeqSteps + 3] = {}, SE[kAeqSteps + 3] = {};
+  SD[0] = SD[1] = SD[2] = 1.0;
+  SE[0] = SE[1] = SE[2] = SE[3] = 1.0;
+  for (int m = 2; m <= kAeqSteps + 1; ++m) SD[m + 1] = SD[m - 1] * (m + 2) / (m - 1);
+  for (int m = 3; m <= kAeqSteps + 1; ++m) SE[m + 1] = SE[m - 1] * (m + 3) / (m - 2);
+  for (int m = 2; m <= kAeqSteps + 1; ++m) t.aD[m] = (2.0 * m + 1) / (m + 2) * (SD[m] / SD[m - 1]);
+  for (int m = 3; m <= kAeqSteps + 1; ++m) t.aE[m] = (2.0 * m + 1) / (m + 3) * (SE[m] / SE[m - 1]);
+  for (int m = 0; m <= kMaxM; ++m) {
+    t.sD[m] = SD[m];
+    t.sE[m] = SE[m];
+    t.sDf[m] = float(SD[m]);
+    t.sEf[m] = float(SE[m]);
+  }
+  for (int m = 0; m <= kAeqSteps + 1; ++m) {
+    t.aDf[m] = float(t.aD[m]);
+    t.aEf[m] = float(t.aE[m]);
+  }
+  return t;
+}
+static __constant__ AeqTab c_aeq = make_aeq_tab();
+
+template <typename T>
+__device__ __forceinline__ T aeq_alpha(bool e, int m);
+template <>
+__device__ __forceinline__ float aeq_alpha<float>(bool e, int m) {
+  return e ? c_aeq.aEf[m] : c_aeq.aDf[m];
+}
+template <>
+__device__ __forceinline__ double aeq_alpha<double>(bool e, int m) {
+  return e ? c_aeq.aE[m] : c_aeq.aD[m];
+}
+template <typename T>
+__device__ __forceinline__ T aeq_scale(bool e, int m);
+template <>
+__device__ __forceinline__ float aeq_scale<float>(bool e, int m) {
+  return e ? c_aeq.sEf[m] : c_aeq.sDf[m];
+}
+template <>
+__device__ __forceinline__ double aeq_scale<double>(bool e, int m) {
+  return e ? c_aeq.sE[m] : c_aeq.sD[m];
+}
+
+// Starting order for truncation nm (>= 4 here) at u = gamma |beta|, and the
+// starting ratio delta_{M+1}/delta_M ~ 1/(1 + 1/gamma).  The truncation error
+// falls by rho^-2 per order: 17/ln(rho) orders for FP64, 8/ln(rho) for FP32.
+// Past kAeqSteps (FP32: 96, so that the growth of at most 2 per order stays
+// in range) the caller uses the quadrature.
+template <typename T>
+__device__ __forceinline__ int aeq_start(float u, float gamma, int nm4, float* r) {
+  *r = gamma / (gamma + 1.f);
+  const float l2 = fmaxf(-__log2f(fmaxf(u / (gamma + 1.f), 1e-30f)), 1e-6f);  // log2(rho)
+  const float need = (sizeof(T) == 8 ? 24.53f : 11.55f) / l2;
+  const int M = nm4 + (int)fminf(need, 4096.f);
+  return M;
+}
+template <typename T>
+__host__ __device__ constexpr int aeq_max_start() { return sizeof(T) == 8 ? kAeqSteps : 96; }
+
+// delta_m for 2 <= m < nm4 (nm4 = max(nm, 4)), and delta_1 for the D chain,
+// handed to put(m, delta).  All lanes of the warp run from the largest
+// starting order among them, so that alpha is read uniformly.
+template <typename T, typename Put>
+__device__ __forceinline__ void aeq_chain(bool e_chain, T b2, T r, int M, int nm4, Put put) {
+  T d1 = r, d0 = T(1);  // delta_{m+1}, delta_m
+  for (int m = M; m >= nm4; --m) {
+    const T dn = fma(-b2, d1, aeq_alpha<T>(e_chain, m) * d0);
+    d1 = d0;
+    d0 = dn;
+  }
+#pragma unroll
+  for (int m = kMaxM - 1 < 3 ? 3 : kMaxM - 1; m >= 3; --m)
+    if (m < nm4) {
+      put(m, d0);
+      const T dn = fma(-b2, d1, aeq_alpha<T>(e_chain, m) * d0);
+      d1 = d0;
+      d0 = dn;
+    }
+  put(2, d0);
+  if (!e_chain) put(1, fma(-b2, d1, aeq_alpha<T>(false, 2) * d0));
 }
 
 // One level of a transposing warp reduction of 32 compensated (hi, lo)

@@ -5,17 +5,15 @@
 //   1. the tile plus a 4-cell halo on each side is staged in shared memory
 //      with 16-byte cp.async copies (velocity-major rows; boundary tiles map
 //      out-of-domain cells through the boundary condition);
-//   2. moments: the five sums of the factored Landau form.  Up to 128
-//      velocities one lane per (cell, sum) adds every row itself (blocks of
-//      four rows, Kahan-compensated in FP32); above that each warp owns a
-//      16-byte column chunk of cells, its lanes own velocity rows, and an
-//      error-free FP32 transposing warp reduction (FP64 shuffles for FP64
-//      populations) combines the lanes;
+//   2. moments: the five sums of the factored Landau form, from three sums per
+//      radial node.  A thread owns one cell and a slice of the rows (blocks of
+//      four rows, Kahan-compensated in FP32); the slices of a cell meet by
+//      shuffles and in shared memory (double-floats in FP32);
 //   3. per cell: Landau matching in FP64 (Sec. II E), the relaxation time, and
-//      the f^eq expansion coefficients (Sec. III D) by a Gauss-Legendre rule
-//      spread over the CTA and reduced by shuffles;
+//      the f^eq expansion coefficients (Sec. III D) by a downward recurrence
+//      over the Legendre order;
 //   4. per (velocity, cell): the WENO5 flux difference (Sec. III F) along the
-//      row, written in terms of first and second differences of J = xi f so
+//      row, written in terms of first and second differences of f so
 //      that a sliding window shares them between neighbouring faces; f^eq
 //      from the per-cell coefficients; Anderson-Witting relaxation
 //      (Eq. L_Sod); the RK combination.  Rows are visited negative-xi first so
@@ -26,6 +24,16 @@
 //      stages 2 and 3).
 // Shared-memory rows have a pitch whose 16-byte count is odd, so the 16-byte
 // accesses of eight consecutive rows fall in distinct bank groups.
+//
+// What bounds it: FP64, the FP64 pipe of the SM (~2 lane operations per cycle):
+// ~61 pipe slots per cell and velocity here (moments 4.5, faces 30, differences
+// 7, f^eq 6, update 7, the rest halo and idle lanes), 99 with five moment sums,
+// IEEE divisions, FP64 maxima and predicated-off orders.  65536 x 600: 4.23 ms
+// per stage (7.34 before); 256 x 60 on 2-cell tiles: 18 us (79 on 16-cell
+// tiles with the quadrature for a_{l,m}).  FP32 with few velocities: the
+// latency of the per-cell phases.
+#include <algorithm>
+
 #include "rslb_device.cuh"
 #include "sod.cuh"
 
@@ -33,10 +41,6 @@ namespace rslb {
 
 constexpr int kMaxQL = 8;
 constexpr int kHalo = 4;
-constexpr int kMaxMP = 16;  // kMaxM rounded up to a whole number of 16-byte vectors
-// Up to this many velocities each moment is summed by one lane over all rows;
-// above it the lanes of a warp take rows and a warp reduction follows.
-constexpr int kSerialMomentRows = 128;
 
 template <typename T> struct V16;
 template <> struct V16<float> {
@@ -63,11 +67,13 @@ __host__ __device__ inline int coef_pitch(int nm) {
   return (nm + n - 1) / n * n;
 }
 
-// Shared-memory carve-up of one CTA (all offsets 16-byte aligned).
+// Shared-memory carve-up of one CTA (all offsets 16-byte aligned).  np partial
+// slots of the moment sums follow the fixed part; with np = 0 the groups add
+// into msum one after another.
 template <typename T>
 struct SodSmem {
-  size_t tile, outb, msum, cell, coef, gco, total;
-  __host__ __device__ SodSmem(int V, int B, int QL, int nm, bool seg) {
+  size_t tile, outb, msum, cell, coef, gco, part, total;
+  __host__ __device__ SodSmem(int V, int B, int QL, int nm, bool seg, int np) {
     auto al = [](size_t x) { return (x + 15) & ~size_t(15); };
     const int P = tile_pitch<T>(B + 2 * kHalo);
     tile = 0;
@@ -76,7 +82,8 @@ struct SodSmem {
     cell = msum + al(sizeof(double) * 5 * B);
     coef = cell + al(sizeof(double) * 8 * B);
     gco = coef + al(sizeof(T) * (size_t)QL * B * coef_pitch<T>(nm));
-    total = gco + al(sizeof(T) * 2 * B);
+    part = gco + al(sizeof(T) * 2 * B);
+    total = part + al(sizeof(double) * 5 * (size_t)np * B);
   }
 };
 
@@ -84,18 +91,11 @@ __device__ __forceinline__ void report_error(int* err, int code, int cell) {
   if (atomicCAS(err, 0, code) == 0) err[1] = cell;
 }
 
-__device__ __forceinline__ double warp_sum(double x) {
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-  return x;
-}
-
 __device__ __forceinline__ float fast_rcp(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-__device__ __forceinline__ double fast_rcp(double x) { return 1.0 / x; }
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -118,67 +118,183 @@ __device__ __forceinline__ T load_cell(const T* __restrict__ fin, const SodGeom&
   return s < 0 ? tb.ghostL[v] : tb.ghostR[v];
 }
 
-// Kahan-compensated accumulation (FP32) / plain accumulation (FP64).
-template <typename T> struct Acc;
-template <> struct Acc<float> {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float y = x - c;
-    const float t = s + y;
-    c = (t - s) - y;
-    s = t;
+// One thread's share of the moments of one cell.  With a = sum f (1+xi)^2,
+// b = sum f (1-xi)^2 and d = sum f (1-xi^2) over the polar nodes of one radial
+// node p, all with non-negative weights,
+//   N+- = sum_k ({a, b}_k + d_k)/2,  A+- = sum_k p_k {a, b}_k,  D = sum_k p_k d_k
+// ((1 +- xi)^2 + (1 - xi^2) = 2 (1 +- xi)): three products per velocity instead
+// of five, the rest once per radial node (flush).
+template <typename T> struct Moments;
+template <> struct Moments<double> {
+  double S[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  double a = 0.0, b = 0.0, d = 0.0;
+  __device__ __forceinline__ void row(double f, const double* w) {
+    const double2 w01 = __ldg(reinterpret_cast<const double2*>(w));
+    a = fma(f, w01.x, a);
+    b = fma(f, w01.y, b);
+    d = fma(f, __ldg(w + 2), d);
   }
-  __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+  __device__ __forceinline__ void block() {}
+  __device__ __forceinline__ void flush(const double* pk) {
+    const double p = pk[0];
+    S[0] = fma(0.5, a + d, S[0]);
+    S[1] = fma(0.5, b + d, S[1]);
+    S[2] = fma(p, a, S[2]);
+    S[3] = fma(p, b, S[3]);
+    S[4] = fma(p, d, S[4]);
+    a = b = d = 0.0;
+  }
+  __device__ __forceinline__ void merge_xor(int off, unsigned mask) {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) S[q] += __shfl_xor_sync(mask, S[q], off);
+  }
+  __device__ __forceinline__ void put(double* slot, int B, bool add) const {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) slot[q * B] = add ? slot[q * B] + S[q] : S[q];
+  }
+  static __device__ __forceinline__ double total(const double* slot, int B5, int n) {
+    double s = slot[0];
+    for (int i = 1; i < n; ++i) s += slot[(size_t)i * B5];
+    return s;
+  }
 };
-template <> struct Acc<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double x) { s += x; }
-  __device__ __forceinline__ double value() const { return s; }
+// FP32: blocks of four rows, Kahan-compensated across blocks; the radial sums
+// and the groups are added as double-floats (error-free TwoSum and products).
+template <> struct Moments<float> {
+  float H[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, L[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  float s[3] = {0.f, 0.f, 0.f}, c[3] = {0.f, 0.f, 0.f}, k[3] = {0.f, 0.f, 0.f};
+  static __device__ __forceinline__ void two_sum(float& h, float& l, float x) {
+    const float t = h + x, bp = t - h;
+    l += (h - (t - bp)) + (x - bp);
+    h = t;
+  }
+  __device__ __forceinline__ void row(float f, const float* w) {
+    const float4 w4 = __ldg(reinterpret_cast<const float4*>(w));
+    k[0] = fmaf(f, w4.x, k[0]);
+    k[1] = fmaf(f, w4.y, k[1]);
+    k[2] = fmaf(f, w4.z, k[2]);
+  }
+  __device__ __forceinline__ void block() {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const float y = k[q] - c[q];
+      const float t = s[q] + y;
+      c[q] = (t - s[q]) - y;
+      s[q] = t;
+      k[q] = 0.f;
+    }
+  }
+  __device__ __forceinline__ void flush(const float* pk) {
+    block();
+    const float ph = pk[0], pl = pk[1];
+    two_sum(H[0], L[0], 0.5f * s[0]);
+    two_sum(H[0], L[0], 0.5f * s[2]);
+    L[0] -= 0.5f * (c[0] + c[2]);
+    two_sum(H[1], L[1], 0.5f * s[1]);
+    two_sum(H[1], L[1], 0.5f * s[2]);
+    L[1] -= 0.5f * (c[1] + c[2]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const float x = ph * s[q];
+      two_sum(H[2 + q], L[2 + q], x);
+      L[2 + q] += fmaf(ph, s[q], -x) + (pl * s[q] - ph * c[q]);
+      s[q] = c[q] = 0.f;
+    }
+  }
+  __device__ __forceinline__ void merge_xor(int off, unsigned mask) {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      const float h = __shfl_xor_sync(mask, H[q], off), l = __shfl_xor_sync(mask, L[q], off);
+      two_sum(H[q], L[q], h);
+      L[q] += l;
+    }
+  }
+  __device__ __forceinline__ void put(double* slot, int B, bool add) const {
+    float2* f = reinterpret_cast<float2*>(slot);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      float2 v = make_float2(H[q], L[q]);
+      if (add) {
+        v = f[q * B];
+        two_sum(v.x, v.y, H[q]);
+        v.y += L[q];
+      }
+      f[q * B] = v;
+    }
+  }
+  static __device__ __forceinline__ double total(const double* slot, int B5, int n) {
+    const float2* f = reinterpret_cast<const float2*>(slot);
+    float2 v = f[0];
+    for (int i = 1; i < n; ++i) {
+      const float2 x = f[(size_t)i * B5];
+      two_sum(v.x, v.y, x.x);
+      v.y += x.y;
+    }
+    return (double)v.x + (double)v.y;
+  }
 };
 
 // ---------------------------------------------------------------------------
 // WENO5 face correction in difference form.
 // For the upwind-ordered values (a, b, c, d, e) of Sec. III F with first
 // differences D0 = b-a, D1 = c-b, D2 = d-c, D3 = e-d and second differences
-// S1 = a-2b+c, S2 = b-2c+d, S3 = c-2d+e (K_q = 13/12 S_q^2):
-//   sigma_1 = K_1 + (3 D1 - D0)^2/4, sigma_2 = K_2 + (D1 + D2)^2/4,
-//   sigma_3 = K_3 + (D3 - 3 D2)^2/4,
+// S1 = a-2b+c, S2 = b-2c+d, S3 = c-2d+e (K_q = 13/3 S_q^2):
+//   4 sigma_1 = K_1 + (3 D1 - D0)^2, 4 sigma_2 = K_2 + (D1 + D2)^2,
+//   4 sigma_3 = K_3 + (D3 - 3 D2)^2,
 //   F^q = c + g_q/6 with g_1 = 5 D1 - 2 D0, g_2 = D1 + 2 D2, g_3 = 4 D2 - D3,
-// so F = c + (omega . g)/6.  With omega_q ~ delta_q / sigma_q^2 multiplied
+// so F = c + (omega . g)/6 (the common factor 4 of the indicators cancels in the
+// weights).  With omega_q ~ delta_q / sigma_q^2 multiplied
 // through by prod_p (sigma_p/sigma_max)^2, the limiting rules (i)-(iii) of
 // the paper all reduce to "correction = 0" when every product vanishes (the
 // g_q of the vanishing stencils are exactly zero there), and rule (iii) is
-// the natural limit of the formula.  Returns (omega . g) (without the 1/6).
+// the natural limit of the formula.  The products are taken in the ratio
+// 1/3 : 2 : 1 of delta_q.  Returns (omega . g) (without the 1/6).  26 FP64
+// operations per face; the scaling and the zero test are integer work on the
+// high words, which the FP64 pipe (the FP64 kernel's limit) does not see.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void weno_scale(float& s1, float& s2, float& s3) {
+  // the power of two at or below the maximum, from the exponent bits; a zero
+  // or subnormal maximum gives the largest such power, which keeps zero
+  // indicators zero and brings subnormal ones into range
+  const float smax = fmaxf(s1, fmaxf(s2, s3));
+  const float inv = __int_as_float(0x7F000000 - (__float_as_int(smax) & 0x7F800000));
+  s1 *= inv;
+  s2 *= inv;
+  s3 *= inv;
+}
+__device__ __forceinline__ void weno_scale(double& s1, double& s2, double& s3) {
+  // the same by subtracting the exponent of the maximum from the high words
+  // (the indicators are >= 0, so their high words order like integers); a
+  // word that would fall below zero becomes a subnormal, whose square is 0.
+  // Indicators all below ~1e-231 are left alone: their squares vanish.
+  const int h1 = __double2hiint(s1), h2 = __double2hiint(s2), h3 = __double2hiint(s3);
+  const int em = max(h1, max(h2, h3)) & 0x7FF00000;
+  const int sh = em < 0x10000000 ? 0 : em - 0x3FF00000;
+  s1 = __hiloint2double(max(h1 - sh, 0), __double2loint(s1));
+  s2 = __hiloint2double(max(h2 - sh, 0), __double2loint(s2));
+  s3 = __hiloint2double(max(h3 - sh, 0), __double2loint(s3));
+}
+// num/den, 0 where den is below the smallest normal number (the reciprocals
+// flush subnormal inputs, and a vanishing denominator means a vanishing correction)
+__device__ __forceinline__ float weno_quotient(float num, float den) {
+  return den > Prec<float>::tiny() ? num * fast_rcp(den) : 0.f;
+}
+__device__ __forceinline__ double weno_quotient(double num, double den) {
+  return __double2hiint(den) >= 0x00100000 ? num * rcp64(den) : 0.0;
+}
+
 template <typename T>
 __device__ __forceinline__ T weno_corr(T D0, T D1, T D2, T D3, T K1, T K2, T K3) {
-  const T e1 = T(3) * D1 - D0, e2 = D1 + D2, e3 = D3 - T(3) * D2;
-  const T s1 = K1 + T(0.25) * e1 * e1;
-  const T s2 = K2 + T(0.25) * e2 * e2;
-  const T s3 = K3 + T(0.25) * e3 * e3;
-  const T g1 = T(5) * D1 - T(2) * D0, g2 = D1 + T(2) * D2, g3 = T(4) * D2 - D3;
-  // A denominator below the smallest normal number counts as zero: the FP32
-  // reciprocal flushes subnormal inputs, and a vanishing denominator means
-  // the correction vanishes (limit rules).
-  // The indicators are scaled by the power of two at or below their maximum
-  // (the weights are homogeneous in sigma; the scaling only keeps the fourth
-  // powers in range), formed from the exponent bits with an AND and a
-  // subtract; a zero or subnormal maximum gives the largest such power, which
-  // keeps zero indicators zero and brings subnormal ones into range.
-  const T tiny = Prec<T>::tiny();
-  const T smax = fmax(s1, fmax(s2, s3));
-  T inv;
-  if constexpr (sizeof(T) == 4)
-    inv = __int_as_float(0x7F000000 - (__float_as_int(smax) & 0x7F800000));
-  else
-    inv = __longlong_as_double(0x7FE0000000000000LL -
-                               (__double_as_longlong(smax) & 0x7FF0000000000000LL));
-  const T r1 = s1 * inv, r2 = s2 * inv, r3 = s3 * inv;
-  const T t1 = r1 * r1, t2 = r2 * r2, t3 = r3 * r3;
-  const T n1 = T(0.1) * (t2 * t3), n2 = T(0.6) * (t1 * t3), n3 = T(0.3) * (t1 * t2);
-  const T den = n1 + n2 + n3;
-  const T num = n1 * g1 + n2 * g2 + n3 * g3;
-  return den > tiny ? num * fast_rcp(den) : T(0);
+  const T e1 = fma(T(3), D1, -D0), e2 = D1 + D2, e3 = fma(T(-3), D2, D3);
+  T s1 = fma(e1, e1, K1), s2 = fma(e2, e2, K2), s3 = fma(e3, e3, K3);
+  weno_scale(s1, s2, s3);
+  const T t1 = s1 * s1, t2 = s2 * s2, t3 = s3 * s3;
+  const T p13 = t1 * t3, n3 = t1 * t2;
+  const T n2 = p13 + p13, n1 = t2 * t3 * T(1.0 / 3.0);
+  const T den = (n3 + n2) + n1;
+  // g_1 = 2 e1 - D1, g_2 = e2 + D2, g_3 = D2 - e3
+  const T num = fma(n1, fma(T(2), e1, -D1), fma(n2, e2 + D2, n3 * (D2 - e3)));
+  return weno_quotient(num, den);
 }
 
 // 16-byte chunk of a shared-memory row as scalars.
@@ -206,52 +322,57 @@ __device__ __forceinline__ void st_chunk(T* p, const T* in) {
 
 // ---------------------------------------------------------------------------
 // Phase 4: sweep one row segment [i0, i0+SL) (local cells; tile element
-// e = cell + kHalo) in chunks of VN cells with a sliding window of J = xi f
-// over cells [i-4, i+VN+4) of the current chunk start i.  POS: xi > 0.
+// e = cell + kHalo) in chunks of VN cells with a sliding window of f over
+// cells [i-4, i+VN+4) of the current chunk start i, and of the differences of
+// J = xi f (rounded products, as the oracle takes them: the noise that the
+// weights amplify then follows the oracle's more closely).  POS: xi > 0.
 // Positive: face s+1/2 uses J_{s-2..s+2} with centre J_s:
 //   (D0..D3) = Delta_{s-2..s+1}, (K1, K2, K3) = K_{s-1}, K_s, K_{s+1}.
 // Negative: the mirror (J_{s+3}, ..., J_{s-1}) with centre J_{s+1}:
 //   (D0..D3) = -Delta_{s+2}, -Delta_{s+1}, -Delta_s, -Delta_{s-1},
-//   (K1, K2, K3) = K_{s+2}, K_{s+1}, K_s.
-// (Delta_s = J_{s+1} - J_s, K_s = 13/12 (J_{s-1} - 2 J_s + J_{s+1})^2.)
-// The flux difference of cell i is then
-//   POS: F_{i+1/2} - F_{i-1/2} = Delta_{i-1} + (C_{i+1/2} - C_{i-1/2})/6,
-//   NEG: F_{i+1/2} - F_{i-1/2} = Delta_i     + (C_{i+1/2} - C_{i-1/2})/6.
-// With the loop fully unrolled, differences shared between neighbouring
-// faces are computed once (common subexpressions across iterations).
+//   (K1, K2, K3) = K_{s+2}, K_{s+1}, K_s; weno_corr is odd in its differences,
+//   so C is minus the value for the un-negated ones.
+// (Delta_s = J_{s+1} - J_s, K_s = 13/3 (J_{s-1} - 2 J_s + J_{s+1})^2.)
+// The flux difference of cell i is
+//   POS: Delta_{i-1} + (C_{i+1/2} - C_{i-1/2})/6,
+//   NEG: Delta_i     + (C_{i+1/2} - C_{i-1/2})/6,
+// and c1 = dt/dz; gco holds (gamma, gamma beta) dt/tau.
 // ---------------------------------------------------------------------------
-template <typename T, bool POS>
-__device__ __forceinline__ T face_corr(const T* J, int wc) {
-  // J: window values, wc: window index of the face's left cell
-  const T k13 = T(13) / T(12);
-  auto D = [&](int c) { return J[c + 1] - J[c]; };
-  auto K = [&](int c) {
-    const T s2 = (J[c + 1] - J[c]) - (J[c] - J[c - 1]);
-    return k13 * s2 * s2;
-  };
-  if constexpr (POS)
-    return weno_corr<T>(D(wc - 2), D(wc - 1), D(wc), D(wc + 1), K(wc - 1), K(wc), K(wc + 1));
-  else
-    return weno_corr<T>(-D(wc + 2), -D(wc + 1), -D(wc), -D(wc - 1), K(wc + 2), K(wc + 1),
-                        K(wc));
-}
-
 template <typename T, bool POS, int SL>
-__device__ __forceinline__ void sweep_segment(const T* row, T* orow, int i0, T xi,
-                                              const T* __restrict__ wp, int nm, int MP,
-                                              const T* __restrict__ ck,
-                                              const T* __restrict__ gco, T inv_dz, T dt) {
+__device__ __forceinline__ void sweep_segment(const T* row, T* orow, int i0, T xi, T c1,
+                                              const T* wp8, const T* __restrict__ wp,
+                                              int wstride, int MP, const T* __restrict__ ck,
+                                              const T* __restrict__ gco) {
   constexpr int VN = V16<T>::n;
   constexpr int NW = VN + 2 * kHalo;  // window cells [i-4, i+VN+4)
   const T sixth = T(1) / T(6);
+  const T k13 = T(13) / T(3);
   T R[NW];  // f at cells i-4+c
-  T J[NW];  // J = xi f at the same cells
+  T Dw[NW - 1], Kw[NW - 1];
+  auto diffs = [&](int c0) {
+#pragma unroll
+    for (int c = 0; c < NW - 1; ++c)
+      if (c >= c0) Dw[c] = Prec<T>::mul(xi, R[c + 1]) - Prec<T>::mul(xi, R[c]);
+#pragma unroll
+    for (int c = 1; c < NW - 1; ++c)
+      if (c >= c0) {
+        const T s2 = Dw[c] - Dw[c - 1];
+        Kw[c] = (k13 * s2) * s2;
+      }
+  };
+  auto face = [&](int wc) {  // the face right of window cell wc
+    if constexpr (POS)
+      return weno_corr<T>(Dw[wc - 2], Dw[wc - 1], Dw[wc], Dw[wc + 1], Kw[wc - 1], Kw[wc],
+                          Kw[wc + 1]);
+    else
+      return weno_corr<T>(Dw[wc + 2], Dw[wc + 1], Dw[wc], Dw[wc - 1], Kw[wc + 2], Kw[wc + 1],
+                          Kw[wc]);
+  };
 #pragma unroll
   for (int c = 0; c < NW; c += VN) ld_chunk<T>(row + i0 + c, R + c);
-#pragma unroll
-  for (int c = 0; c < NW; ++c) J[c] = xi * R[c];
-  // correction at the left face of cell i0 (window cell of its left cell: 3)
-  T Cl = face_corr<T, POS>(J, kHalo - 1);
+  Kw[0] = T(0);
+  diffs(0);
+  T Cl = face(kHalo - 1);
 #pragma unroll
   for (int t = 0; t < SL / VN; ++t) {
     const int i = i0 + t * VN;
@@ -259,37 +380,73 @@ __device__ __forceinline__ void sweep_segment(const T* row, T* orow, int i0, T x
 #pragma unroll
     for (int c = 0; c < VN; ++c) {
       const int wc = kHalo + c;  // window index of cell i + c
-      const T Cr = face_corr<T, POS>(J, wc);
-      const T dF = (POS ? (J[wc] - J[wc - 1]) : (J[wc + 1] - J[wc])) + (Cr - Cl) * sixth;
+      const T Cr = face(wc);
+      const T dF = POS ? fma(Cr - Cl, sixth, Dw[wc - 1]) : fma(Cl - Cr, sixth, Dw[wc]);
       Cl = Cr;
       const T* cc = ck + (size_t)(i + c) * MP;
+      // f^eq: a real loop over the orders in FP64 (an instruction that is
+      // predicated off still takes its slot on the FP64 pipe) and past the
+      // first eight in FP32.  Coefficients past nm are zero, so any row of the
+      // weight table serves them.
       T feq = T(0);
+      auto orders = [&](int m0) {
+        T cv[VN];
+        ld_chunk<T>(cc + m0, cv);
 #pragma unroll
-      for (int m0 = 0; m0 < kMaxMP; m0 += VN) {
-        if (m0 < nm) {
-          T cv[VN];
-          ld_chunk<T>(cc + m0, cv);
+        for (int q = 0; q < VN; ++q) feq = fma(cv[q], __ldg(wp + min(m0 + q, kMaxM - 1) * wstride), feq);
+      };
+      if constexpr (sizeof(T) == 8) {
+#pragma unroll 1
+        for (int m0 = 0; m0 < MP; m0 += VN) orders(m0);
+      } else {
 #pragma unroll
-          for (int q = 0; q < VN; ++q) feq += cv[q] * wp[m0 + q];
+        for (int m0 = 0; m0 < 8; m0 += VN)
+          if (m0 < MP) {
+            T cv[VN];
+            ld_chunk<T>(cc + m0, cv);
+#pragma unroll
+            for (int q = 0; q < VN; ++q) feq = fma(cv[q], wp8[m0 + q], feq);
+          }
+        if (MP > 8) {
+#pragma unroll 1
+          for (int m0 = 8; m0 < MP; m0 += VN) orders(m0);
         }
       }
       const T f = R[kHalo + c];
-      const T coll = (gco[2 * (i + c)] - gco[2 * (i + c) + 1] * xi) * (f - feq);
-      const T L = -dF * inv_dz - coll;
-      out[c] = f + dt * L;
+      const T rate = fma(-xi, gco[2 * (i + c) + 1], gco[2 * (i + c)]);
+      out[c] = fma(-rate, f - feq, fma(-c1, dF, f));
     }
     if (t + 1 < SL / VN) {
       // slide the window by one chunk: load the chunk at cells i+VN+4 ..
 #pragma unroll
-      for (int c = 0; c < NW - VN; ++c) {
-        J[c] = J[c + VN];
-        R[c] = R[c + VN];
+      for (int c = 0; c < NW - VN; ++c) R[c] = R[c + VN];
+#pragma unroll
+      for (int c = 0; c < NW - 1 - VN; ++c) {
+        Dw[c] = Dw[c + VN];
+        Kw[c] = Kw[c + VN];
       }
       ld_chunk<T>(row + i + NW, R + NW - VN);  // tile element of cell i+VN+4 is i + NW
-#pragma unroll
-      for (int c = 0; c < VN; ++c) J[NW - VN + c] = xi * R[NW - VN + c];
+      diffs(NW - 1 - VN);
     }
     st_chunk<T>(orow + kHalo + i, out);
+  }
+}
+
+// The integrals X3_m, X4_m of one cell by the 32-node rule, for |beta| so close
+// to 1 that the recurrence would need more than its table (u beyond ~7 (FP64)
+// or ~11 (FP32)): the truncated f^eq is strongly negative there, so no flow
+// the method can follow reaches this; kept for the stray cell that does.
+template <typename T>
+__device__ __noinline__ void aeq_far(const double* __restrict__ gl_t,
+                                     const double* __restrict__ gl_w, T u, T sh2, int nm, T* X) {
+  T J3[kMaxM], J4[kMaxM];
+  for (int m = 0; m < kMaxM; ++m) { J3[m] = T(0); J4[m] = T(0); }
+  const T A = asinh(u), uinv = T(1) / u;
+  for (int i = 0; i < kAeqNodes; ++i)
+    aeq_node<T>(T(gl_t[i]), T(gl_w[i]), A, sh2, uinv, false, nm, J3, J4);
+  for (int m = 0; m < nm; ++m) {
+    X[m] = J3[m] * (A * uinv);
+    X[kMaxM + m] = J4[m] * (A * uinv);
   }
 }
 
@@ -297,27 +454,26 @@ template <typename T, int B, int NT>
 __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __restrict__ fn,
                                          T* fout, int stage, int* err, const SodGeom& g,
                                          const SodTables<T>& tb, const int* __restrict__ rowv,
-                                         int nneg, int nseg, int s0) {
+                                         int nneg, int nseg, int np, int s0) {
   constexpr int VN = V16<T>::n;
   constexpr int W = B + 2 * kHalo;
   constexpr int P = tile_pitch<T>(W);
   constexpr int CH = B / VN;  // 16-byte chunks of interior cells
+  constexpr bool kF64 = sizeof(T) == 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int V = g.V;
-  const SodSmem<T> lay(V, B, g.QL, g.nm, nseg > 1);
+  const SodSmem<T> lay(V, B, g.QL, g.nm, nseg > 1, np);
   T* tile = reinterpret_cast<T*>(smem_raw + lay.tile);
   T* outb = (nseg > 1) ? reinterpret_cast<T*>(smem_raw + lay.outb) : nullptr;
   double* msum = reinterpret_cast<double*>(smem_raw + lay.msum);
-  // per-cell results of the Landau phase for the coefficient phase, [8][B]
-  // values of the kernel's type (the FP32 kernel takes its coefficient
-  // arithmetic in FP32)
   T* cellT = reinterpret_cast<T*>(smem_raw + lay.cell);
   T* coef = reinterpret_cast<T*>(smem_raw + lay.coef);
   T* gco = reinterpret_cast<T*>(smem_raw + lay.gco);
+  double* part = np ? reinterpret_cast<double*>(smem_raw + lay.part) : msum;
   const int MP = coef_pitch<T>(g.nm);
 
   const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
+  const int lane = tid & 31;
 
   // ---- 1. stage tile + halo ----
   const bool interior = (s0 - kHalo >= 0) && (s0 + B + kHalo <= g.Z);
@@ -338,192 +494,185 @@ __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __r
 
   const bool collide = g.tau_mode != kTauNone;
   if (collide) {
-    // ---- 2. moments ----
-    if (V <= kSerialMomentRows) {
-      // few velocities: lane 5c + q sums moment q of cell c of the warp's
-      // 16-byte chunk over every row by itself (blocks of four rows, then
-      // compensated), so no cross-lane reduction is needed
-      const int c = lane / 5, q = lane - 5 * (lane / 5);
-      for (int ch = warp; ch < CH; ch += NT / 32) {
-        if (lane >= VN * 5) break;
-        const T* col = tile + kHalo + ch * VN + c;
-        const T* wq = tb.mw + (size_t)q * V;
-        Acc<T> acc;
-        int v = 0;
-        for (; v + 4 <= V; v += 4) {
-          T blk = col[v * P] * wq[v];
-          blk += col[(v + 1) * P] * wq[v + 1];
-          blk += col[(v + 2) * P] * wq[v + 2];
-          blk += col[(v + 3) * P] * wq[v + 3];
-          acc.add(blk);
+    // ---- 2. moments: thread (cell c, row group gr); the group's rows are a
+    // contiguous slice, so it meets at most two or three radial nodes ----
+    {
+      constexpr int G = NT / B;                    // row groups
+      constexpr int WB = B < 32 ? B : 32;          // lanes per group in a warp
+      constexpr int NS = NT / (B < 32 ? 32 : B);   // slots: groups after the in-warp merge
+      const int c = tid % B, gr = tid / B;
+      const bool work = gr < G;  // whole warps (B >= 32: NT - G B is a multiple of 32)
+      if (work) {
+        Moments<T> m;
+        const int v1 = (int)((long long)V * (gr + 1) / G);
+        int v = (int)((long long)V * gr / G);
+        const T* col = tile + kHalo + c;
+        while (v < v1) {
+          const int k = v / g.Qx, ve = min(v1, (k + 1) * g.Qx);
+          for (; v + 4 <= ve; v += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) m.row(col[(v + u) * P], tb.m3 + 4 * (v + u));
+            m.block();
+          }
+          for (; v < ve; ++v) m.row(col[v * P], tb.m3 + 4 * v);
+          m.flush(tb.pk + 2 * k);
         }
-        T blk = T(0);
-        for (; v < V; ++v) blk += col[v * P] * wq[v];
-        acc.add(blk);
-        msum[q * B + ch * VN + c] = acc.value();
-      }
-    } else {
-      // warp = 16-byte chunk of cells (warps loop over the chunks), lanes = rows
-      for (int ch = warp; ch < CH; ch += NT / 32) {
-      Acc<T> acc[VN][5];
-      for (int v0 = lane; v0 < V; v0 += 128) {
-        T blk[VN][5];
 #pragma unroll
-        for (int c = 0; c < VN; ++c)
-#pragma unroll
-          for (int q = 0; q < 5; ++q) blk[c][q] = T(0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int v = v0 + 32 * u;
-          if (v < V) {
-            T x[VN];
-            ld_chunk<T>(tile + v * P + kHalo + ch * VN, x);
-            T w[5];
-#pragma unroll
-            for (int q = 0; q < 5; ++q) w[q] = tb.mw[q * V + v];
-#pragma unroll
-            for (int c = 0; c < VN; ++c)
-#pragma unroll
-              for (int q = 0; q < 5; ++q) blk[c][q] += x[c] * w[q];
+        for (int off = WB; off < 32; off *= 2) m.merge_xor(off, 0xffffffffu);
+        // slot sl of cell c; slots beyond np are added in later rounds
+        const int sl = B < 32 ? tid / 32 : gr;
+        const bool owner = B >= 32 || lane < B;
+        if (np >= NS) {
+          if (owner) m.put(part + (size_t)sl * 5 * B + c, B, false);
+        } else {
+          const int n = np ? np : 1;
+          for (int r = 0; r * n < NS; ++r) {
+            if (owner && sl / n == r) m.put(part + (size_t)(sl % n) * 5 * B + c, B, r > 0);
+            asm volatile("bar.sync 1, %0;" ::"n"(NS * (B < 32 ? 32 : B)) : "memory");
           }
         }
-#pragma unroll
-        for (int c = 0; c < VN; ++c)
-#pragma unroll
-          for (int q = 0; q < 5; ++q) acc[c][q].add(blk[c][q]);
       }
-      if constexpr (sizeof(T) == 4) {
-        // FP32 transposing reduction of the compensated pairs (sum, -c):
-        // lane l ends with value l; only hi + lo is formed in FP64
-        static_assert(VN * 5 <= 32, "moment values per warp");
-        float h[32], lo[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          h[i] = 0.f;
-          lo[i] = 0.f;
-        }
-#pragma unroll
-        for (int c = 0; c < VN; ++c)
-#pragma unroll
-          for (int q = 0; q < 5; ++q) {
-            h[c * 5 + q] = acc[c][q].s;
-            lo[c * 5 + q] = -acc[c][q].c;
-          }
-        tr_level<16>(h, lo, lane);
-        tr_level<8>(h, lo, lane);
-        tr_level<4>(h, lo, lane);
-        tr_level<2>(h, lo, lane);
-        tr_level<1>(h, lo, lane);
-        if (lane < VN * 5) {
-          const int c = lane / 5, q = lane - 5 * (lane / 5);
-          msum[q * B + ch * VN + c] = (double)h[0] + (double)lo[0];
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < VN; ++c)
-#pragma unroll
-          for (int q = 0; q < 5; ++q) {
-            const double s = warp_sum(acc[c][q].value());
-            if (lane == 0) msum[q * B + ch * VN + c] = s;
-          }
-      }
+      __syncthreads();
+      const int n = np >= NS ? NS : (np ? np : 1);
+      for (int e = tid; e < 5 * B; e += NT) {
+        // np = 0 shares msum: each element is read and written by one thread
+        const double t = Moments<T>::total(part + e, 5 * B, n);
+        msum[e] = t;
       }
     }
     __syncthreads();
 
-    // ---- 3a. Landau matching and relaxation time, one thread per cell ----
-    if (tid < B) {
-      const int c = tid;
+    // ---- 3. Landau matching (FP64), relaxation time and f^eq coefficients.
+    // FP32: one thread per cell does all.  FP64: two lanes per cell of warp 0
+    // run the two recurrences side by side (an FP64 instruction costs a
+    // sub-partition ~64 cycles however many lanes are active), and the
+    // coefficients follow by (cell, m) over the CTA ----
+    constexpr bool kCanSplit = kF64 && 2 * B <= 32;
+    const bool split = kCanSplit && g.QL >= 2;
+    const int nt3 = split ? 2 * B : B;
+    if (tid < nt3) {
+      const int c = tid % B;
+      const bool second = tid >= B;  // the E chain's lane when split
+      const int wl = min(32, nt3 - (tid & ~31));
+      const unsigned mask = wl == 32 ? 0xffffffffu : ((1u << wl) - 1u);
       LandauOut Lo = landau_factored(msum[c], msum[B + c], msum[2 * B + c], msum[3 * B + c],
                                      msum[4 * B + c]);
       T g0 = T(0), g1 = T(0);
       if (!Lo.ok) {
-        if (s0 + c < g.Z) report_error(err, 6, s0 + c);
-        Lo.n = 1.0; Lo.T = 1.0; Lo.beta = 0.0; Lo.gamma = 1.0; Lo.u = 0.0;
+        if (!second && s0 + c < g.Z) report_error(err, 6, s0 + c);
+        Lo.n = 0.0; Lo.T = 1.0; Lo.beta = 0.0; Lo.gamma = 1.0; Lo.u = 0.0;
       } else if (g.tau_mode == kTauEtas) {
-        const double tau = g.tau_AW0 / Lo.T *
-                           (1.0 - 0.25 * log(Lo.n / (Lo.T * Lo.T * Lo.T) * g.lambda_ref));
-        g0 = T(Lo.gamma / tau);
-        g1 = T(Lo.gamma * Lo.beta / tau);
-      } else if constexpr (sizeof(T) == 4) {
-        const float itau = 1.f / float(g.tau);
-        g0 = float(Lo.gamma) * itau;
-        g1 = float(Lo.gamma * Lo.beta) * itau;
+        const double lam = Lo.n * g.lambda_ref * rcp64(Lo.T * Lo.T * Lo.T);
+        const double r = g.dt * Lo.T * rcp64(g.tau_AW0 * fma(-0.25, log(lam), 1.0));
+        g0 = T(Lo.gamma * r);
+        g1 = T(Lo.ub * r);
       } else {
-        g0 = Lo.gamma / g.tau;
-        g1 = Lo.gamma * Lo.beta / g.tau;
+        const T r = T(g.dt_tau);
+        g0 = T(Lo.gamma) * r;
+        g1 = T(Lo.ub) * r;
       }
-      if constexpr (sizeof(T) == 4) {
-        // FP32 from here on: the coefficients are computed in FP32
-        const float u = float(Lo.u);
-        const float A = asinhf(u);
-        cellT[0 * B + c] = float(Lo.n);
-        cellT[1 * B + c] = float(Lo.T);
-        cellT[2 * B + c] = u;
-        cellT[3 * B + c] = A;
-        cellT[4 * B + c] = (u > 0.f) ? A / u : 1.f;
-        cellT[5 * B + c] = u * u / (float(Lo.gamma) + 1.f);  // 2 sinh^2(A/2) = gamma - 1
+      if (!second) {
+        gco[2 * c] = g0;
+        gco[2 * c + 1] = g1;
+      }
+      const int nm = g.nm, nm4 = max(nm, 4);
+      float r;
+      const int M = aeq_start<T>(float(Lo.u), float(Lo.gamma), nm4, &r);
+      const bool far = M > aeq_max_start<T>();
+      const int Mw = __reduce_max_sync(mask, min(M, aeq_max_start<T>()));
+      const T beta = T(Lo.beta), gam = T(Lo.gamma), b2 = far ? T(0) : beta * beta;
+      const T n4 = T(0.25 * Lo.n);
+      // c_{k,m} = (m + 1/2) beta^m [p3 + L1_k (p3 - p4)], p3 = A3 S_m delta_m,
+      // p4 = A4 S_m eps_m (A4 with the factor T), from the norms of the chains
+      if (split) {
+        T* dst = coef + ((size_t)(second ? B : 0) + c) * MP;  // slot k = 0: delta, 1: eps
+        T d2 = T(0), d1 = T(0);
+        aeq_chain<T>(second, b2, T(r), Mw, nm4, [&](int m, T x) {
+          if (m < nm && m >= 2) dst[m] = x;
+          if (m == 2) d2 = x;
+          if (m == 1) d1 = x;
+        });
+        if (!second) {
+          dst[0] = d1;
+          if (nm > 1) dst[1] = d1;
+          cellT[c] = n4 * (gam + gam) * T(rcp64(double(d1)));
+        } else {
+          dst[0] = fma(T(0.25), b2, T(0.75)) * d2;
+          if (nm > 1) dst[1] = d2;
+          cellT[B + c] = n4 * T(Lo.T) * (T(8.0 / 3.0) * gam * gam) * T(rcp64(double(d2)));
+          cellT[2 * B + c] = beta;
+        }
+        if (far) {
+          T X[2 * kMaxM];
+          aeq_far<T>(tb.gl_t, tb.gl_w, T(Lo.u), T(Lo.u * Lo.u / (Lo.gamma + 1.0)), nm, X);
+          // as delta_m, eps_m that give X3_m, X4_m with A = n/4 (T), sign^m in beta
+          for (int m = 0; m < nm; ++m)
+            dst[m] = X[second ? kMaxM + m : m] / aeq_scale<T>(second, m);
+          cellT[second ? B + c : c] = second ? n4 * T(Lo.T) : n4;
+          if (second) cellT[2 * B + c] = Lo.beta < 0.0 ? T(-1) : T(1);
+        }
       } else {
-        const double A = asinh(Lo.u);
-        const double sh = sinh(0.5 * A);
-        cellT[0 * B + c] = Lo.n;
-        cellT[1 * B + c] = Lo.T;
-        cellT[2 * B + c] = Lo.u;
-        cellT[3 * B + c] = A;
-        cellT[4 * B + c] = (Lo.u > 0.0) ? A / Lo.u : 1.0;
-        cellT[5 * B + c] = 2.0 * sh * sh;
-      }
-      cellT[6 * B + c] = (Lo.beta < 0.0) ? T(-1) : T(1);
-      cellT[7 * B + c] = Lo.ok ? T(1) : T(0);
-      gco[2 * c] = g0;
-      gco[2 * c + 1] = g1;
-    }
-    __syncthreads();
-
-    // ---- 3b. f^eq coefficients: G threads per cell share the nodes ----
-    {
-      constexpr int G = (256 / B) < 32 ? (256 / B) : 32;
-      const int c = tid / G, q = tid - c * G;
-      if (c < B) {
-        const T ud = cellT[2 * B + c];
-        const T A = cellT[3 * B + c], sh2 = cellT[5 * B + c];
-        const T uinv = (ud > T(0)) ? T(1) / ud : T(0);
-        const bool at_rest = !(ud > T(0));
-        T J3[kMaxM], J4[kMaxM];
+        T D[kMaxM], E[kMaxM];
 #pragma unroll
-        for (int m = 0; m < kMaxM; ++m) { J3[m] = T(0); J4[m] = T(0); }
-        // FP32 with N_Omega <= 7: the 16-node rule (stored after the 32-node one)
-        const bool short_rule = sizeof(T) == 4 && g.nm <= 8;
-        const int nn = short_rule ? kAeqNodesF32 : kAeqNodes, n0 = short_rule ? kAeqNodes : 0;
-        for (int i = q; i < nn; i += G)
-          aeq_node<T>(T(tb.gl_t[n0 + i]), T(tb.gl_w[n0 + i]), A, sh2, uinv, at_rest, g.nm, J3, J4);
+        for (int m = 0; m < kMaxM; ++m) { D[m] = T(0); E[m] = T(0); }
+        aeq_chain<T>(false, b2, T(r), Mw, nm4, [&](int m, T x) { D[m] = x; });
+        aeq_chain<T>(true, b2, T(r), Mw, nm4, [&](int m, T x) { E[m] = x; });
+        // relative to the norms X3_0 = 2 u0 and X4_0 = (2/3) u0^2 (3 + beta^2),
+        // which are taken in FP64: the isotropic part of f^eq has one rounding
+        const T rD = T(1) / D[1], rE = T(1) / (fma(T(0.25), b2, T(0.75)) * E[2]);
+        T A3 = T(0.5 * Lo.n * Lo.gamma);
+        T A4 = T(Lo.n * Lo.T * Lo.gamma * Lo.gamma * fma(Lo.beta, Lo.beta * (1.0 / 6.0), 0.5));
+        T q = beta;
+        D[0] = D[1] = T(1);
+        E[1] = E[2] * rE;
+        E[0] = T(1);
 #pragma unroll
-        for (int off = G / 2; off >= 1; off >>= 1)
+        for (int m = 2; m < kMaxM; ++m) {
+          D[m] *= rD;
+          E[m] *= rE;
+        }
+        if (far) {
+          T X[2 * kMaxM];
+          aeq_far<T>(tb.gl_t, tb.gl_w, T(Lo.u), T(Lo.u * Lo.u / (Lo.gamma + 1.0)), nm, X);
 #pragma unroll
           for (int m = 0; m < kMaxM; ++m)
-            if (m < g.nm) {
-              J3[m] += __shfl_xor_sync(0xffffffffu, J3[m], off, G);
-              J4[m] += __shfl_xor_sync(0xffffffffu, J4[m], off, G);
+            if (m < nm) {
+              D[m] = X[m] / aeq_scale<T>(false, m);
+              E[m] = X[kMaxM + m] / aeq_scale<T>(true, m);
             }
-        if (q == 0) {
-          // c''_{k,m} = sgn^m (2m+1)/2 (n r/4) [J3_m + (3 - x_k)(J3_m - theta J4_m)]
-          const T fac = cellT[7 * B + c] * cellT[0 * B + c] * cellT[4 * B + c] * T(0.25);
-          const T theta = cellT[1 * B + c];
-          const T sgn = cellT[6 * B + c];
-          T sm = fac;
-#pragma unroll
-          for (int m = 0; m < kMaxM; ++m) {
-            if (m < g.nm) {
-              const T h = sm * T(0.5 * (2 * m + 1));
-              const T d = J3[m] - theta * J4[m];
-              for (int k = 0; k < g.QL; ++k)
-                coef[((size_t)k * B + c) * MP + m] = h * (J3[m] + tb.L1k[k] * d);
-              sm *= sgn;
-            }
-          }
-          for (int m = g.nm; m < MP; ++m)
-            for (int k = 0; k < g.QL; ++k) coef[((size_t)k * B + c) * MP + m] = T(0);
+          A3 = T(0.25 * Lo.n);
+          A4 = T(0.25 * Lo.n * Lo.T);
+          q = Lo.beta < 0.0 ? T(-1) : T(1);
         }
+        T bm = T(1);
+#pragma unroll
+        for (int m = 0; m < kMaxM; ++m) {
+          if (m < nm) {
+            const T um = T(m + 0.5) * bm;
+            const T p3 = um * (A3 * (aeq_scale<T>(false, m) * D[m]));
+            const T pd = p3 - um * (A4 * (aeq_scale<T>(true, m) * E[m]));
+            for (int k = 0; k < g.QL; ++k)
+              coef[((size_t)k * B + c) * MP + m] = fma(tb.L1k[k], pd, p3);
+            bm *= q;
+          }
+        }
+        for (int m = nm; m < MP; ++m)
+          for (int k = 0; k < g.QL; ++k) coef[((size_t)k * B + c) * MP + m] = T(0);
+      }
+    }
+    if (split) {
+      __syncthreads();
+      for (int e = tid; e < B * MP; e += NT) {
+        const int c = e / MP, m = e - c * MP;
+        T p3 = T(0), pd = T(0);
+        if (m < g.nm) {
+          const T q = cellT[2 * B + c];
+          T um = T(m + 0.5);
+          for (int i = 0; i < m; ++i) um *= q;
+          p3 = um * (cellT[c] * (aeq_scale<T>(false, m) * coef[(size_t)c * MP + m]));
+          pd = p3 - um * (cellT[B + c] * (aeq_scale<T>(true, m) * coef[((size_t)B + c) * MP + m]));
+        }
+        for (int k = 0; k < g.QL; ++k) coef[((size_t)k * B + c) * MP + m] = fma(tb.L1k[k], pd, p3);
       }
     }
     __syncthreads();
@@ -534,36 +683,46 @@ __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __r
   }
 
   // ---- 4. WENO5 + relaxation + RK update, row sweeps ----
-  const T inv_dz = T(g.inv_dz), dt = T(g.dt);
+  const T c1 = T(g.inv_dz * g.dt);
   const int SLr = B / nseg;
-  for (int u = tid; u < V * nseg; u += NT) {
-    const int ir = u % V, seg = u / V;
+  // unsegmented rows: the negative ones padded to whole warps, so that no warp
+  // runs both directions
+  const int pad = nseg == 1 ? (32 - nneg % 32) % 32 : 0;
+  for (int u = tid; u < V * nseg + pad; u += NT) {
+    if (u >= nneg && u < nneg + pad) continue;
+    const int up = u >= nneg ? u - pad : u;
+    const int ir = up % V, seg = up / V;
     const int v = rowv[ir];
     const bool pos = ir >= nneg;
     const T xi = tb.xi[v];
     const int k = tb.kidx[v];
-    T wp[kMaxMP];
+    const T* wp = tb.wp + v;
+    T wp8[8];
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int m = 0; m < kMaxMP; ++m) wp[m] = (m < g.nm) ? tb.wp[m * V + v] : T(0);
+      for (int m = 0; m < 8; ++m) wp8[m] = (m < g.nm) ? wp[m * V] : T(0);
+    }
     const T* row = tile + v * P;
     T* orow = (nseg > 1) ? (outb + v * B - kHalo) : (tile + v * P);
     const T* ck = coef + (size_t)k * B * MP;
     const int i0 = seg * SLr;
     // the segment length is one of B, B/2, B/4, B/8 (>= one 16-byte chunk)
     if (SLr == B) {
-      if (pos) sweep_segment<T, true, B>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
-      else sweep_segment<T, false, B>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
-    } else if (SLr == B / 2) {
-      if (pos) sweep_segment<T, true, B / 2>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
-      else sweep_segment<T, false, B / 2>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
-    } else if constexpr (B / 4 >= VN) {
+      if (pos) sweep_segment<T, true, B>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
+      else sweep_segment<T, false, B>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
+    } else if constexpr (B / 2 >= VN) {
+     if (SLr == B / 2) {
+      if (pos) sweep_segment<T, true, B / 2>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
+      else sweep_segment<T, false, B / 2>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
+     } else if constexpr (B / 4 >= VN) {
       if (SLr == B / 4) {
-        if (pos) sweep_segment<T, true, B / 4>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
-        else sweep_segment<T, false, B / 4>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
+        if (pos) sweep_segment<T, true, B / 4>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
+        else sweep_segment<T, false, B / 4>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
       } else if constexpr (B / 8 >= VN) {
-        if (pos) sweep_segment<T, true, B / 8>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
-        else sweep_segment<T, false, B / 8>(row, orow, i0, xi, wp, g.nm, MP, ck, gco, inv_dz, dt);
+        if (pos) sweep_segment<T, true, B / 8>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
+        else sweep_segment<T, false, B / 8>(row, orow, i0, xi, c1, wp8, wp, V, MP, ck, gco);
       }
+     }
     }
   }
   __syncthreads();
@@ -605,14 +764,15 @@ template <typename T, int B, int NT>
 __global__ void __launch_bounds__(NT, 2)
 sod_stage_kernel(const T* __restrict__ fin, const T* __restrict__ fn, T* fout, int stage,
                  int* err, SodGeom g, SodTables<T> tb, const int* __restrict__ rowv, int nneg,
-                 int nseg) {
-  sod_tile<T, B, NT>(fin, fn, fout, stage, err, g, tb, rowv, nneg, nseg, blockIdx.x * B);
+                 int nseg, int np) {
+  sod_tile<T, B, NT>(fin, fn, fout, stage, err, g, tb, rowv, nneg, nseg, np, blockIdx.x * B);
 }
 
 template <typename T, int B, int NT>
 __global__ void __launch_bounds__(NT, 2)
 sod_batch_kernel(const SodRunDesc<T>* __restrict__ runs, const SodTask* __restrict__ tasks,
-                 int ntasks, const long long* __restrict__ step, int stage, int* err, int nseg) {
+                 int ntasks, const long long* __restrict__ step, int stage, int* err, int nseg,
+                 int np) {
   const long long n = *step;
   for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
     const SodTask tk = tasks[t];
@@ -620,20 +780,40 @@ sod_batch_kernel(const SodRunDesc<T>* __restrict__ runs, const SodTask* __restri
     if (n >= R.nsteps) break;  // tasks are ordered by decreasing step count
     const T* fin = stage == 0 ? R.F0 : (stage == 1 ? R.F1 : R.F2);
     T* fout = stage == 0 ? R.F1 : (stage == 1 ? R.F2 : R.F0);
-    sod_tile<T, B, NT>(fin, R.F0, fout, stage, err, R.g, R.tb, R.rowv, R.nneg, nseg, tk.s0);
+    sod_tile<T, B, NT>(fin, R.F0, fout, stage, err, R.g, R.tb, R.rowv, R.nneg, nseg, np, tk.s0);
     __syncthreads();
   }
 }
 
-template <typename T, int B, int NT>
-static size_t smem_for(int V, int QL, int nm, int nseg) {
-  return SodSmem<T>(V, B, QL, nm, nseg > 1).total;
+constexpr int kNT = 320;           // threads of the scalar kernels
+constexpr int kMaxSmem = 232448;   // opt-in shared memory per CTA
+
+static int pick_nseg(int V, int B, int VN) {
+  int nseg = 1;
+  while (nseg < 8 && B / (2 * nseg) >= VN && V * 2 * nseg <= kNT) nseg *= 2;
+  return nseg;
 }
 
-static int pick_nseg(int V, int B, int NT, int VN) {
-  int nseg = 1;
-  while (nseg < 8 && B / (2 * nseg) >= VN && V * 2 * nseg <= NT) nseg *= 2;
-  return nseg;
+// Shared memory of a tile without the partial slots of the moment sums; what
+// the kernels accept is decided by this size.
+template <typename T>
+static size_t smem_base(int V, int B, int QL, int nm) {
+  return SodSmem<T>(V, B, QL, nm, pick_nseg(V, B, V16<T>::n) > 1, 0).total;
+}
+
+// Partial slots: one per row group of the CTA where they fit beside the tile
+// without costing the second CTA of an SM, fewer (added in rounds) otherwise.
+template <typename T>
+static int pick_np(int V, int B, int QL, int nm) {
+  const size_t base = smem_base<T>(V, B, QL, nm), half = kMaxSmem / 2 - 2048;
+  const size_t room = (base <= half ? half : (size_t)kMaxSmem) - std::min<size_t>(base, kMaxSmem);
+  const size_t full = kNT / (B < 32 ? 32 : B);
+  return (int)std::min(full, room / (sizeof(double) * 5 * B));
+}
+
+template <typename T>
+static size_t smem_for(int V, int B, int QL, int nm) {
+  return SodSmem<T>(V, B, QL, nm, pick_nseg(V, B, V16<T>::n) > 1, pick_np<T>(V, B, QL, nm)).total;
 }
 
 // Opt every stage kernel into the large dynamic shared-memory carve-out
@@ -645,6 +825,8 @@ cudaError_t sod_set_attributes() {
                        (const void*)sod_stage_kernel<float, 16, 320>,
                        (const void*)sod_stage_kernel<double, 16, 320>,
                        (const void*)sod_stage_kernel<double, 8, 320>,
+                       (const void*)sod_stage_kernel<double, 4, 320>,
+                       (const void*)sod_stage_kernel<double, 2, 320>,
                        (const void*)sod_batch_kernel<float, 128, 320>,
                        (const void*)sod_batch_kernel<float, 64, 320>,
                        (const void*)sod_batch_kernel<float, 32, 320>,
@@ -660,7 +842,7 @@ cudaError_t sod_set_attributes() {
   return sod32p_set_attributes();
 }
 
-SodLaunch sod_pick_launch(bool fp64, int V, int QL, int nm, int max_smem) {
+SodLaunch sod_pick_launch(bool fp64, int V, int QL, int nm, int max_smem, int Z, int nsm) {
   SodLaunch L{0, 0};
   if (QL > kMaxQL || V < 1 || nm < 1 || nm > kMaxM) return L;
   const size_t half = (size_t)max_smem / 2 - 2048;
@@ -671,19 +853,31 @@ SodLaunch sod_pick_launch(bool fp64, int V, int QL, int nm, int max_smem) {
     // few velocities: wide tiles share each tile's fixed costs among more
     // cells and give the row segments more cells (65536 cells, V = 24: 0.15 ms
     // per step with 128-cell tiles, 0.18 with 64, 0.26 with 32)
-    if (V < 48 && smem_for<float, 128, 320>(V, QL, nm, pick_nseg(V, 128, 320, 4)) <= half)
-      return {128, 0};
-    if (V < 128 && smem_for<float, 64, 320>(V, QL, nm, pick_nseg(V, 64, 320, 4)) <= half)
-      return {64, 0};
-    const int n32 = pick_nseg(V, 32, 320, 4), n16 = pick_nseg(V, 16, 320, 4);
-    if (smem_for<float, 32, 320>(V, QL, nm, n32) <= half) return {32, 0};
-    if (smem_for<float, 16, 320>(V, QL, nm, n16) <= half) return {16, 0};
-    if (smem_for<float, 16, 320>(V, QL, nm, n16) <= (size_t)max_smem) return {16, 0};
+    if (V < 48 && smem_base<float>(V, 128, QL, nm) <= half) return {128, 0};
+    if (V < 128 && smem_base<float>(V, 64, QL, nm) <= half) return {64, 0};
+    if (smem_base<float>(V, 32, QL, nm) <= half) return {32, 0};
+    if (smem_base<float>(V, 16, QL, nm) <= half) return {16, 0};
+    if (smem_base<float>(V, 16, QL, nm) <= (size_t)max_smem) return {16, 0};
   } else {
-    const int n16 = pick_nseg(V, 16, 320, 2), n8 = pick_nseg(V, 8, 320, 2);
-    if (smem_for<double, 16, 320>(V, QL, nm, n16) <= half) return {16, 0};
-    if (smem_for<double, 8, 320>(V, QL, nm, n8) <= half) return {8, 0};
-    if (smem_for<double, 8, 320>(V, QL, nm, n8) <= (size_t)max_smem) return {8, 0};
+    if (smem_base<double>(V, 16, QL, nm) <= half) L.B = 16;
+    else if (smem_base<double>(V, 8, QL, nm) <= (size_t)max_smem) L.B = 8;
+    // The FP64 pipe of an SM (~2 lane operations per cycle) sets the time of a
+    // tile: about 49 operations per cell and velocity and 42 per row for the
+    // halo, so a tube with few tiles runs faster on narrower ones until every
+    // SM has one.  17000 lane operations stand for the phases that wait on
+    // latency (two CTAs per SM overlap them).
+    if (L.B && nsm > 0) {
+      double best = 0.0;
+      for (int B = L.B, first = 1; B >= 2; B /= 2, first = 0) {
+        const long long tiles = (Z + B - 1) / B;
+        const double t = (double)((tiles + nsm - 1) / nsm) * V * (49.0 * B + 42.0) +
+                         17000.0 * (double)((tiles + 2 * nsm - 1) / (2 * nsm));
+        if (first || t < best) {
+          best = t;
+          L.B = B;
+        }
+      }
+    }
   }
   return L;
 }
@@ -692,19 +886,12 @@ template <typename T, int B>
 static cudaError_t launch_b(const SodGeom& g, const SodTables<T>& tb, const int* rowv, int nneg,
                             const T* fin, const T* fn, T* fout, int stage, int* err,
                             cudaStream_t st) {
-  constexpr int NT = 320;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(sod_stage_kernel<T, B, NT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  const int nseg = pick_nseg(g.V, B, NT, V16<T>::n);
-  const size_t smem = smem_for<T, B, NT>(g.V, g.QL, g.nm, nseg);
+  const int nseg = pick_nseg(g.V, B, V16<T>::n);
+  const int np = pick_np<T>(g.V, B, g.QL, g.nm);
+  const size_t smem = smem_for<T>(g.V, B, g.QL, g.nm);
   const int grid = (g.Z + B - 1) / B;
-  sod_stage_kernel<T, B, NT><<<grid, NT, smem, st>>>(fin, fn, fout, stage, err, g, tb, rowv,
-                                                     nneg, nseg);
+  sod_stage_kernel<T, B, kNT><<<grid, kNT, smem, st>>>(fin, fn, fout, stage, err, g, tb, rowv,
+                                                       nneg, nseg, np);
   return cudaGetLastError();
 }
 
@@ -731,6 +918,12 @@ cudaError_t sod_stage_launch(const SodLaunch& L, const SodGeom& g, const SodTabl
     case 8:
       if constexpr (sizeof(T) == 8) return launch_b<T, 8>(g, tb, rowv, nneg, fin, fn, fout, stage, err, st);
       break;
+    case 4:
+      if constexpr (sizeof(T) == 8) return launch_b<T, 4>(g, tb, rowv, nneg, fin, fn, fout, stage, err, st);
+      break;
+    case 2:
+      if constexpr (sizeof(T) == 8) return launch_b<T, 2>(g, tb, rowv, nneg, fin, fn, fout, stage, err, st);
+      break;
     default: break;
   }
   return cudaErrorInvalidValue;
@@ -748,13 +941,9 @@ template cudaError_t sod_stage_launch<double>(const SodLaunch&, const SodGeom&,
 size_t sod_stage_smem_bytes(bool fp64, int B, int V, int QL, int nm) {
   if (!fp64) {
     if (B == kSod32Cells) return sod32_smem_bytes(V, QL);
-    if (B == 128) return smem_for<float, 128, 320>(V, QL, nm, pick_nseg(V, 128, 320, 4));
-    if (B == 64) return smem_for<float, 64, 320>(V, QL, nm, pick_nseg(V, 64, 320, 4));
-    if (B == 32) return smem_for<float, 32, 320>(V, QL, nm, pick_nseg(V, 32, 320, 4));
-    if (B == 16) return smem_for<float, 16, 320>(V, QL, nm, pick_nseg(V, 16, 320, 4));
+    if (B == 128 || B == 64 || B == 32 || B == 16) return smem_for<float>(V, B, QL, nm);
   } else {
-    if (B == 16) return smem_for<double, 16, 320>(V, QL, nm, pick_nseg(V, 16, 320, 2));
-    if (B == 8) return smem_for<double, 8, 320>(V, QL, nm, pick_nseg(V, 8, 320, 2));
+    if (B == 16 || B == 8) return smem_for<double>(V, B, QL, nm);
   }
   return 0;
 }
@@ -764,45 +953,37 @@ cudaError_t sod32_batch_launch(size_t smem, int grid, const SodRunDesc<float>* r
                                int* err, const void* maps, cudaStream_t st);
 
 // Batched stages: all runs of a class share V (so nseg and the tile width).
+template <typename T, int B>
+static cudaError_t batch_b(size_t smem, int grid, const SodRunDesc<T>* runs, const SodTask* tasks,
+                           int ntasks, const long long* step, int stage, int* err, int V, int QL,
+                           int nm, cudaStream_t st) {
+  sod_batch_kernel<T, B, kNT><<<grid, kNT, smem, st>>>(runs, tasks, ntasks, step, stage, err,
+                                                       pick_nseg(V, B, V16<T>::n),
+                                                       pick_np<T>(V, B, QL, nm));
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t sod_batch_stage_launch(int B, size_t smem, int grid, const SodRunDesc<T>* runs,
                                    const SodTask* tasks, int ntasks, const long long* step,
-                                   int stage, int* err, int V, cudaStream_t st,
+                                   int stage, int* err, int V, int QL, int nm, cudaStream_t st,
                                    const void* maps) {
   if (ntasks == 0) return cudaSuccess;
   if constexpr (sizeof(T) == 4) {
-    if (B == kSod32Cells)
-      return sod32_batch_launch(smem, grid, runs, tasks, ntasks, step, stage, err, maps, st);
-    if (B == 128) {
-      sod_batch_kernel<T, 128, 320><<<grid, 320, smem, st>>>(runs, tasks, ntasks, step, stage, err,
-                                                            pick_nseg(V, 128, 320, 4));
-      return cudaGetLastError();
-    }
-    if (B == 64) {
-      sod_batch_kernel<T, 64, 320><<<grid, 320, smem, st>>>(runs, tasks, ntasks, step, stage, err,
-                                                           pick_nseg(V, 64, 320, 4));
-      return cudaGetLastError();
-    }
-    if (B == 32) {
-      sod_batch_kernel<T, 32, 320><<<grid, 320, smem, st>>>(runs, tasks, ntasks, step, stage, err,
-                                                           pick_nseg(V, 32, 320, 4));
-      return cudaGetLastError();
-    }
-    if (B == 16) {
-      sod_batch_kernel<T, 16, 320><<<grid, 320, smem, st>>>(runs, tasks, ntasks, step, stage, err,
-                                                           pick_nseg(V, 16, 320, 4));
-      return cudaGetLastError();
+    switch (B) {
+      case kSod32Cells:
+        return sod32_batch_launch(smem, grid, runs, tasks, ntasks, step, stage, err, maps, st);
+      case 128: return batch_b<T, 128>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+      case 64: return batch_b<T, 64>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+      case 32: return batch_b<T, 32>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+      case 16: return batch_b<T, 16>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+      default: break;
     }
   } else {
-    if (B == 16) {
-      sod_batch_kernel<T, 16, 320><<<grid, 320, smem, st>>>(runs, tasks, ntasks, step, stage, err,
-                                                           pick_nseg(V, 16, 320, 2));
-      return cudaGetLastError();
-    }
-    if (B == 8) {
-      sod_batch_kernel<T, 8, 320><<<grid, 320, smem, st>>>(runs, tasks, ntasks, step, stage, err,
-                                                          pick_nseg(V, 8, 320, 2));
-      return cudaGetLastError();
+    switch (B) {
+      case 16: return batch_b<T, 16>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+      case 8: return batch_b<T, 8>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+      default: break;
     }
   }
   return cudaErrorInvalidValue;
@@ -810,10 +991,10 @@ cudaError_t sod_batch_stage_launch(int B, size_t smem, int grid, const SodRunDes
 
 template cudaError_t sod_batch_stage_launch<float>(int, size_t, int, const SodRunDesc<float>*,
                                                    const SodTask*, int, const long long*, int,
-                                                   int*, int, cudaStream_t, const void*);
+                                                   int*, int, int, int, cudaStream_t, const void*);
 template cudaError_t sod_batch_stage_launch<double>(int, size_t, int, const SodRunDesc<double>*,
                                                     const SodTask*, int, const long long*, int,
-                                                    int*, int, cudaStream_t, const void*);
+                                                    int*, int, int, int, cudaStream_t, const void*);
 
 // ---------------------------------------------------------------------------
 // Initialisation: per-cell FP64 coefficients, then populations.

@@ -19,12 +19,15 @@ struct SodGeom {
   int nm;    // N_Omega + 1
   int bc, tau_mode;
   double inv_dz, dt, tau, tau_AW0, lambda_ref;
+  double dt_tau;  // dt / tau (kTauConst)
 };
 
 // Per-velocity tables in the working precision (device pointers).
 template <typename T>
 struct SodTables {
   const T* mw;      // [5][V]: 1+xi, 1-xi, p(1+xi)^2, p(1-xi)^2, p(1-xi^2)
+  const T* m3;      // [V][4]: (1+xi)^2, (1-xi)^2, 1-xi^2, 0
+  const T* pk;      // [QL][2]: p_k as hi + lo in T
   const T* xi;      // [V]
   const T* wp;      // [kMaxM][V]: w_j w_k P_m(xi_j)
   const int* kidx;  // [V]
@@ -94,7 +97,9 @@ bool sod32_make_maps(void* out4, const float* F0, const float* F1, const float* 
 cudaError_t sod32_set_attributes();
 
 // Pick the tile width for V velocities; returns B = 0 if V does not fit.
-SodLaunch sod_pick_launch(bool fp64, int V, int QL, int nm, int max_smem);
+// With Z cells on nsm SMs the FP64 width also follows the cell count (nsm = 0:
+// the widest that fits).
+SodLaunch sod_pick_launch(bool fp64, int V, int QL, int nm, int max_smem, int Z, int nsm);
 
 // Enqueue one RK stage (stage = 0, 1, 2): fout = stage update of fin (and fn).
 // rowv: velocity rows ordered with negative xi first (nneg of them), so that
@@ -126,7 +131,7 @@ cudaError_t sod32p_stage_launch(const SodGeom& g, const SodTables<float>& tb, co
 template <typename T>
 cudaError_t sod_batch_stage_launch(int B, size_t smem, int grid, const SodRunDesc<T>* runs,
                                    const SodTask* tasks, int ntasks, const long long* step,
-                                   int stage, int* err, int V, cudaStream_t st,
+                                   int stage, int* err, int V, int QL, int nm, cudaStream_t st,
                                    const void* maps = nullptr);
 size_t sod_stage_smem_bytes(bool fp64, int B, int V, int QL, int nm);
 
