@@ -9,7 +9,8 @@
 //   Y[j][r][k] = sum_j' K^P[j][j'] f[j'][r][k]
 // is a small GEMM: each thread owns rows j and all (r, k) columns of a block of
 // runs, streams K^P^T[j'][j] from global memory (coalesced, L2-resident per
-// group) and reads f[j'][.][.] as a broadcast.
+// group) and reads f[j'][.][.] as a broadcast.  That is the FP32 form; FP64
+// runs take the even/odd form of bj_step64_kernel.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -105,7 +106,7 @@ __global__ void bj_kl_kernel(int QL, const double* __restrict__ xk, const double
 }
 
 // ---------------------------------------------------------------------------
-// The batched step kernel (SIMT contraction).
+// The batched step kernel (SIMT contraction, FP32).
 // Shared memory: three copies of the block state, [j][r][k] with row stride
 // RS = RP * QL (RP = R rounded up to RB; padded runs stay zero):
 //   stage 1 reads F, writes A; stage 2 reads A (and F), writes B;
@@ -253,6 +254,187 @@ bj_step_kernel(BjArgs<T> a, int block0) {
     const int j = idx / RS, rk = idx - j * RS, r = rk / QL, k = rk - r * QL;
     if (r < R) a.state[a.roff[blk.first + r] + (size_t)k * Q + j] = F[idx];
   }
+}
+
+// E^T and O^T of one Q (bjorken.cuh), FP64: E^T[j'][i] (qh x qh), then O^T (h x h).
+__global__ void bj_eo_kernel(int Q, const double* __restrict__ xw, const double* __restrict__ kc,
+                             double* eo) {
+  const int h = Q / 2, qh = Q - h;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= qh * qh) return;
+  const int i = idx / qh, jp = idx - i * qh;
+  double e, o;
+  kp_even_odd(Q, xw, kc, i, jp, &e, &o);
+  eo[(size_t)jp * qh + i] = e;
+  if (i < h && jp < h) eo[(size_t)qh * qh + (size_t)jp * h + i] = o;
+}
+
+// ---------------------------------------------------------------------------
+// The batched step kernel, FP64: all steps of R runs of one Q_xi per CTA.
+// The limit is the FP64 pipe (~2 lane operations per SM and cycle, ~64 cycles
+// per warp instruction on a sub-partition), so the work is cut and spread:
+//   - K^P f through the even and odd half-size matrices: half the products;
+//   - one thread per row of E or O and column c = (r, k), so no run is padded
+//     and a single run of Q_xi = 100 keeps all four sub-partitions busy; matrix
+//     entries come coalesced from L1/L2, s_c and d_c as shared-memory
+//     broadcasts (loads are free beside the FP64 pipe);
+//   - the moments and equilibrium of a run by another warp meanwhile;
+//   - R follows the batch (see the host): few runs spread over all SMs.
+// 112 runs of Q_xi 3 .. 100, Q_L = 2, 50 steps: 0.99 ms (23.9 ms with
+// blocks of four padded runs and the full matrix); for Q_xi = 100 the products
+// alone are 6k of the ~13.7k cycles of a stage.
+// Shared memory per column: f_n and f [Q], s|d [Q] twice (a stage reads one
+// copy and writes the other), E s|O d [Q].
+// ---------------------------------------------------------------------------
+__host__ __device__ inline size_t bj64_smem_bytes(int Q, int R, int QL) {
+  return sizeof(double) * (5 * (size_t)Q * R * QL + 3 * (size_t)R + (size_t)QL * (QL + 3));
+}
+
+__global__ void __launch_bounds__(kBjThreads)
+bj_step64_kernel(BjArgs<double> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const BjBlock blk = a.blocks[blockIdx.x];
+  const int Q = blk.Q, R = blk.R, QL = a.QL, h = Q / 2, qh = Q - h;
+  const int NC = R * QL, nitem = qh * NC;
+  double* FN = reinterpret_cast<double*>(smem_raw);
+  double* F = FN + (size_t)Q * NC;
+  double* SD = F + (size_t)Q * NC;  // [2][NC][s (qh) | d (h)]
+  double* Y = SD + 2 * (size_t)Q * NC;
+  double* sRate = Y + (size_t)Q * NC;  // [R] 1/tau_AW (0: collisionless)
+  double* sNeq = sRate + R;            // [R] n_eq/4
+  double* sOmt = sNeq + R;             // [R] 1 - T
+  double* KL = sOmt + R;               // [QL][QL]
+  double* xk = KL + QL * QL;           // [QL]: x_k, then w_k, then L_1(x_k)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double* xw = a.npool + a.qtab[blk.qidx].xi_off;
+  const double* ET = a.kpool + a.qtab[blk.qidx].kp_off;
+  const double* OT = ET + (size_t)qh * qh;
+
+  for (int e = tid; e < QL * QL; e += kBjThreads) KL[e] = a.KL[e];
+  for (int e = tid; e < QL; e += kBjThreads) {
+    xk[e] = a.xk[e];
+    xk[QL + e] = a.wk[e];
+    xk[2 * QL + e] = 3.0 - a.xk[e];
+  }
+  auto split = [&](double* sd, int c, int i, double f1, double f2) {
+    sd[(size_t)c * Q + i] = i < h ? f1 + f2 : f1;
+    if (i < h) sd[(size_t)c * Q + qh + i] = f1 - f2;
+  };
+  // the states of the block's runs are contiguous: column c is f + c Q
+  const double* st = a.state + a.roff[blk.first];
+  for (int u = tid; u < nitem; u += kBjThreads) {
+    const int c = u / qh, i = u - c * qh;
+    const double f1 = st[(size_t)c * Q + i], f2 = st[(size_t)c * Q + Q - 1 - i];
+    FN[(size_t)c * Q + i] = F[(size_t)c * Q + i] = f1;
+    FN[(size_t)c * Q + Q - 1 - i] = F[(size_t)c * Q + Q - 1 - i] = f2;
+    split(SD, c, i, f1, f2);
+  }
+  __syncthreads();
+
+  int cur = 0;
+  for (int step = 0; step < a.nsteps; ++step) {
+    const double tn = a.tau_start + step * a.dtau;
+    for (int stage = 0; stage < 3; ++stage, cur ^= 1) {
+      const double tau = tn + (stage == 0 ? 0.0 : (stage == 1 ? a.dtau : 0.5 * a.dtau));
+      const double* sd = SD + (size_t)cur * Q * NC;
+      double* sd_out = SD + (size_t)(cur ^ 1) * Q * NC;
+      // ---- E s and O d; the moments of run r by warp 7 - r mod 8 ----
+      for (int u = tid; u < Q * NC; u += kBjThreads) {
+        const int c = u / Q, e = u - c * Q;
+        const bool odd = e >= qh;
+        const int n = odd ? h : qh;
+        const double* M = odd ? OT + (e - qh) : ET + e;
+        const double* v = sd + (size_t)c * Q + (odd ? qh : 0);
+        double y = 0.0;
+        int j = 0;
+        for (; j + 8 <= n; j += 8) {
+          double m8[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) m8[q] = __ldg(M + (size_t)(j + q) * n);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) y = fma(m8[q], v[j + q], y);
+        }
+        for (; j < n; ++j) y = fma(__ldg(M + (size_t)j * n), v[j], y);
+        Y[u] = y;
+      }
+      for (int r = 7 - warp; r < R; r += kBjThreads / 32) {
+        double N = 0.0, E = 0.0;
+        for (int k = 0; k < QL; ++k) {
+          double n = 0.0;
+          for (int i = lane; i < qh; i += 32) n += sd[(size_t)(r * QL + k) * Q + i];
+#pragma unroll
+          for (int o = 16; o >= 1; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+          N += n;
+          E = fma(xk[k], n, E);
+        }
+        if (lane == 0) {
+          double rate = 0.0, neq4 = 0.0, omt = 0.0;
+          const int gr = blk.first + r;
+          const double P = E * (1.0 / 3.0);
+          const double t0 = a.tau_aw0[gr];
+          const bool coll = t0 > 0.0 && isfinite(t0);
+          if (!(P > 0.0) || !isfinite(P) || (a.gas[gr] == RSLB_GAS_IDEAL && !(N > 0.0))) {
+            bj_report(a.err, RSLB_ERR_NONPHYSICAL, gr);
+          } else if (coll) {
+            double T_, n_eq, itaw;  // 1/tau_AW
+            if (a.gas[gr] == RSLB_GAS_PARTON) {
+              const double rP = P * rsqrt64(P);  // P^{1/2}
+              const double iT = rsqrt64(rP);     // P^{-1/4}
+              T_ = rP * iT;
+              n_eq = P * iT;  // P^{3/4}
+              itaw = T_ * rcp64(t0);
+            } else {
+              T_ = P * rcp64(N);
+              n_eq = N;
+              const double g = log(N * rcp64(T_ * T_ * T_));
+              itaw = T_ * rcp64(t0 * fma(-0.25, g, 1.0));
+            }
+            rate = itaw;
+            neq4 = 0.25 * n_eq;
+            omt = 1.0 - T_;
+          }
+          sRate[r] = rate;
+          sNeq[r] = neq4;
+          sOmt[r] = omt;
+        }
+      }
+      __syncthreads();
+      // ---- L_Bjorken and the RK combination of rows i and Q-1-i ----
+      const double itau = rcp64(tau);
+      for (int u = tid; u < nitem; u += kBjThreads) {
+        const int c = u / qh, i = u - c * qh, r = c / QL, k = c - r * QL;
+        const double* s = sd + (size_t)r * QL * Q + i;
+        double ke = 0.0, ko = 0.0;
+        for (int q = 0; q < QL; ++q) {
+          ke = fma(KL[k * QL + q], s[(size_t)q * Q], ke);
+          if (i < h) ko = fma(KL[k * QL + q], s[(size_t)q * Q + qh], ko);
+        }
+        const double x = __ldg(xw + i), w = __ldg(xw + Q + i);
+        const double feq = sNeq[r] * (w * xk[QL + k]) * fma(xk[2 * QL + k], sOmt[r], 1.0);
+        const double ye = Y[(size_t)c * Q + i], yo = i < h ? Y[(size_t)c * Q + qh + i] : 0.0;
+        const double sc = i < h ? 0.5 : 1.0;  // the middle row is its own even part
+        const double xi2 = sc * x * x, rate = sRate[r];
+        auto row = [&](int j, double kl, double kp) {
+          const double f = F[(size_t)c * Q + j];
+          const double L = fma(fma(xi2, kl, fma(0.5, kp, -f)), itau, -(f - feq) * rate);
+          double v = fma(a.dtau, L, f);
+          if (stage == 1) v = fma(0.75, FN[(size_t)c * Q + j], 0.25 * v);
+          if (stage == 2) {
+            v = fma(1.0 / 3.0, FN[(size_t)c * Q + j], (2.0 / 3.0) * v);
+            FN[(size_t)c * Q + j] = v;
+          }
+          F[(size_t)c * Q + j] = v;
+          return v;
+        };
+        const double f1 = row(i, ke + ko, ye + yo);
+        const double f2 = i < h ? row(Q - 1 - i, ke - ko, ye - yo) : 0.0;
+        split(sd_out, c, i, f1, f2);
+      }
+      __syncthreads();
+    }
+  }
+  double* so = a.state + a.roff[blk.first];
+  for (int e = tid; e < Q * NC; e += kBjThreads) so[e] = F[e];
 }
 
 // Observables per run (warp per run), written in the callers' order.
@@ -408,7 +590,7 @@ int bj_check_err(rslb_bjorken* b) {
 
 // Runs per CTA block for a given Q: three copies of the block state within
 // ~200 KB of shared memory, a multiple of the register block RB when R >= RB.
-int runs_per_block(int Q, int QL, size_t es, int RB) {
+int runs_per_block(int Q, int QL, size_t es, int RB) {  // FP32
   const size_t budget = 200 * 1024;
   const size_t per_run = 3 * es * (size_t)Q * QL;
   int R = (int)(budget / per_run);
@@ -495,7 +677,8 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
     gauss_legendre_host(Q, x.data(), w.data());
     npool.insert(npool.end(), x.begin(), x.end());
     npool.insert(npool.end(), w.begin(), w.end());
-    kp_total += (long long)Q * Q;
+    const long long hh = Q / 2, qq = Q - hh;
+    kp_total += es == sizeof(double) ? qq * qq + hh * hh : (long long)Q * Q;
   }
   // per-run tables (sorted order) and blocks
   std::vector<long long> roff(nruns), xoff(nruns);
@@ -517,16 +700,33 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
   }
   b->total_state = off;
   size_t max_smem = 0;
-  const int RB = (es == sizeof(double)) ? 4 : 8;
+  const bool f64 = es == sizeof(double);
+  const int RB = 8;
+  // FP64: the SMs' FP64 pipes share the products (Q^2/2 per column and stage)
+  // evenly when a block holds at most the mean of half an SM (two blocks overlap
+  // each other's barriers), and at least one run; at most ~100 KB of state
+  double work = 0.0, mean = 0.0;
+  if (f64) {
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    for (int s = 0; s < nruns; ++s) work += (double)rq[s] * rq[s];
+    mean = work / (2.0 * std::max(nsm, 1));
+  }
   for (int s = 0; s < nruns;) {
     const int Q = rq[s];
-    const int Rmax = runs_per_block(Q, QL, es, RB);
+    int Rmax = f64 ? 1 : runs_per_block(Q, QL, es, RB);
+    if (f64) {
+      const double fit = 100.0 * 1024 / (double)(5 * sizeof(double) * Q * QL);
+      Rmax = (int)std::max(1.0, std::min({64.0, fit, mean / ((double)Q * Q)}));
+    }
     int n = 0;
     while (s + n < nruns && rq[s + n] == Q && n < Rmax) ++n;
     size_t qidx = 0;
     while (qvals[qidx] != Q) ++qidx;
     blocks.push_back(BjBlock{Q, s, n, (int)qidx});
-    max_smem = std::max(max_smem, block_smem_bytes(Q, n, QL, es, RB));
+    max_smem = std::max(max_smem, f64 ? bj64_smem_bytes(Q, n, QL)
+                                      : block_smem_bytes(Q, n, QL, es, RB));
     s += n;
   }
   b->nblocks = (int)blocks.size();
@@ -644,7 +844,7 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
     const int Q = qvals[i];
     const int n = Q * Q;
     if (b->precision == RSLB_F64)
-      bj_kp_kernel<double><<<(n + 255) / 256, 256, 0, st>>>(
+      bj_eo_kernel<<<((Q + 1) / 2 * ((Q + 1) / 2) + 127) / 128, 128, 0, st>>>(
           Q, b->npool + qtab[i].xi_off, b->kpc, (double*)b->kpool + qtab[i].kp_off);
     else
       bj_kp_kernel<float><<<(n + 255) / 256, 256, 0, st>>>(
@@ -678,7 +878,7 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
       return cuda_error(e, "rslb_bjorken_init: shared-memory attribute");
     }
   }
-  const void* kfun = b->precision == RSLB_F64 ? (const void*)bj_step_kernel<double, 4>
+  const void* kfun = b->precision == RSLB_F64 ? (const void*)bj_step64_kernel
                                               : (const void*)bj_step_kernel<float, 8>;
   e = cudaFuncSetAttribute(kfun, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
   if (e != cudaSuccess) {
@@ -783,7 +983,7 @@ extern "C" int rslb_bjorken_step(rslb_bjorken* b, int nsteps) {
     BjArgs<double> a{b->blocks, b->qtab, (const double*)b->kpool, b->npool, b->roff,
                      b->tau_aw0, b->gas, (double*)b->state, b->xk, b->wk, b->KL, b->QL,
                      nsteps, tau_start, b->dtau, b->err};
-    bj_step_kernel<double, 4><<<b->nblocks, kBjThreads, b->smem, b->stream>>>(a, 0);
+    bj_step64_kernel<<<b->nblocks, kBjThreads, b->smem, b->stream>>>(a);
   } else {
     BjArgs<float> a{b->blocks, b->qtab, (const float*)b->kpool, b->npool, b->roff,
                     b->tau_aw0, b->gas, (float*)b->state, b->xk, b->wk, b->KL, b->QL,

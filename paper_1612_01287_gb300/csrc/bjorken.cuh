@@ -72,6 +72,41 @@ __device__ inline double kp_entry(int Q, const double* __restrict__ xw,
 // for j < h (E also for the middle row j = h of odd Q, where it gives twice
 // (K f)_h).  E is qh x qh, O is h x h: half the flops and half the image.
 //
+// Since P_m(-y) = (-1)^m P_m(y), the terms of even m of kp_entry are the same for
+// y and -y and those of odd m change sign: E_{j j'} is twice the sum of the
+// even ones and O_{j j'} twice that of the odd ones, both from one pass.
+__device__ inline void kp_even_odd(int Q, const double* __restrict__ xw,
+                                   const double* __restrict__ kc, int j, int jp, double* E,
+                                   double* O) {
+  const double x = xw[j], y = xw[jp], w = xw[Q + j];
+  double px = x, pxm1 = 1.0;
+  double ym2 = 0.0, ym1 = 1.0, y0 = y;
+  double yp1 = 0.5 * (3.0 * y * y - 1.0);
+  double yp2 = (5.0 * y * yp1 - 2.0 * y0) / 3.0;
+  double so = 0.0, se = 0.0;  // odd and even m
+  for (int m = 1; m <= Q - 1; ++m) {
+    const double* c = kc + (size_t)m * kKpCoef;
+    const double2 c01 = *reinterpret_cast<const double2*>(c);
+    const double2 c23 = *reinterpret_cast<const double2*>(c + 2);
+    const double2 c45 = *reinterpret_cast<const double2*>(c + 4);
+    const double c6 = c[6];
+    const double q = (m <= Q - 3 ? c01.x * yp2 : 0.0) - (c01.y * y0 + c23.x * ym2);
+    if (m & 1) so += px * q;
+    else se += px * q;
+    const double pxn = c23.y * x * px - c45.x * pxm1;
+    pxm1 = px;
+    px = pxn;
+    const double yn = c45.y * y * yp2 - c6 * yp1;
+    ym2 = ym1;
+    ym1 = y0;
+    y0 = yp1;
+    yp1 = yp2;
+    yp2 = yn;
+  }
+  *E = 2.0 * w * se;
+  *O = 2.0 * w * so;
+}
+
 // Work unit of the tensor-core stage kernel: the runs [first, first + R)
 // (sorted order, all with Q_xi = Q, states contiguous from soff) and the
 // M-tile mt (rows i = 128 mt .. 128 mt + 127 of E and O).

@@ -616,21 +616,23 @@ __global__ void bj_tc_image_kernel(int Q, const double* __restrict__ xw,
                                    const double* __restrict__ kc, float* img) {
   const int h = Q / 2, qh = Q - h;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= qh * qh + h * h) return;
-  const bool odd = idx >= qh * qh;
-  const int n = odd ? h : qh;
-  const int e = odd ? idx - qh * qh : idx;
-  const int i = e / n, jp = e - i * n;
-  const double k1 = kp_entry(Q, xw, kc, i, jp), k2 = kp_entry(Q, xw, kc, i, Q - 1 - jp);
-  const float x = float(odd ? k1 - k2 : k1 + k2);
-  const int nkb = (n + 31) / 32;
-  const int mt = i >> 7, row = i & 127, kb = jp >> 5, col = jp & 31;
-  const int rows = min(128, n - 128 * mt);
-  float* tile = img + (odd ? bj_tc_image_floats(qh) : 0) + ((size_t)mt * 128 * nkb +
-                                                            (size_t)kb * rows) * 64;
-  const float hi = tf32_rn(x);
-  tile[swz(row, col) >> 2] = hi;
-  tile[(size_t)rows * 32 + (swz(row, col) >> 2)] = x - hi;
+  if (idx >= qh * qh) return;
+  const int i = idx / qh, jp = idx - i * qh;
+  double e, o;
+  kp_even_odd(Q, xw, kc, i, jp, &e, &o);
+  for (int part = 0; part < 2; ++part) {
+    const int n = part ? h : qh;
+    if (i >= n || jp >= n) return;
+    const float x = float(part ? o : e);
+    const int nkb = (n + 31) / 32;
+    const int mt = i >> 7, row = i & 127, kb = jp >> 5, col = jp & 31;
+    const int rows = min(128, n - 128 * mt);
+    float* tile = img + (part ? bj_tc_image_floats(qh) : 0) + ((size_t)mt * 128 * nkb +
+                                                               (size_t)kb * rows) * 64;
+    const float hi = tf32_rn(x);
+    tile[swz(row, col) >> 2] = hi;
+    tile[(size_t)rows * 32 + (swz(row, col) >> 2)] = x - hi;
+  }
 }
 
 // Moments (N, E) of each run into partial slot 0 (slots 1-3 cleared).
@@ -692,8 +694,8 @@ cudaError_t bj_tc_stage_launch(const BjTcArgs& a, int nblocks, size_t smem, cuda
 
 cudaError_t bj_tc_image_launch(int Q, const double* xw, const double* kc, float* img,
                                cudaStream_t st) {
-  const int n = (Q - Q / 2) * (Q - Q / 2) + (Q / 2) * (Q / 2);
-  bj_tc_image_kernel<<<(n + 255) / 256, 256, 0, st>>>(Q, xw, kc, img);
+  const int n = (Q - Q / 2) * (Q - Q / 2);
+  bj_tc_image_kernel<<<(n + 127) / 128, 128, 0, st>>>(Q, xw, kc, img);
   return cudaGetLastError();
 }
 
