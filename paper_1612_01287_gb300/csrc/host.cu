@@ -781,15 +781,48 @@ struct rslb_sod_batch {
   int nsm;
   cudaGraphExec_t graph;
   bool graph_failed;
+  // one stream per class after the first (empty: all classes on `stream`), and
+  // the events that fork them from and join them to `stream`
+  std::vector<cudaStream_t> side;
+  std::vector<cudaEvent_t> joined;
+  cudaEvent_t forked;
 };
 
 namespace {
 
-__global__ void batch_step_increment(long long* step) { *step += 1; }
+__global__ void batch_step_increment(long long* step, int n) { *step += n; }
+
+void batch_free_streams(rslb_sod_batch* b) {
+  for (cudaStream_t s : b->side) cudaStreamDestroy(s);
+  for (cudaEvent_t e : b->joined) cudaEventDestroy(e);
+  if (b->forked) cudaEventDestroy(b->forked);
+  b->side.clear();
+  b->joined.clear();
+  b->forked = nullptr;
+}
+
+// The side streams; without them the classes run one after another.
+void batch_make_streams(rslb_sod_batch* b) {
+  if (b->cls.size() < 2) return;
+  bool ok = cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming) == cudaSuccess;
+  for (size_t i = 1; i < b->cls.size() && ok; ++i) {
+    cudaStream_t s = nullptr;
+    cudaEvent_t e = nullptr;
+    ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
+    if (ok) b->side.push_back(s);
+    ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (ok) b->joined.push_back(e);
+  }
+  if (!ok) {
+    batch_free_streams(b);
+    cudaGetLastError();
+  }
+}
 
 void batch_free(rslb_sod_batch* b) {
   if (!b) return;
   if (b->graph) cudaGraphExecDestroy(b->graph);
+  batch_free_streams(b);
   for (auto& c : b->cls) {
     if (c.runs_dev) cudaFree(c.runs_dev);
     if (c.maps_dev) cudaFree(c.maps_dev);
@@ -801,22 +834,45 @@ void batch_free(rslb_sod_batch* b) {
   delete b;
 }
 
+// Tiles of one class per resident CTA and launch, at most, when classes run side
+// by side: a CTA that holds its place for a few tiles only lets the block
+// scheduler fill in other classes; the cap keeps the launches of finished
+// runs (whose CTAs return at once) short.
+constexpr int kBatchWaves = 4;
+
+// nsteps steps of every class.  The classes share nothing, so each is a chain of
+// its own on its own stream: a class whose tiles do not fill the GPU, or whose
+// last wave is nearly empty, leaves the SMs to the others instead of holding
+// them up three times a step.  The step counter advances once, after all of
+// them; a launch knows its step within the call (step_off).
 template <typename T>
 cudaError_t batch_enqueue(rslb_sod_batch* b, int nsteps) {
-  for (int n = 0; n < nsteps; ++n) {
-    for (int stage = 0; stage < 3; ++stage)
-      for (const SodClass& c : b->cls) {
-        cudaError_t e = sod_batch_stage_launch<T>(
-            c.B, c.smem, c.ctas_per_sm * b->nsm, (const SodRunDesc<T>*)c.runs_dev, c.tasks_dev,
-            c.ntasks, b->step_dev, stage, b->err, c.V, c.QL, c.nm, b->stream,
-            c.B == kSod32Cells ? c.maps_dev : nullptr);
-        if (e != cudaSuccess) return e;
-      }
-    batch_step_increment<<<1, 1, 0, b->stream>>>(b->step_dev);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  const bool fork = !b->side.empty();
+  if (fork) e = cudaEventRecord(b->forked, b->stream);
+  for (size_t i = 0; i < b->cls.size() && e == cudaSuccess; ++i) {
+    const SodClass& c = b->cls[i];
+    cudaStream_t st = fork && i > 0 ? b->side[i - 1] : b->stream;
+    if (st != b->stream) e = cudaStreamWaitEvent(st, b->forked, 0);
+    for (int n = 0; n < nsteps; ++n)
+      for (int stage = 0; stage < 3 && e == cudaSuccess; ++stage)
+        e = sod_batch_stage_launch<T>(
+            c.B, c.smem, std::min(c.ntasks, c.ctas_per_sm * b->nsm * (fork ? kBatchWaves : 1)),
+            (const SodRunDesc<T>*)c.runs_dev, c.tasks_dev, c.ntasks, b->step_dev, n, stage,
+            b->err, c.V, c.QL, c.nm, st, c.B == kSod32Cells ? c.maps_dev : nullptr);
+    if (st != b->stream) {
+      // joined even after an error, so that a capture on `stream` can end
+      const cudaError_t j = cudaEventRecord(b->joined[i - 1], st);
+      if (e == cudaSuccess) e = j;
+    }
   }
-  return cudaSuccess;
+  for (size_t i = 0; i < b->joined.size() && fork; ++i) {
+    const cudaError_t j = cudaStreamWaitEvent(b->stream, b->joined[i], 0);
+    if (e == cudaSuccess) e = j;
+  }
+  if (e != cudaSuccess) return e;
+  batch_step_increment<<<1, 1, 0, b->stream>>>(b->step_dev, nsteps);
+  return cudaGetLastError();
 }
 
 // Tuning results of this process: (device, FP64, V, Q_L, N_Omega + 1) ->
@@ -936,12 +992,14 @@ int batch_build_classes(rslb_sod_batch* b, int autotune) {
           cudaEventCreate(&e1);
           // stage 0 reads F0 and writes F1 only: safe to repeat
           sod_batch_stage_launch<T>(B, smem, k * b->nsm, (const SodRunDesc<T>*)c.runs_dev, td,
-                                    (int)tasks.size(), b->step_dev, 0, b->err, V, QL, nm, b->stream,
+                                    (int)tasks.size(), b->step_dev, 0, 0, b->err, V, QL, nm,
+                                    b->stream,
                                     B == kSod32Cells ? c.maps_dev : nullptr);
           cudaEventRecord(e0, b->stream);
           for (int rep = 0; rep < 3; ++rep)
             sod_batch_stage_launch<T>(B, smem, k * b->nsm, (const SodRunDesc<T>*)c.runs_dev, td,
-                                      (int)tasks.size(), b->step_dev, 0, b->err, V, QL, nm, b->stream,
+                                      (int)tasks.size(), b->step_dev, 0, 0, b->err, V, QL, nm,
+                                      b->stream,
                                       B == kSod32Cells ? c.maps_dev : nullptr);
           cudaEventRecord(e1, b->stream);
           cudaEventSynchronize(e1);
@@ -1003,6 +1061,7 @@ extern "C" int rslb_sod_batch_init(rslb_sod_batch** out, const rslb_sod_run* run
   b->total_cv = 0.0;
   b->graph = nullptr;
   b->graph_failed = false;
+  b->forked = nullptr;
   int rc = RSLB_OK;
   for (int r = 0; r < nruns && !rc; ++r) {
     const rslb_sod_run& R = runs[r];
@@ -1067,6 +1126,13 @@ extern "C" int rslb_sod_batch_init(rslb_sod_batch** out, const rslb_sod_run* run
     cudaMemset(b->err, 0, 2 * sizeof(int));
     rc = b->fp64 ? batch_build_classes<double>(b, o->autotune)
                  : batch_build_classes<float>(b, o->autotune);
+  }
+  if (!rc) {
+    // the heaviest classes are launched first (rslb_sod_batch_tuning lists them by V)
+    std::stable_sort(b->cls.begin(), b->cls.end(), [](const SodClass& x, const SodClass& y) {
+      return (double)x.V * x.ntasks * x.B > (double)y.V * y.ntasks * y.B;
+    });
+    batch_make_streams(b);
   }
   if (rc) {
     batch_free(b);
@@ -1137,9 +1203,15 @@ extern "C" int rslb_sod_batch_tuning(const rslb_sod_batch* b, int g, int* V, int
   clear_error();
   if (!b || g < 0 || g >= (int)b->cls.size())
     return set_error(RSLB_ERR_ARG, "rslb_sod_batch_tuning: bad group");
-  if (V) *V = b->cls[g].V;
-  if (tile_cells) *tile_cells = b->cls[g].B;
-  if (ctas_per_sm) *ctas_per_sm = b->cls[g].ctas_per_sm;
+  // groups in ascending (V, N_Omega)
+  std::vector<const SodClass*> by;
+  for (const SodClass& c : b->cls) by.push_back(&c);
+  std::sort(by.begin(), by.end(), [](const SodClass* x, const SodClass* y) {
+    return std::tie(x->V, x->nm) < std::tie(y->V, y->nm);
+  });
+  if (V) *V = by[g]->V;
+  if (tile_cells) *tile_cells = by[g]->B;
+  if (ctas_per_sm) *ctas_per_sm = by[g]->ctas_per_sm;
   return RSLB_OK;
 }
 

@@ -771,9 +771,9 @@ sod_stage_kernel(const T* __restrict__ fin, const T* __restrict__ fn, T* fout, i
 template <typename T, int B, int NT>
 __global__ void __launch_bounds__(NT, 2)
 sod_batch_kernel(const SodRunDesc<T>* __restrict__ runs, const SodTask* __restrict__ tasks,
-                 int ntasks, const long long* __restrict__ step, int stage, int* err, int nseg,
-                 int np) {
-  const long long n = *step;
+                 int ntasks, const long long* __restrict__ step, int step_off, int stage,
+                 int* err, int nseg, int np) {
+  const long long n = *step + step_off;
   for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
     const SodTask tk = tasks[t];
     const SodRunDesc<T> R = runs[tk.run];
@@ -949,15 +949,15 @@ size_t sod_stage_smem_bytes(bool fp64, int B, int V, int QL, int nm) {
 }
 
 cudaError_t sod32_batch_launch(size_t smem, int grid, const SodRunDesc<float>* runs,
-                               const SodTask* tasks, int ntasks, const long long* step, int stage,
-                               int* err, const void* maps, cudaStream_t st);
+                               const SodTask* tasks, int ntasks, const long long* step, int step_off,
+                               int stage, int* err, const void* maps, cudaStream_t st);
 
 // Batched stages: all runs of a class share V (so nseg and the tile width).
 template <typename T, int B>
 static cudaError_t batch_b(size_t smem, int grid, const SodRunDesc<T>* runs, const SodTask* tasks,
-                           int ntasks, const long long* step, int stage, int* err, int V, int QL,
+                           int ntasks, const long long* step, int step_off, int stage, int* err, int V, int QL,
                            int nm, cudaStream_t st) {
-  sod_batch_kernel<T, B, kNT><<<grid, kNT, smem, st>>>(runs, tasks, ntasks, step, stage, err,
+  sod_batch_kernel<T, B, kNT><<<grid, kNT, smem, st>>>(runs, tasks, ntasks, step, step_off, stage, err,
                                                        pick_nseg(V, B, V16<T>::n),
                                                        pick_np<T>(V, B, QL, nm));
   return cudaGetLastError();
@@ -966,23 +966,24 @@ static cudaError_t batch_b(size_t smem, int grid, const SodRunDesc<T>* runs, con
 template <typename T>
 cudaError_t sod_batch_stage_launch(int B, size_t smem, int grid, const SodRunDesc<T>* runs,
                                    const SodTask* tasks, int ntasks, const long long* step,
-                                   int stage, int* err, int V, int QL, int nm, cudaStream_t st,
+                                   int step_off, int stage, int* err, int V, int QL, int nm, cudaStream_t st,
                                    const void* maps) {
   if (ntasks == 0) return cudaSuccess;
   if constexpr (sizeof(T) == 4) {
     switch (B) {
       case kSod32Cells:
-        return sod32_batch_launch(smem, grid, runs, tasks, ntasks, step, stage, err, maps, st);
-      case 128: return batch_b<T, 128>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
-      case 64: return batch_b<T, 64>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
-      case 32: return batch_b<T, 32>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
-      case 16: return batch_b<T, 16>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+        return sod32_batch_launch(smem, grid, runs, tasks, ntasks, step, step_off, stage, err, maps,
+                                  st);
+      case 128: return batch_b<T, 128>(smem, grid, runs, tasks, ntasks, step, step_off, stage, err, V, QL, nm, st);
+      case 64: return batch_b<T, 64>(smem, grid, runs, tasks, ntasks, step, step_off, stage, err, V, QL, nm, st);
+      case 32: return batch_b<T, 32>(smem, grid, runs, tasks, ntasks, step, step_off, stage, err, V, QL, nm, st);
+      case 16: return batch_b<T, 16>(smem, grid, runs, tasks, ntasks, step, step_off, stage, err, V, QL, nm, st);
       default: break;
     }
   } else {
     switch (B) {
-      case 16: return batch_b<T, 16>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
-      case 8: return batch_b<T, 8>(smem, grid, runs, tasks, ntasks, step, stage, err, V, QL, nm, st);
+      case 16: return batch_b<T, 16>(smem, grid, runs, tasks, ntasks, step, step_off, stage, err, V, QL, nm, st);
+      case 8: return batch_b<T, 8>(smem, grid, runs, tasks, ntasks, step, step_off, stage, err, V, QL, nm, st);
       default: break;
     }
   }
@@ -990,10 +991,10 @@ cudaError_t sod_batch_stage_launch(int B, size_t smem, int grid, const SodRunDes
 }
 
 template cudaError_t sod_batch_stage_launch<float>(int, size_t, int, const SodRunDesc<float>*,
-                                                   const SodTask*, int, const long long*, int,
+                                                   const SodTask*, int, const long long*, int, int,
                                                    int*, int, int, int, cudaStream_t, const void*);
 template cudaError_t sod_batch_stage_launch<double>(int, size_t, int, const SodRunDesc<double>*,
-                                                    const SodTask*, int, const long long*, int,
+                                                    const SodTask*, int, const long long*, int, int,
                                                     int*, int, int, int, cudaStream_t, const void*);
 
 // ---------------------------------------------------------------------------

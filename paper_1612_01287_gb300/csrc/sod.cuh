@@ -131,7 +131,7 @@ cudaError_t sod32p_stage_launch(const SodGeom& g, const SodTables<float>& tb, co
 template <typename T>
 cudaError_t sod_batch_stage_launch(int B, size_t smem, int grid, const SodRunDesc<T>* runs,
                                    const SodTask* tasks, int ntasks, const long long* step,
-                                   int stage, int* err, int V, int QL, int nm, cudaStream_t st,
+                                   int step_off, int stage, int* err, int V, int QL, int nm, cudaStream_t st,
                                    const void* maps = nullptr);
 size_t sod_stage_smem_bytes(bool fp64, int B, int V, int QL, int nm);
 

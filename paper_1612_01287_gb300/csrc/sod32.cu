@@ -170,9 +170,9 @@ sod32_stage_kernel(const float* __restrict__ fin, const float* __restrict__ fn, 
 // are staged by plain loads.
 __global__ void __launch_bounds__(kNT, kMinCtas)
 sod32_batch_kernel(const SodRunDesc<float>* __restrict__ runs, const SodTask* __restrict__ tasks,
-                   int ntasks, const long long* __restrict__ step, int stage, int* err,
+                   int ntasks, const long long* __restrict__ step, int step_off, int stage, int* err,
                    const CUtensorMap* __restrict__ maps) {
-  const long long n = *step;
+  const long long n = *step + step_off;
   int bar_uses = 0;
   for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
     const SodTask tk = tasks[t];
@@ -230,9 +230,9 @@ bool sod32_make_map(CUtensorMap* m, const float* f, int Z, int ldz, int V, int b
 }
 
 cudaError_t sod32_batch_launch(size_t smem, int grid, const SodRunDesc<float>* runs,
-                               const SodTask* tasks, int ntasks, const long long* step, int stage,
-                               int* err, const void* maps, cudaStream_t st) {
-  sod32_batch_kernel<<<grid, kNT, smem, st>>>(runs, tasks, ntasks, step, stage, err,
+                               const SodTask* tasks, int ntasks, const long long* step, int step_off,
+                               int stage, int* err, const void* maps, cudaStream_t st) {
+  sod32_batch_kernel<<<grid, kNT, smem, st>>>(runs, tasks, ntasks, step, step_off, stage, err,
                                               static_cast<const CUtensorMap*>(maps));
   return cudaGetLastError();
 }
