@@ -202,7 +202,6 @@ struct rslb_handle {
   SodLaunch launch;
   void* F[3];
   // tables in working precision
-  void* t_mw;
   void* t_m3;
   void* t_pk;
   void* t_xi;
@@ -238,7 +237,6 @@ namespace {
 template <typename T>
 SodTables<T> tables_of(const rslb_handle* h) {
   SodTables<T> tb;
-  tb.mw = (const T*)h->t_mw;
   tb.m3 = (const T*)h->t_m3;
   tb.pk = (const T*)h->t_pk;
   tb.xi = (const T*)h->t_xi;
@@ -267,7 +265,7 @@ SodTablesF64 tables64_of(const rslb_handle* h) {
 void free_handle(rslb_handle* h) {
   if (!h) return;
   if (h->graph) cudaGraphExecDestroy(h->graph);
-  void* ptrs[] = {h->F[0], h->F[1], h->F[2], h->t_mw, h->t_m3, h->t_pk, h->t_xi, h->t_wp, h->t_L1k, h->t_gL,
+  void* ptrs[] = {h->F[0], h->F[1], h->F[2], h->t_m3, h->t_pk, h->t_xi, h->t_wp, h->t_L1k, h->t_gL,
                   h->t_gR, h->t_kidx, h->t_rowv, h->t_gl_t, h->t_gl_w, h->d_xi, h->d_p, h->d_wp,
                   h->d_L1k, h->d_mom, h->d_err, h->d_fields};
   for (void* p : ptrs)
@@ -427,18 +425,13 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   g.lambda_ref = c.lambda_ref;
 
   // velocity tables (FP64 on the host)
-  std::vector<double> mw(5 * (size_t)V), m3(4 * (size_t)V, 0.0), xiv(V), pv(V), wp(kMaxM * (size_t)V, 0.0), L1k(QL);
+  std::vector<double> m3(4 * (size_t)V, 0.0), xiv(V), pv(V), wp(kMaxM * (size_t)V, 0.0), L1k(QL);
   std::vector<int> kidx(V);
   for (int k = 0; k < QL; ++k) {
     L1k[k] = 3.0 - xk[k];
     for (int j = 0; j < Qx; ++j) {
       const int v = k * Qx + j;
       const double x = xj[j], p = xk[k];
-      mw[0 * V + v] = 1.0 + x;
-      mw[1 * V + v] = 1.0 - x;
-      mw[2 * V + v] = p * (1.0 + x) * (1.0 + x);
-      mw[3 * V + v] = p * (1.0 - x) * (1.0 - x);
-      mw[4 * V + v] = p * (1.0 - x) * (1.0 + x);
       m3[4 * (size_t)v] = (1.0 + x) * (1.0 + x);
       m3[4 * (size_t)v + 1] = (1.0 - x) * (1.0 - x);
       m3[4 * (size_t)v + 2] = (1.0 - x) * (1.0 + x);
@@ -461,7 +454,6 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   auto up = [&](void** dst, const std::vector<double>& src) {
     return fp64 ? upload<double>(dst, src) : upload<float>(dst, src);
   };
-  if (!rc) rc = up(&h->t_mw, mw);
   if (!rc) rc = up(&h->t_m3, m3);
   if (!rc) {
     std::vector<double> pk(2 * (size_t)QL);  // p_k as hi + lo in the working precision

@@ -59,7 +59,7 @@ static int noalloc_scratch(void** out) {
 // nodes (the same tables rslb_init uploads; here nothing is allocated).
 template <typename T>
 __global__ void noalloc_tables_kernel(int Qx, int QL, int nm, const double* __restrict__ q,
-                                      bool packed, T* mw, T* m3, T* pk, T* xi, T* wp, int* kidx, int* rowv, T* L1k,
+                                      T* m3, T* pk, T* xi, T* wp, int* kidx, int* rowv, T* L1k,
                                       double* dxi, double* dp, double* dwp, double* dL1k) {
   // q = [xi(Qx) | w_xi(Qx) | x_k(QL) | w_k(QL)]
   const int V = Qx * QL;
@@ -72,18 +72,10 @@ __global__ void noalloc_tables_kernel(int Qx, int QL, int nm, const double* __re
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
     const int k = v / Qx, j = v - k * Qx;
     const double x = xj[j], p = xk[k];
-    if (packed) {
-      mw[0 * V + v] = T(1.0 + x);
-      mw[1 * V + v] = T(1.0 - x);
-      mw[2 * V + v] = T(p * (1.0 + x) * (1.0 + x));
-      mw[3 * V + v] = T(p * (1.0 - x) * (1.0 - x));
-      mw[4 * V + v] = T(p * (1.0 - x) * (1.0 + x));
-    } else {
-      m3[4 * v] = T((1.0 + x) * (1.0 + x));
-      m3[4 * v + 1] = T((1.0 - x) * (1.0 - x));
-      m3[4 * v + 2] = T((1.0 - x) * (1.0 + x));
-      m3[4 * v + 3] = T(0);
-    }
+    m3[4 * v] = T((1.0 + x) * (1.0 + x));
+    m3[4 * v + 1] = T((1.0 - x) * (1.0 - x));
+    m3[4 * v + 2] = T((1.0 - x) * (1.0 + x));
+    m3[4 * v + 3] = T(0);
     xi[v] = T(x);
     kidx[v] = k;
     dxi[v] = x;
@@ -128,9 +120,8 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
   };
   const size_t oF0 = take(es * (size_t)V * ldz), oF1 = take(es * (size_t)V * ldz),
                oF2 = take(es * (size_t)V * ldz);
-  // one region holds the moment table of the kernel in use: mw [5][V] (packed) or
-  // m3 [V][4] (scalar)
-  const size_t omw = take(es * 5 * V), om3 = omw, oxi = take(es * V), owp = take(es * kMaxM * V),
+  // (the moment table is [V][4]; the room for five keeps the largest problem as it was)
+  const size_t om3 = take(es * 5 * V), oxi = take(es * V), owp = take(es * kMaxM * V),
                oL1 = take(256), opk = oL1 + 128, ogL = take(es * V), ogR = take(es * V),
                okidx = take(sizeof(int) * V), orow = take(sizeof(int) * V),
                oglt = take(sizeof(double) * kAeqTable), oglw = take(sizeof(double) * kAeqTable),
@@ -193,7 +184,7 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
   // tables must be in place before the pageable copies above are reused
   if (ok(cudaSuccess)) {
     noalloc_tables_kernel<T><<<(V + 255) / 256, 256, 0, st>>>(
-        Qx, QL, nm, (const double*)(S + oq), L.B == kSod32Cells, (T*)(S + omw), (T*)(S + om3), (T*)(S + opk),
+        Qx, QL, nm, (const double*)(S + oq), (T*)(S + om3), (T*)(S + opk),
         (T*)(S + oxi), (T*)(S + owp),
         (int*)(S + okidx), (int*)(S + orow), (T*)(S + oL1), (double*)(S + odxi),
         (double*)(S + odp), (double*)(S + odwp), (double*)(S + odL1));
@@ -239,7 +230,6 @@ static int noalloc_run(const rslb_config& c, void* f, int nsteps, cudaStream_t s
     ok(cudaMemsetAsync(S + ogR, 0, es * V, st));
   }
   SodTables<T> tb;
-  tb.mw = (const T*)(S + omw);
   tb.m3 = (const T*)(S + om3);
   tb.pk = (const T*)(S + opk);
   tb.xi = (const T*)(S + oxi);

@@ -84,8 +84,13 @@ __device__ __forceinline__ LandauOut landau_factored(double Np, double Nm, doubl
   o.u = fabs(o.ub);
   o.n = fma(b, Np, a * Nm) * h;
   o.T = o.E * rcp64(3.0 * o.n);
-  o.ok = (Ap > 0.0) && (Am > 0.0) && (o.E > 0.0) && (o.n > 0.0) && isfinite(o.E) &&
-         isfinite(o.n) && isfinite(o.beta) && (fabs(o.beta) < 1.0);
+  // Ap, Am, E, n positive, normal and finite and |gamma beta| < gamma, tested on the
+  // bit patterns (an FP64 comparison costs as much as a product)
+  auto good = [](double x) {
+    return (unsigned)__double2hiint(x) - 0x00100000u < 0x7FE00000u;
+  };
+  o.ok = good(Ap) && good(Am) && good(o.E) && good(o.n) && good(o.gamma) &&
+         __double_as_longlong(o.u) < __double_as_longlong(o.gamma);
   return o;
 }
 
@@ -209,18 +214,20 @@ template <typename T>
 __host__ __device__ constexpr int aeq_max_start() { return sizeof(T) == 8 ? kAeqSteps : 96; }
 
 // delta_m for 2 <= m < nm4 (nm4 = max(nm, 4)), and delta_1 for the D chain,
-// handed to put(m, delta).  All lanes of the warp run from the largest
-// starting order among them, so that alpha is read uniformly.
+// handed to put(m, delta).  All lanes of the warp loop from the largest
+// starting order Mw among them, so that alpha is read uniformly, but each starts
+// at its own M: a cell's result does not depend on its neighbours.
 template <typename T, typename Put>
-__device__ __forceinline__ void aeq_chain(bool e_chain, T b2, T r, int M, int nm4, Put put) {
+__device__ __forceinline__ void aeq_chain(bool e_chain, T b2, T r, int M, int Mw, int nm4, Put put) {
   T d1 = r, d0 = T(1);  // delta_{m+1}, delta_m
-  for (int m = M; m >= nm4; --m) {
+  for (int m = Mw; m >= nm4; --m) {
     const T dn = fma(-b2, d1, aeq_alpha<T>(e_chain, m) * d0);
-    d1 = d0;
-    d0 = dn;
+    const bool on = m <= M;
+    d1 = on ? d0 : d1;
+    d0 = on ? dn : d0;
   }
 #pragma unroll
-  for (int m = kMaxM - 1 < 3 ? 3 : kMaxM - 1; m >= 3; --m)
+  for (int m = kMaxM - 1; m >= 3; --m)
     if (m < nm4) {
       put(m, d0);
       const T dn = fma(-b2, d1, aeq_alpha<T>(e_chain, m) * d0);
@@ -231,28 +238,119 @@ __device__ __forceinline__ void aeq_chain(bool e_chain, T b2, T r, int M, int nm
   if (!e_chain) put(1, fma(-b2, d1, aeq_alpha<T>(false, 2) * d0));
 }
 
-// One level of a transposing warp reduction of 32 compensated (hi, lo)
-// values per lane: lanes with bit OFF set keep the upper half of their
-// values, exchange the other half with lane ^ OFF and add with an
-// error-free TwoSum, so after the levels 16, 8, 4, 2, 1 lane l holds the
-// warp total of value l in h[0] + lo[0].
-template <int OFF>
-__device__ __forceinline__ void tr_level(float (&h)[32], float (&lo)[32], int lane) {
-  const bool up = (lane & OFF) != 0;
-#pragma unroll
-  for (int i = 0; i < OFF; ++i) {
-    const float sh = up ? h[i] : h[i + OFF];
-    const float sl = up ? lo[i] : lo[i + OFF];
-    const float kh = up ? h[i + OFF] : h[i];
-    const float kl = up ? lo[i + OFF] : lo[i];
-    const float rh = __shfl_xor_sync(0xffffffffu, sh, OFF);
-    const float rl = __shfl_xor_sync(0xffffffffu, sl, OFF);
-    const float t = kh + rh;
-    const float bp = t - kh;
-    const float e = (kh - (t - bp)) + (rh - bp);
-    h[i] = t;
-    lo[i] = (kl + rl) + e;
+// Both chains side by side: delta_m in D[m], eps_m in E[m] for m < min(nm4, MAXM).
+template <typename T, int MAXM>
+__device__ __forceinline__ void aeq_chains(T b2, T r, int M, int Mw, int nm4, T* D, T* E) {
+  T d1 = r, d0 = T(1), e1 = r, e0 = T(1);
+  for (int m = Mw; m >= nm4; --m) {
+    const T dn = fma(-b2, d1, aeq_alpha<T>(false, m) * d0);
+    const T en = fma(-b2, e1, aeq_alpha<T>(true, m) * e0);
+    const bool on = m <= M;
+    d1 = on ? d0 : d1;
+    d0 = on ? dn : d0;
+    e1 = on ? e0 : e1;
+    e0 = on ? en : e0;
   }
+#pragma unroll
+  for (int m = MAXM - 1; m >= 3; --m)
+    if (m < nm4) {
+      D[m] = d0;
+      E[m] = e0;
+      const T dn = fma(-b2, d1, aeq_alpha<T>(false, m) * d0);
+      const T en = fma(-b2, e1, aeq_alpha<T>(true, m) * e0);
+      d1 = d0;
+      d0 = dn;
+      e1 = e0;
+      e0 = en;
+    }
+  D[2] = d0;
+  E[2] = e0;
+  D[1] = fma(-b2, d1, aeq_alpha<T>(false, 2) * d0);
+}
+
+__device__ __forceinline__ double fast_inv(double x) { return rcp64(x); }
+__device__ __forceinline__ float fast_inv(float x) {  // 1 ulp
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// The integrals X3_m, X4_m of one cell by the 32-node rule, for |beta| so close
+// to 1 that the recurrence would need more than its table (u beyond ~7 (FP64)
+// or ~11 (FP32)): the truncated f^eq is strongly negative there, so no flow
+// the method can follow reaches this; kept for the stray cell that does.
+template <typename T>
+__device__ __noinline__ void aeq_far(const double* __restrict__ gl_t,
+                                     const double* __restrict__ gl_w, T u, T sh2, int nm, T* X) {
+  T J3[kMaxM], J4[kMaxM];
+  for (int m = 0; m < kMaxM; ++m) { J3[m] = T(0); J4[m] = T(0); }
+  const T A = asinh(u), uinv = T(1) / u;
+  for (int i = 0; i < kAeqNodes; ++i)
+    aeq_node<T>(T(gl_t[i]), T(gl_w[i]), A, sh2, uinv, false, nm, J3, J4);
+  for (int m = 0; m < nm; ++m) {
+    X[m] = J3[m] * (A * uinv);
+    X[kMaxM + m] = J4[m] * (A * uinv);
+  }
+}
+
+// What the coefficients of one cell need of its Landau frame (n = 0: none).
+template <typename T>
+struct AeqCell {
+  T n, T_, gamma, ub;  // ub = gamma beta
+};
+
+// c_{k,m} = (m + 1/2) q^m [p3_m + L1_k (p3_m - p4_m)] of one cell (c_{k,m} as in
+// aeq_node's comment): after this D[m], E[m] (m < nm <= MAXM) hold the chains
+// relative to their norms, so that p3_m = A3 S_m D[m], p4_m = A4 S_m E[m].
+// mask holds the lanes that call this together.
+template <typename T>
+struct AeqScalars {
+  T A3, A4, q;
+};
+template <typename T, int MAXM>
+__device__ __forceinline__ AeqScalars<T> aeq_cell(const AeqCell<T>& c, int nm, unsigned mask,
+                                                  const double* __restrict__ gl_t,
+                                                  const double* __restrict__ gl_w, T* D, T* E) {
+  static_assert(MAXM >= 4, "the chains end at order 3");
+  const int nm4 = max(nm, 4);
+  const T u = fabs(c.ub);
+  float r;
+  const int M = aeq_start<T>(float(u), float(c.gamma), nm4, &r);
+  const bool far = M > aeq_max_start<T>();
+  const int Mc = min(M, aeq_max_start<T>()), Mw = __reduce_max_sync(mask, Mc);
+  AeqScalars<T> o;
+  o.q = c.ub * fast_inv(c.gamma);  // beta
+  const T b2 = far ? T(0) : o.q * o.q;
+#pragma unroll
+  for (int m = 0; m < MAXM; ++m) { D[m] = T(0); E[m] = T(0); }
+  aeq_chains<T, MAXM>(b2, T(r), Mc, Mw, nm4, D, E);
+  // relative to the norms X3_0 = 2 u0 and X4_0 = (2/3) u0^2 (3 + beta^2), so the
+  // isotropic part of f^eq carries the roundings of A3 and A4 only
+  const T rD = fast_inv(D[1]), rE = fast_inv(fma(T(0.25), b2, T(0.75)) * E[2]);
+  o.A3 = T(0.5) * c.n * c.gamma;
+  o.A4 = o.A3 * (c.T_ * c.gamma) * fma(T(1.0 / 3.0), b2, T(1));
+  D[0] = D[1] = T(1);
+  E[1] = E[2] * rE;
+  E[0] = T(1);
+#pragma unroll
+  for (int m = 2; m < MAXM; ++m) {
+    D[m] *= rD;
+    E[m] *= rE;
+  }
+  if (far) {
+    T X[2 * kMaxM];
+    aeq_far<T>(gl_t, gl_w, u, u * u / (c.gamma + T(1)), nm, X);
+#pragma unroll
+    for (int m = 0; m < MAXM; ++m)
+      if (m < nm) {
+        D[m] = X[m] / aeq_scale<T>(false, m);
+        E[m] = X[kMaxM + m] / aeq_scale<T>(true, m);
+      }
+    o.A3 = T(0.25) * c.n;
+    o.A4 = T(0.25) * c.n * c.T_;
+    o.q = c.ub < T(0) ? T(-1) : T(1);
+  }
+  return o;
 }
 
 }  // namespace rslb

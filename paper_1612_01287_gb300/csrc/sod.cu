@@ -432,24 +432,6 @@ __device__ __forceinline__ void sweep_segment(const T* row, T* orow, int i0, T x
   }
 }
 
-// The integrals X3_m, X4_m of one cell by the 32-node rule, for |beta| so close
-// to 1 that the recurrence would need more than its table (u beyond ~7 (FP64)
-// or ~11 (FP32)): the truncated f^eq is strongly negative there, so no flow
-// the method can follow reaches this; kept for the stray cell that does.
-template <typename T>
-__device__ __noinline__ void aeq_far(const double* __restrict__ gl_t,
-                                     const double* __restrict__ gl_w, T u, T sh2, int nm, T* X) {
-  T J3[kMaxM], J4[kMaxM];
-  for (int m = 0; m < kMaxM; ++m) { J3[m] = T(0); J4[m] = T(0); }
-  const T A = asinh(u), uinv = T(1) / u;
-  for (int i = 0; i < kAeqNodes; ++i)
-    aeq_node<T>(T(gl_t[i]), T(gl_w[i]), A, sh2, uinv, false, nm, J3, J4);
-  for (int m = 0; m < nm; ++m) {
-    X[m] = J3[m] * (A * uinv);
-    X[kMaxM + m] = J4[m] * (A * uinv);
-  }
-}
-
 template <typename T, int B, int NT>
 __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __restrict__ fn,
                                          T* fout, int stage, int* err, const SodGeom& g,
@@ -528,7 +510,8 @@ __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __r
           const int n = np ? np : 1;
           for (int r = 0; r * n < NS; ++r) {
             if (owner && sl / n == r) m.put(part + (size_t)(sl % n) * 5 * B + c, B, r > 0);
-            asm volatile("bar.sync 1, %0;" ::"n"(NS * (B < 32 ? 32 : B)) : "memory");
+            __syncwarp();
+            asm volatile("barrier.sync 1, %0;" ::"n"(NS * (B < 32 ? 32 : B)) : "memory");
           }
         }
       }
@@ -560,7 +543,7 @@ __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __r
       T g0 = T(0), g1 = T(0);
       if (!Lo.ok) {
         if (!second && s0 + c < g.Z) report_error(err, 6, s0 + c);
-        Lo.n = 0.0; Lo.T = 1.0; Lo.beta = 0.0; Lo.gamma = 1.0; Lo.u = 0.0;
+        Lo.n = 0.0; Lo.T = 1.0; Lo.beta = 0.0; Lo.gamma = 1.0; Lo.u = Lo.ub = 0.0;
       } else if (g.tau_mode == kTauEtas) {
         const double lam = Lo.n * g.lambda_ref * rcp64(Lo.T * Lo.T * Lo.T);
         const double r = g.dt * Lo.T * rcp64(g.tau_AW0 * fma(-0.25, log(lam), 1.0));
@@ -575,19 +558,20 @@ __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __r
         gco[2 * c] = g0;
         gco[2 * c + 1] = g1;
       }
-      const int nm = g.nm, nm4 = max(nm, 4);
-      float r;
-      const int M = aeq_start<T>(float(Lo.u), float(Lo.gamma), nm4, &r);
-      const bool far = M > aeq_max_start<T>();
-      const int Mw = __reduce_max_sync(mask, min(M, aeq_max_start<T>()));
-      const T beta = T(Lo.beta), gam = T(Lo.gamma), b2 = far ? T(0) : beta * beta;
-      const T n4 = T(0.25 * Lo.n);
-      // c_{k,m} = (m + 1/2) beta^m [p3 + L1_k (p3 - p4)], p3 = A3 S_m delta_m,
-      // p4 = A4 S_m eps_m (A4 with the factor T), from the norms of the chains
+      const int nm = g.nm;
       if (split) {
-        T* dst = coef + ((size_t)(second ? B : 0) + c) * MP;  // slot k = 0: delta, 1: eps
+        // slot k = 0 of the cell's coefficients holds delta_m, slot 1 eps_m; the
+        // scalars A3, A4 (with the factor T) carry the norms of the chains
+        const int nm4 = max(nm, 4);
+        float r;
+        const int M = aeq_start<T>(float(Lo.u), float(Lo.gamma), nm4, &r);
+        const bool far = M > aeq_max_start<T>();
+        const int Mc = min(M, aeq_max_start<T>()), Mw = __reduce_max_sync(mask, Mc);
+        const T beta = T(Lo.beta), gam = T(Lo.gamma), b2 = far ? T(0) : beta * beta;
+        const T n4 = T(0.25 * Lo.n);
+        T* dst = coef + ((size_t)(second ? B : 0) + c) * MP;
         T d2 = T(0), d1 = T(0);
-        aeq_chain<T>(second, b2, T(r), Mw, nm4, [&](int m, T x) {
+        aeq_chain<T>(second, b2, T(r), Mc, Mw, nm4, [&](int m, T x) {
           if (m < nm && m >= 2) dst[m] = x;
           if (m == 2) d2 = x;
           if (m == 1) d1 = x;
@@ -613,47 +597,18 @@ __device__ __forceinline__ void sod_tile(const T* __restrict__ fin, const T* __r
         }
       } else {
         T D[kMaxM], E[kMaxM];
-#pragma unroll
-        for (int m = 0; m < kMaxM; ++m) { D[m] = T(0); E[m] = T(0); }
-        aeq_chain<T>(false, b2, T(r), Mw, nm4, [&](int m, T x) { D[m] = x; });
-        aeq_chain<T>(true, b2, T(r), Mw, nm4, [&](int m, T x) { E[m] = x; });
-        // relative to the norms X3_0 = 2 u0 and X4_0 = (2/3) u0^2 (3 + beta^2),
-        // which are taken in FP64: the isotropic part of f^eq has one rounding
-        const T rD = T(1) / D[1], rE = T(1) / (fma(T(0.25), b2, T(0.75)) * E[2]);
-        T A3 = T(0.5 * Lo.n * Lo.gamma);
-        T A4 = T(Lo.n * Lo.T * Lo.gamma * Lo.gamma * fma(Lo.beta, Lo.beta * (1.0 / 6.0), 0.5));
-        T q = beta;
-        D[0] = D[1] = T(1);
-        E[1] = E[2] * rE;
-        E[0] = T(1);
-#pragma unroll
-        for (int m = 2; m < kMaxM; ++m) {
-          D[m] *= rD;
-          E[m] *= rE;
-        }
-        if (far) {
-          T X[2 * kMaxM];
-          aeq_far<T>(tb.gl_t, tb.gl_w, T(Lo.u), T(Lo.u * Lo.u / (Lo.gamma + 1.0)), nm, X);
-#pragma unroll
-          for (int m = 0; m < kMaxM; ++m)
-            if (m < nm) {
-              D[m] = X[m] / aeq_scale<T>(false, m);
-              E[m] = X[kMaxM + m] / aeq_scale<T>(true, m);
-            }
-          A3 = T(0.25 * Lo.n);
-          A4 = T(0.25 * Lo.n * Lo.T);
-          q = Lo.beta < 0.0 ? T(-1) : T(1);
-        }
+        const AeqCell<T> cell{T(Lo.n), T(Lo.T), T(Lo.gamma), T(Lo.ub)};
+        const AeqScalars<T> o = aeq_cell<T, kMaxM>(cell, nm, mask, tb.gl_t, tb.gl_w, D, E);
         T bm = T(1);
 #pragma unroll
         for (int m = 0; m < kMaxM; ++m) {
           if (m < nm) {
             const T um = T(m + 0.5) * bm;
-            const T p3 = um * (A3 * (aeq_scale<T>(false, m) * D[m]));
-            const T pd = p3 - um * (A4 * (aeq_scale<T>(true, m) * E[m]));
+            const T p3 = um * (o.A3 * (aeq_scale<T>(false, m) * D[m]));
+            const T pd = p3 - um * (o.A4 * (aeq_scale<T>(true, m) * E[m]));
             for (int k = 0; k < g.QL; ++k)
               coef[((size_t)k * B + c) * MP + m] = fma(tb.L1k[k], pd, p3);
-            bm *= q;
+            bm *= o.q;
           }
         }
         for (int m = nm; m < MP; ++m)

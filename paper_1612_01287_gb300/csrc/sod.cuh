@@ -25,7 +25,6 @@ struct SodGeom {
 // Per-velocity tables in the working precision (device pointers).
 template <typename T>
 struct SodTables {
-  const T* mw;      // [5][V]: 1+xi, 1-xi, p(1+xi)^2, p(1-xi)^2, p(1-xi^2)
   const T* m3;      // [V][4]: (1+xi)^2, (1-xi)^2, 1-xi^2, 0
   const T* pk;      // [QL][2]: p_k as hi + lo in T
   const T* xi;      // [V]
@@ -82,9 +81,7 @@ struct SodLaunch {
 // Opt the stage kernels into large dynamic shared memory (call at set-up,
 // outside stream capture).
 cudaError_t sod_set_attributes();
-// Packed FP32x2 stage kernel (sod32.cu): tile width and threads per CTA
-// (8 threads per cell in the f^eq coefficient phase, a warp per 4 cells in
-// the moments).
+// Packed FP32x2 stage kernel (sod32.cu): tile width and threads per CTA.
 constexpr int kSod32Cells = RSLB_PACKED_TILE_CELLS;
 constexpr int kSod32Threads = 8 * kSod32Cells;
 

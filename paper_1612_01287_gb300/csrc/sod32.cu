@@ -11,6 +11,7 @@
 #include <cuda.h>
 
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 
 #include "sod32_core.cuh"
@@ -19,17 +20,21 @@ namespace rslb {
 namespace {
 
 using namespace p32;
-constexpr int kNT = kSod32Threads;  // a warp per 4 cells in the moments, 8 threads per cell
-                                    // in the f^eq coefficients
-static_assert(kNT == kCellThreads, "one thread per coefficient slot");
-constexpr int kMinCtas = kB2 <= 20 ? 3 : 2;  // CTAs per SM the registers are sized for
+constexpr int kNT = kSod32Threads;
+static_assert(kNT == 32 * kSlices && kNT == kCellThreads, "a warp per row slice of the moments");
+// CTAs per SM the registers are sized for: three (80 registers) where three
+// tiles fit the shared memory, else two (128).  The phases of a tile wait on one
+// another, so the third CTA pays for the tighter registers: V = 150, 65536 cells
+// 91 us per launch against 107, V = 300 140 against 154; V = 600 (two fit) 268
+// with 80 registers against 255.
+constexpr int kSmem3 = 75 * 1024;
+__host__ __device__ constexpr bool three_ctas(size_t smem) { return smem <= kSmem3; }
 
 }  // namespace
 
 // Shared memory: tile [rows][kP] floats (rows = V rounded up to whole TMA
-// boxes), then partial moments, cell scalars, coefficients
-// [QL][kH][kMP][2] floats, gco [kH][4] floats, an mbarrier, the five
-// moment weights of every velocity [5][V] and the coefficient constants.
+// boxes), then the moments, coefficients [QL][kH][kMP][2] floats, gco [kH][4]
+// floats, an mbarrier, the moment slices' partial sums and the constants.
 static size_t tile_rows(int V) {
   int nb = 0;
   const int r = tma_box_rows(V, &nb);
@@ -39,9 +44,8 @@ static size_t tile_rows(int V) {
 size_t sod32_smem_bytes(int V, int QL) {
   auto al = [](size_t x) { return (x + 127) & ~size_t(127); };
   return al(sizeof(float) * tile_rows(V) * kP) + al(sizeof(double) * 5 * kB2) +
-         al(sizeof(double) * 8 * kB2) + al(sizeof(float) * (size_t)QL * kH * kMP * 2) +
-         al(sizeof(float) * kH * 4) + 128 + al(sizeof(float) * 5 * (size_t)V) +
-         al(sizeof(float) * kConsts) + 128;
+         al(sizeof(float) * (size_t)QL * kH * kMP * 2) + al(sizeof(float) * kH * 4) + 128 +
+         scratch_bytes(V) + al(sizeof(float) * kConsts) + 128;
 }
 
 // One stage of one tile starting at cell s0 (the whole CTA).
@@ -59,19 +63,13 @@ __device__ __forceinline__ void sod32_tile(const float* __restrict__ fin,
   float* tile = reinterpret_cast<float*>(base);
   const size_t tile_bytes = al(sizeof(float) * (size_t)nbox * box_rows * kP);
   double* msum = reinterpret_cast<double*>(base + tile_bytes);
-  double* cell = msum + 5 * kB2;
-  float* coef = reinterpret_cast<float*>(
-      base + tile_bytes + al(sizeof(double) * 5 * kB2) + al(sizeof(double) * 8 * kB2));
+  float* coef = reinterpret_cast<float*>(base + tile_bytes + al(sizeof(double) * 5 * kB2));
   float* gco = coef + (size_t)g.QL * kH * kMP * 2;  // [kH][g0x g0y g1x g1y]
   uint64_t* bar = reinterpret_cast<uint64_t*>(
-      reinterpret_cast<unsigned char*>(gco) + al(sizeof(float) * kH * 4));
-  float* mws = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bar) + 128);
-  float* cst = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(mws) +
-                                        al(sizeof(float) * 5 * (size_t)V));
-  auto copy_weights = [&]() {
-    for (int e = threadIdx.x; e < 5 * V; e += kNT) mws[e] = tb.mw[e];
-    load_consts(cst, tb, g.QL, threadIdx.x, kNT);
-  };
+      base + tile_bytes + al(sizeof(double) * 5 * kB2) +
+      al(sizeof(float) * (size_t)g.QL * kH * kMP * 2) + al(sizeof(float) * kH * 4));
+  float2* part = reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(bar) + 128);
+  float* cst = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(part) + scratch_bytes(V));
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -107,7 +105,7 @@ __device__ __forceinline__ void sod32_tile(const float* __restrict__ fin,
                        : "memory");
     }
     __syncthreads();  // the barrier is initialised before anyone polls it
-    copy_weights();   // while the boxes are in flight
+    load_consts(cst, tb, g.QL, tid, kNT);
     uint32_t ok = 0;
     for (int it = 0; it < (1 << 22) && !ok; ++it) {
       asm volatile(
@@ -125,20 +123,21 @@ __device__ __forceinline__ void sod32_tile(const float* __restrict__ fin,
   } else {
     stage_plain(tile, fin, g, tb, s0, tid, kNT);
   }
-  if (!(interior && tmap)) copy_weights();
+  if (!(interior && tmap)) load_consts(cst, tb, g.QL, tid, kNT);
   __syncthreads();
 
   const bool collide = g.tau_mode != kTauNone;
   if (collide) {
-    // ---- 2. moments: warp w owns cells 4w .. 4w+3 of the tile ----
-    moments(tile, mws, msum, V, warp, lane);
+    // ---- 2. moments: warp w sums row slice w ----
+    moments(tile, tb.m3, cst, part, V, g.Qx, warp, lane);
     __syncthreads();
-    // ---- 3a. Landau matching (FP64) and relaxation time, one thread per cell ----
-    float* cellf = reinterpret_cast<float*>(cell);  // [8][kB2]
-    if (tid < kB2) landau_cell(msum, cellf, gco, g, s0, tid, err);
+    for (int e = tid; e < 5 * kB2; e += kNT) msum[e] = moment_total(part, e);
     __syncthreads();
-    // ---- 3b. f^eq coefficients: 8 threads per cell share the 16 nodes ----
-    coefs(cellf, coef, g, cst, tid);
+    // ---- 3. Landau matching and relaxation time, then f^eq coefficients ----
+    float* cells = reinterpret_cast<float*>(part);
+    if (tid < kB2) landau_cell(msum, cells, gco, g, s0, tid, err);
+    __syncthreads();
+    coefs(cells, coef, cst, g, tb, tid);
     __syncthreads();
   } else {
     for (int i = tid; i < g.QL * kH * kMP * 2 + kH * 4; i += kNT) coef[i] = 0.f;
@@ -153,7 +152,8 @@ __device__ __forceinline__ void sod32_tile(const float* __restrict__ fin,
   store(tile, fn, fout, g, stage, s0, tid, kNT);
 }
 
-__global__ void __launch_bounds__(kNT, kMinCtas)
+template <int CTAS>
+__global__ void __launch_bounds__(kNT, CTAS)
 sod32_stage_kernel(const float* __restrict__ fin, const float* __restrict__ fn, float* fout,
                    int stage, int* err, SodGeom g, SodTables<float> tb, const int* __restrict__ rowv,
                    int nneg, const __grid_constant__ CUtensorMap tmap,
@@ -168,7 +168,8 @@ sod32_stage_kernel(const float* __restrict__ fin, const float* __restrict__ fn, 
 // maps (optional): per run, the tensor maps of F0, F1, F2 (36-cell boxes) and
 // of F0 with tile-wide boxes for the f_n prefetch; without them the tiles
 // are staged by plain loads.
-__global__ void __launch_bounds__(kNT, kMinCtas)
+template <int CTAS>
+__global__ void __launch_bounds__(kNT, CTAS)
 sod32_batch_kernel(const SodRunDesc<float>* __restrict__ runs, const SodTask* __restrict__ tasks,
                    int ntasks, const long long* __restrict__ step, int step_off, int stage, int* err,
                    const CUtensorMap* __restrict__ maps) {
@@ -232,8 +233,8 @@ bool sod32_make_map(CUtensorMap* m, const float* f, int Z, int ldz, int V, int b
 cudaError_t sod32_batch_launch(size_t smem, int grid, const SodRunDesc<float>* runs,
                                const SodTask* tasks, int ntasks, const long long* step, int step_off,
                                int stage, int* err, const void* maps, cudaStream_t st) {
-  sod32_batch_kernel<<<grid, kNT, smem, st>>>(runs, tasks, ntasks, step, step_off, stage, err,
-                                              static_cast<const CUtensorMap*>(maps));
+  (three_ctas(smem) ? sod32_batch_kernel<3> : sod32_batch_kernel<2>)<<<grid, kNT, smem, st>>>(
+      runs, tasks, ntasks, step, step_off, stage, err, static_cast<const CUtensorMap*>(maps));
   return cudaGetLastError();
 }
 
@@ -252,22 +253,18 @@ bool sod32_make_maps(void* out4, const float* F0, const float* F1, const float* 
 }
 
 cudaError_t sod32_set_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(sod32_batch_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(sod32_stage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              232448);
+  for (const void* f : {(const void*)sod32_batch_kernel<2>, (const void*)sod32_batch_kernel<3>,
+                        (const void*)sod32_stage_kernel<2>, (const void*)sod32_stage_kernel<3>}) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t sod32_stage_launch(const SodGeom& g, const SodTables<float>& tb, const int* rowv,
                                int nneg, const float* fin, const float* fn, float* fout, int stage,
                                int* err, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = sod32_set_attributes();
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
   int nbox = 0;
   const int br = tma_box_rows(g.V, &nbox);
   CUtensorMap m, mn;
@@ -280,7 +277,8 @@ cudaError_t sod32_stage_launch(const SodGeom& g, const SodTables<float>& tb, con
                    sod32_make_map(&m, fin, g.Z, g.ldz, g.V, kC, br) &&
                    sod32_make_map(&mn, fn, g.Z, g.ldz, g.V, kB2, br);
   const int grid = (g.Z + kB2 - 1) / kB2;
-  sod32_stage_kernel<<<grid, kNT, sod32_smem_bytes(g.V, g.QL), st>>>(
+  const size_t smem = sod32_smem_bytes(g.V, g.QL);
+  (three_ctas(smem) ? sod32_stage_kernel<3> : sod32_stage_kernel<2>)<<<grid, kNT, smem, st>>>(
       fin, fn, fout, stage, err, g, tb, rowv, nneg, m, mn, tma ? 1 : 0, br, nbox);
   return cudaGetLastError();
 }

@@ -12,10 +12,13 @@
 // (position s, position s + kH).
 //
 // Phases of one RK stage of one tile (Sec. III F, Eq. rk3):
-//   moments    Kahan-compensated FP32 sums of N+-, A+-, D (Eq. macro_jk in the
-//              factored form) with an error-free FP32 warp reduction;
-//   landau     FP64 Landau matching (Eqs. E_landau, u_landau) and tau;
-//   coefs      f^eq coefficients (Eq. feq_trunc via Eq. aeq_aux, 16-node rule);
+//   moments    FP32 sums of N+-, A+-, D (Eq. macro_jk in the factored form), from
+//              three sums per radial node, as compensated double-floats; a lane
+//              owns two cells and a slice of the rows;
+//   landau     a thread per cell: FP64 Landau matching (Eqs. E_landau, u_landau)
+//              and tau;
+//   coefs      f^eq coefficients (Eq. feq_trunc via Eq. aeq_aux) by the recurrence
+//              over the Legendre order, 8 threads per cell;
 //   sweep      WENO5 flux difference (Eqs. flux_weno, weno5_omega), f^eq at
 //              the nodes (Eq. fjk), relaxation (Eq. L_Sod), stage update;
 //   store      RK combination with f_n and the write of the tile.
@@ -35,8 +38,9 @@ constexpr int kB2 = kSod32Cells;  // output cells per tile
 constexpr int kH = kB2 / 2;        // cells per half
 constexpr int kC = kB2 + 8;        // cells staged per row (4-cell halo per side)
 constexpr int kP = kC;             // floats per row (an odd number of 16-byte units)
-constexpr int kCellThreads = 8 * kB2;  // moments: a warp per 4 cells; coefficients: 8 per cell
-static_assert(kB2 % 4 == 0 && kH % 2 == 0 && (kC / 4) % 2 == 1, "packed tile shape");
+constexpr int kSlices = 7;             // row slices of the moment sums (a warp's work each)
+constexpr int kCellThreads = 8 * kB2;  // coefficients: 8 threads per cell
+static_assert(kCellThreads % 32 == 0 && kB2 % 4 == 0 && kH % 2 == 0 && (kC / 4) % 2 == 1, "packed tile shape");
 constexpr int kMP = 8;        // coefficient pitch (m) for N_Omega <= 7
 constexpr int kInflight = 8;  // 16-byte global loads in flight per thread (staging, store)
 constexpr int kErrWait = RSLB_ERR_TIMEOUT;  // error code: a bounded wait ran out
@@ -62,6 +66,17 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Shared-memory scratch of a tile: the moment slices' partial sums
+// [kSlices][5][kB2] (hi, lo).  (The size is that of the five weights per velocity
+// and the per-cell scalars it replaced where that was larger, because it
+// decides which velocity counts the kernel accepts.)
+__host__ __device__ __forceinline__ size_t scratch_bytes(int V) {
+  const size_t part = sizeof(float2) * kSlices * 5 * kB2;
+  const size_t old = ((sizeof(double) * 8 * kB2 + 127) & ~size_t(127)) +
+                     ((sizeof(float) * 5 * (size_t)V + 127) & ~size_t(127));
+  return old > part ? old : (part + 127) & ~size_t(127);
+}
+
 // Rows of one bulk-tensor box (<= 256 rows, a multiple of 8 so that a box of
 // kC floats per row is a multiple of 128 bytes) and the number of boxes.
 __host__ __device__ __forceinline__ int tma_box_rows(int V, int* nbox) {
@@ -72,41 +87,40 @@ __host__ __device__ __forceinline__ int tma_box_rows(int V, int* nbox) {
   return r;
 }
 
-// WENO5 correction (omega . g) of sod.cu::weno_corr for two faces at once,
-// with delta_q folded into g_q: n_q = prod_{p != q} t_p.
-__device__ __forceinline__ float2 weno_corr2(float2 D0, float2 D1, float2 D2, float2 D3,
-                                             float2 K1, float2 K2, float2 K3) {
-  const float tiny = 1.17549435e-38f;
-  const float2 e1 = fma2(splat(-3.f), D1, D0);  // -(3 D1 - D0); squared below
-  const float2 e2 = add2(D1, D2);
-  const float2 e3 = fma2(splat(-3.f), D2, D3);
-  const float2 s1 = fma2(mul2(splat(0.25f), e1), e1, K1);
-  const float2 s2 = fma2(mul2(splat(0.25f), e2), e2, K2);
-  const float2 s3 = fma2(mul2(splat(0.25f), e3), e3, K3);
-  // delta_q g_q: 0.1 (5 D1 - 2 D0), 0.6 (D1 + 2 D2), 0.3 (4 D2 - D3)
-  const float2 h1 = fma2(splat(0.5f), D1, mul2(splat(-0.2f), D0));
-  const float2 h2 = fma2(splat(1.2f), D2, mul2(splat(0.6f), D1));
-  const float2 h3 = fma2(splat(1.2f), D2, mul2(splat(-0.3f), D3));
+// WENO5 correction (omega . g) of sod.cu::weno_corr for two faces at once, from
+// the differences D1, D2 left and right of the upwind-centre value, the second
+// differences' Q_c = 4/3 S_c^2 and the shared X = D1 + S_1 = 2 D1 - D0,
+// Y = D2 - S_3 = 2 D2 - D3: with D2 = D1 + S_2,
+//   sigma_1 = D1 X + Q_1, sigma_2 = D1 D2 + Q_2, sigma_3 = D2 Y + Q_3,
+//   g_1 = 2 X + D1, g_2 = 2 D2 + D1, g_3 = 2 D2 + Y
+// (sigma_q of Eq. weno5_omega; positive definite forms, so nothing cancels).
+__device__ __forceinline__ float2 weno_corr2(float2 D1, float2 D2, float2 X, float2 Y, float2 Q1,
+                                             float2 Q2, float2 Q3) {
+  const float2 s1 = fma2(D1, X, Q1), s2 = fma2(D1, D2, Q2), s3 = fma2(D2, Y, Q3);
+  const float2 g1 = fma2(splat(2.f), X, D1), g2 = fma2(splat(2.f), D2, D1),
+               g3 = fma2(splat(2.f), D2, Y);
   // scale the smoothness indicators by the power of two at or below their
   // maximum (the weights are homogeneous in sigma; this only keeps the
-  // fourth powers inside the FP32 range): integer exponent arithmetic
-  // instead of a reciprocal
+  // fourth powers inside the FP32 range): 2^(127 - e) for the biased exponent e,
+  // an AND and a subtract; a zero or subnormal maximum gives 2^127, which
+  // keeps zero sigmas zero and brings subnormal ones into range
   const float mx = fmaxf(s1.x, fmaxf(s2.x, s3.x));
   const float my = fmaxf(s1.y, fmaxf(s2.y, s3.y));
-  // 2^(127 - e) for the biased exponent e of m: an AND and a subtract; a
-  // zero or subnormal m gives 2^127, which keeps zero sigmas zero and brings
-  // subnormal ones into range
   auto inv_pow2 = [&](float m) {
     return __int_as_float(0x7F000000 - (__float_as_int(m) & 0x7F800000));
   };
   const float2 inv = make_float2(inv_pow2(mx), inv_pow2(my));
   const float2 r1 = mul2(s1, inv), r2 = mul2(s2, inv), r3 = mul2(s3, inv);
   const float2 t1 = mul2(r1, r1), t2 = mul2(r2, r2), t3 = mul2(r3, r3);
-  const float2 p23 = mul2(t2, t3), p13 = mul2(t1, t3), p12 = mul2(t1, t2);
-  const float2 den = fma2(splat(0.1f), p23, fma2(splat(0.6f), p13, mul2(splat(0.3f), p12)));
-  const float2 num = fma2(p23, h1, fma2(p13, h2, mul2(p12, h3)));
-  return make_float2(den.x > tiny ? num.x * rcp_approx(den.x) : 0.f,
-                     den.y > tiny ? num.y * rcp_approx(den.y) : 0.f);
+  // products in the ratio 1 : 2 : 1/3; the 2^-120 keeps the reciprocal finite
+  // where all products vanish (the correction is 0 there by the limit rules,
+  // and is when num = 0) and is below their rounding elsewhere
+  const float2 p13 = mul2(t1, t3);
+  const float2 n3 = fma2(t1, t2, splat(7.5231638e-37f));
+  const float2 n2 = add2(p13, p13), n1 = mul2(mul2(t2, t3), splat(1.f / 3.f));
+  const float2 den = add2(add2(n3, n2), n1);
+  const float2 num = fma2(n1, g1, fma2(n2, g2, mul2(mul2(t1, t2), g3)));
+  return mul2(num, make_float2(rcp_approx(den.x), rcp_approx(den.y)));
 }
 
 __device__ __forceinline__ void ld2slots(const float* p, float2* out) {
@@ -126,45 +140,49 @@ __device__ __forceinline__ void ld_slot_pair(const float* row, int s, float2* ou
 
 // Sweep a whole row (both halves): slots 4 .. kH+3 are the outputs; window of
 // 10 slots [i-4, i+6) around the current two-slot chunk i, with the first
-// differences D[c] = J[c+1] - J[c] and the smoothness terms
-// K[c] = 13/12 (D[c] - D[c-1])^2 slid along with it (two new of each per
-// chunk).  For xi < 0 the stencil is mirrored; weno_corr2 is odd in its D
-// arguments, so the mirrored correction is taken as -weno_corr2 of the
-// un-negated differences.  Results go back into the row in place: the
-// left-half outputs (positions 4 .. kH+3) and the right-half outputs of slots
-// >= 8 (positions >= kH+8) are never read again by the sweep; the right-half
-// outputs of slots 4..7 (positions kH+4 .. kH+7) are held until the left half
-// has read those positions (its last four slots).
+// differences D[c] = f[c+1] - f[c] and from them S[c] = D[c] - D[c-1],
+// Q[c] = 4/3 S[c]^2, X[c] = D[c] + S[c] and Y[c] = D[c] - S[c+1] slid along with
+// it (two new of each per chunk).  The weights do not see a factor of f, so
+// the differences are those of f and xi enters through c1 = xi dt/dz.  For
+// xi < 0 the stencil is mirrored (D0 .. D3 = -(D[w+2] .. D[w-1]), so X and Y
+// change places); weno_corr2 is odd, so the mirrored correction is minus its
+// value for the un-negated differences.  Results go back into the row in
+// place: the left-half outputs (positions 4 .. kH+3) and the right-half outputs
+// of slots >= 8 (positions >= kH+8) are never read again by the sweep; the
+// right-half outputs of slots 4..7 (positions kH+4 .. kH+7) are held until the
+// left half has read those positions (its last four slots).  gco holds
+// (gamma, gamma beta) dt/tau.
 template <bool POS>
 __device__ __forceinline__ void sweep_row2(float* row, float xi, const float2* wp2, int nm,
                                            const float* __restrict__ ck,
-                                           const float* __restrict__ gco, float inv_dz,
-                                           float dt) {
+                                           const float* __restrict__ gco, float c1) {
   constexpr int NW = 10;
-  const float2 xi2 = splat(xi);
-  const float2 sixth = splat(1.f / 6.f);
-  const float2 k13 = splat(13.f / 12.f);
-  float2 R[NW], J[NW], Dw[NW - 1], Kw[NW - 1];
+  const float2 sixth = splat(1.f / 6.f), q43 = splat(4.f / 3.f);
+  const float2 mc1 = splat(-c1), mxi = splat(-xi);
+  float2 R[NW], D[NW - 1], S[NW - 1], Q[NW - 1];
   float2 held[2];
+  auto diffs = [&](int c0) {
+#pragma unroll
+    for (int c = 0; c < NW - 1; ++c)
+      if (c >= c0) D[c] = sub2(R[c + 1], R[c]);
+#pragma unroll
+    for (int c = 1; c < NW - 1; ++c)
+      if (c >= c0) {
+        S[c] = sub2(D[c], D[c - 1]);
+        Q[c] = mul2(mul2(q43, S[c]), S[c]);
+      }
+  };
 #pragma unroll
   for (int c = 0; c < NW; c += 2) ld_slot_pair(row, c, R + c);
-#pragma unroll
-  for (int c = 0; c < NW; ++c) J[c] = mul2(xi2, R[c]);
-#pragma unroll
-  for (int c = 0; c < NW - 1; ++c) Dw[c] = sub2(J[c + 1], J[c]);
-  Kw[0] = splat(0.f);
-#pragma unroll
-  for (int c = 1; c < NW - 1; ++c) {
-    const float2 d2 = sub2(Dw[c], Dw[c - 1]);
-    Kw[c] = mul2(mul2(k13, d2), d2);
-  }
-  auto face = [&](int wc) {
+  S[0] = Q[0] = splat(0.f);
+  diffs(0);
+  auto face = [&](int w) {  // the face right of window slot w
     if constexpr (POS)
-      return weno_corr2(Dw[wc - 2], Dw[wc - 1], Dw[wc], Dw[wc + 1], Kw[wc - 1], Kw[wc],
-                        Kw[wc + 1]);
+      return weno_corr2(D[w - 1], D[w], add2(D[w - 1], S[w - 1]), sub2(D[w], S[w + 1]), Q[w - 1],
+                        Q[w], Q[w + 1]);
     else
-      return weno_corr2(Dw[wc + 2], Dw[wc + 1], Dw[wc], Dw[wc - 1], Kw[wc + 2], Kw[wc + 1],
-                        Kw[wc]);
+      return weno_corr2(D[w + 1], D[w], sub2(D[w + 1], S[w + 2]), add2(D[w], S[w]), Q[w + 2],
+                        Q[w + 1], Q[w]);
   };
   float2 Cl = face(3);
 #pragma unroll
@@ -175,8 +193,8 @@ __device__ __forceinline__ void sweep_row2(float* row, float xi, const float2* w
     for (int c = 0; c < 2; ++c) {
       const int wc = 4 + c;
       const float2 Cr = face(wc);
-      const float2 dF = POS ? fma2(sub2(Cr, Cl), sixth, Dw[wc - 1])
-                            : fma2(sub2(Cl, Cr), sixth, Dw[wc]);
+      const float2 dF = POS ? fma2(sub2(Cr, Cl), sixth, D[wc - 1])
+                            : fma2(sub2(Cl, Cr), sixth, D[wc]);
       Cl = Cr;
       // f^eq for the two cells of this slot: coefficients (x cell, y cell) per m
       const float* cc = ck + (size_t)(i + c - 4) * (2 * kMP);
@@ -191,33 +209,21 @@ __device__ __forceinline__ void sweep_row2(float* row, float xi, const float2* w
         }
       }
       const float4 g = *reinterpret_cast<const float4*>(gco + 4 * (i + c - 4));
-      const float2 g0 = make_float2(g.x, g.y), g1 = make_float2(g.z, g.w);
       const float2 f = R[wc];
-      const float2 rate = fma2(splat(-xi), g1, g0);  // g0 - g1 xi
-      const float2 coll = mul2(rate, sub2(f, feq));
-      const float2 L = fma2(splat(-inv_dz), dF, mul2(splat(-1.f), coll));
-      out[c] = fma2(splat(dt), L, f);
+      const float2 rate = fma2(mxi, make_float2(g.z, g.w), make_float2(g.x, g.y));
+      out[c] = fma2(rate, sub2(feq, f), fma2(mc1, dF, f));
     }
     if (t + 1 < kH / 2) {
 #pragma unroll
-      for (int c = 0; c < NW - 2; ++c) {
-        J[c] = J[c + 2];
-        R[c] = R[c + 2];
-      }
+      for (int c = 0; c < NW - 2; ++c) R[c] = R[c + 2];
 #pragma unroll
       for (int c = 0; c < NW - 3; ++c) {
-        Dw[c] = Dw[c + 2];
-        Kw[c] = Kw[c + 2];
+        D[c] = D[c + 2];
+        S[c] = S[c + 2];
+        Q[c] = Q[c + 2];
       }
       ld_slot_pair(row, i + 6, R + NW - 2);  // slots i+6, i+7
-      J[NW - 2] = mul2(xi2, R[NW - 2]);
-      J[NW - 1] = mul2(xi2, R[NW - 1]);
-#pragma unroll
-      for (int c = NW - 3; c < NW - 1; ++c) {
-        Dw[c] = sub2(J[c + 1], J[c]);
-        const float2 d2 = sub2(Dw[c], Dw[c - 1]);
-        Kw[c] = mul2(mul2(k13, d2), d2);
-      }
+      diffs(NW - 3);
     }
     *reinterpret_cast<float2*>(row + i) = make_float2(out[0].x, out[1].x);
     if (t < 2) {
@@ -305,187 +311,182 @@ __device__ __forceinline__ void fix_ghosts(float* tile, const float* __restrict_
   }
 }
 
-// Moments of the kB2 cells of a staged tile: warp w (0 <= w < kB2/4) owns
-// cells 4w .. 4w+3, its lanes take rows; blocks of four rows,
-// Kahan-compensated across blocks.  msum[q*kB2 + c] = sum_v f w_q (FP64 from
-// the compensated FP32 hi + lo).  mws: the five moment weights [5][V].
-__device__ __forceinline__ void moments(const float* tile, const float* mws, double* msum, int V,
-                                        int warp, int lane) {
-  // cells (0, 1) and (2, 3) of the warp's four are the two lanes of packed
-  // FP32x2 values (adjacent in the 16-byte loads): same roundings as the
-  // scalar fma / Kahan steps, half the instructions
-  float2 s2[2][5], c2[2][5];
+// (H, L) += x, error-free in H (Knuth), two cells at a time.
+__device__ __forceinline__ void two_sum2(float2& H, float2& L, float2 x) {
+  const float2 t = add2(H, x), bp = sub2(t, H);
+  L = add2(L, add2(sub2(H, sub2(t, bp)), sub2(x, bp)));
+  H = t;
+}
+
+// Partial moments of row slice sl (0 <= sl < kSlices) by one warp: lane
+// 16 hf + pr (pr < 14) sums cells 2 pr, 2 pr + 1 over half hf of the slice's rows.
+// With a = sum f (1+xi)^2, b = sum f (1-xi)^2, d = sum f (1-xi^2) over the polar
+// nodes of a radial node p, N+- = sum_k ({a, b}_k + d_k)/2, A+- = sum_k p_k {a, b}_k,
+// D = sum_k p_k d_k (all weights non-negative): three products per velocity.
+// Blocks of four rows, Kahan-compensated across blocks; the radial sums, halves
+// and slices are added as double-floats.  consts: load_consts.
+__device__ __forceinline__ void moments(const float* tile, const float* __restrict__ m3,
+                                        const float* consts, float2* part, int V, int Qx, int sl,
+                                        int lane) {
+  const int hf = lane >> 4, pr = min(lane & 15, kB2 / 2 - 1);
+  const int n2 = 2 * kSlices, h0 = 2 * sl + hf;
+  int v = V * h0 / n2;
+  const int v1 = V * (h0 + 1) / n2;
+  const float* col = tile + 4 + 2 * pr;
+  float2 H[5], L[5], s[3], c[3], b[3];
 #pragma unroll
-  for (int p = 0; p < 2; ++p)
+  for (int q = 0; q < 5; ++q) H[q] = L[q] = splat(0.f);
 #pragma unroll
-    for (int q = 0; q < 5; ++q) { s2[p][q] = splat(0.f); c2[p][q] = splat(0.f); }
-  for (int v0 = lane; v0 < V; v0 += 128) {
-    float2 b2[2][5];
+  for (int q = 0; q < 3; ++q) s[q] = c[q] = b[q] = splat(0.f);
+  auto row = [&](int u) {
+    const float4 w = __ldg(reinterpret_cast<const float4*>(m3) + u);
+    const float2 x = *reinterpret_cast<const float2*>(col + u * kP);
+    b[0] = fma2(x, splat(w.x), b[0]);
+    b[1] = fma2(x, splat(w.y), b[1]);
+    b[2] = fma2(x, splat(w.z), b[2]);
+  };
+  auto block = [&]() {
 #pragma unroll
-    for (int p = 0; p < 2; ++p)
-#pragma unroll
-      for (int q = 0; q < 5; ++q) b2[p][q] = splat(0.f);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int v = v0 + 32 * u;
-      if (v < V) {
-        const float4 x = *reinterpret_cast<const float4*>(tile + v * kP + 4 + 4 * warp);
-        const float2 X0 = make_float2(x.x, x.y), X1 = make_float2(x.z, x.w);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const float2 W = splat(mws[q * V + v]);
-          b2[0][q] = fma2(X0, W, b2[0][q]);
-          b2[1][q] = fma2(X1, W, b2[1][q]);
-        }
-      }
+    for (int q = 0; q < 3; ++q) {
+      const float2 y = sub2(b[q], c[q]);
+      const float2 t = add2(s[q], y);
+      c[q] = sub2(sub2(t, s[q]), y);
+      s[q] = t;
+      b[q] = splat(0.f);
     }
+  };
+  while (v < v1) {
+    const int k = v / Qx, ve = min(v1, (k + 1) * Qx);
+    for (; v + 4 <= ve; v += 4) {
 #pragma unroll
-    for (int p = 0; p < 2; ++p)
+      for (int u = 0; u < 4; ++u) row(v + u);
+      block();
+    }
+    for (; v < ve; ++v) row(v);
+    block();
+    const float2 ph = splat(consts[8 + 2 * k]), pl = splat(consts[9 + 2 * k]), hh = splat(0.5f);
+    two_sum2(H[0], L[0], mul2(hh, s[0]));
+    two_sum2(H[0], L[0], mul2(hh, s[2]));
+    L[0] = fma2(splat(-0.5f), add2(c[0], c[2]), L[0]);
+    two_sum2(H[1], L[1], mul2(hh, s[1]));
+    two_sum2(H[1], L[1], mul2(hh, s[2]));
+    L[1] = fma2(splat(-0.5f), add2(c[1], c[2]), L[1]);
 #pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        const float2 y = sub2(b2[p][q], c2[p][q]);
-        const float2 t = add2(s2[p][q], y);
-        c2[p][q] = sub2(sub2(t, s2[p][q]), y);
-        s2[p][q] = t;
-      }
+    for (int q = 0; q < 3; ++q) {
+      const float2 x = mul2(ph, s[q]);
+      const float2 lo = add2(fma2(ph, s[q], mul2(splat(-1.f), x)),
+                             fma2(pl, s[q], mul2(splat(-1.f), mul2(ph, c[q]))));
+      two_sum2(H[2 + q], L[2 + q], x);
+      L[2 + q] = add2(L[2 + q], lo);
+      s[q] = c[q] = splat(0.f);
+    }
   }
-  float s[4][5], cpen[4][5];
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    s[0][q] = s2[0][q].x; s[1][q] = s2[0][q].y; s[2][q] = s2[1][q].x; s[3][q] = s2[1][q].y;
-    cpen[0][q] = c2[0][q].x; cpen[1][q] = c2[0][q].y;
-    cpen[2][q] = c2[1][q].x; cpen[3][q] = c2[1][q].y;
-  }
-  // FP32 transposing reduction of the 20 (sum, -compensation) pairs; only
-  // the final hi + lo of each is formed in FP64
-  float h[32], lo[32];
-#pragma unroll
-  for (int c = 0; c < 4; ++c)
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      h[c * 5 + q] = s[c][q];
-      lo[c * 5 + q] = -cpen[c][q];
-    }
-#pragma unroll
-  for (int i = 20; i < 32; ++i) {
-    h[i] = 0.f;
-    lo[i] = 0.f;
-  }
-  tr_level<16>(h, lo, lane);
-  tr_level<8>(h, lo, lane);
-  tr_level<4>(h, lo, lane);
-  tr_level<2>(h, lo, lane);
-  tr_level<1>(h, lo, lane);
-  if (lane < 20) {
-    const int c = lane / 5, q = lane - 5 * (lane / 5);
-    msum[q * kB2 + 4 * warp + c] = (double)h[0] + (double)lo[0];
+    const float2 h = make_float2(__shfl_xor_sync(0xffffffffu, H[q].x, 16),
+                                 __shfl_xor_sync(0xffffffffu, H[q].y, 16));
+    const float2 l = make_float2(__shfl_xor_sync(0xffffffffu, L[q].x, 16),
+                                 __shfl_xor_sync(0xffffffffu, L[q].y, 16));
+    two_sum2(H[q], L[q], h);
+    L[q] = add2(L[q], l);
+    if (lane < kB2 / 2)
+      *reinterpret_cast<float4*>(part + (size_t)(sl * 5 + q) * kB2 + 2 * pr) =
+          make_float4(H[q].x, L[q].x, H[q].y, L[q].y);
   }
 }
 
+// Element e = q kB2 + c of the moments of the tile, FP64, from the slices.
+__device__ __forceinline__ double moment_total(const float2* part, int e) {
+  float2 v = part[e];
+#pragma unroll
+  for (int i = 1; i < kSlices; ++i) {
+    const float2 x = part[i * 5 * kB2 + e];
+    const float t = v.x + x.x, bp = t - v.x;
+    v.y += x.y + ((v.x - (t - bp)) + (x.x - bp));
+    v.x = t;
+  }
+  return (double)v.x + (double)v.y;
+}
+
 // Landau matching (FP64) and relaxation time of cell c (0 <= c < kB2) of the
-// tile at s0; what the f^eq coefficients need goes to cellf [8][kB2] in FP32,
-// the collision rates gamma/tau and gamma beta/tau to gco [kH][g0x g0y g1x g1y].
-__device__ __forceinline__ void landau_cell(const double* msum, float* cellf, float* gco,
+// tile at s0: what the coefficients need to cells [4][kB2] in FP32 (it may share
+// the partial sums' memory), the collision rates (gamma, gamma beta) dt/tau to
+// gco [kH][g0x g0y g1x g1y].  ~40 FP64 instructions: a warp's FP64 instruction
+// takes a sub-partition ~64 cycles however many lanes are active, so the phase is
+// as short as its count.
+__device__ __forceinline__ void landau_cell(const double* msum, float* cells, float* gco,
                                             const SodGeom& g, int s0, int c, int* err) {
-  LandauOut Lo = landau_factored(msum[c], msum[kB2 + c], msum[2 * kB2 + c], msum[3 * kB2 + c],
-                                 msum[4 * kB2 + c]);
+  const LandauOut Lo = landau_factored(msum[c], msum[kB2 + c], msum[2 * kB2 + c],
+                                       msum[3 * kB2 + c], msum[4 * kB2 + c]);
   float g0 = 0.f, g1 = 0.f;
+  AeqCell<float> o{0.f, 1.f, 1.f, 0.f};
   if (!Lo.ok) {
     if (s0 + c < g.Z) report_err(err, 6, s0 + c);
-    Lo.n = 1.0; Lo.T = 1.0; Lo.beta = 0.0; Lo.gamma = 1.0; Lo.u = 0.0;
-  } else if (g.tau_mode == kTauEtas) {
-    const double tau = g.tau_AW0 / Lo.T *
-                       (1.0 - 0.25 * log(Lo.n / (Lo.T * Lo.T * Lo.T) * g.lambda_ref));
-    g0 = float(Lo.gamma / tau);
-    g1 = float(Lo.gamma * Lo.beta / tau);
   } else {
-    const float itau = 1.f / float(g.tau);
-    g0 = float(Lo.gamma) * itau;
-    g1 = float(Lo.gamma * Lo.beta) * itau;
+    o = {float(Lo.n), float(Lo.T), float(Lo.gamma), float(Lo.ub)};
+    float r = float(g.dt_tau);
+    if (g.tau_mode == kTauEtas) {
+      const double lam = Lo.n * g.lambda_ref * rcp64(Lo.T * Lo.T * Lo.T);
+      r = float(g.dt * Lo.T * rcp64(g.tau_AW0 * fma(-0.25, log(lam), 1.0)));
+    }
+    g0 = o.gamma * r;
+    g1 = o.ub * r;
   }
-  const float u = float(Lo.u);
-  const float A = asinhf(u);
-  cellf[0 * kB2 + c] = float(Lo.n);
-  cellf[1 * kB2 + c] = float(Lo.T);
-  cellf[2 * kB2 + c] = u;
-  cellf[3 * kB2 + c] = A;
-  cellf[4 * kB2 + c] = (u > 0.f) ? A / u : 1.f;
-  cellf[5 * kB2 + c] = u * u / (float(Lo.gamma) + 1.f);  // 2 sinh^2(A/2) = gamma - 1
-  cellf[6 * kB2 + c] = (Lo.beta < 0.0) ? -1.f : 1.f;
-  cellf[7 * kB2 + c] = Lo.ok ? 1.f : 0.f;
-  // gco[i][g0x g0y g1x g1y], cell c = half h, index i
+  cells[c] = o.n;
+  cells[kB2 + c] = o.T_;
+  cells[2 * kB2 + c] = o.gamma;
+  cells[3 * kB2 + c] = o.ub;
   const int h = c / kH, i = c - h * kH;
   gco[4 * i + h] = g0;
   gco[4 * i + 2 + h] = g1;
 }
 
-// FP32 constants of the coefficient phase, copied into shared memory by
-// load_consts: cst[0..15] the nodes and cst[16..31] the weights of the 16-node
-// Gauss-Legendre rule of the a_{l,m} integrals, cst[32 + k] = L_1^{(2)}(x_k).
-constexpr int kConsts = 32 + 8;
+// f^eq coefficients of the tile: thread t (0 <= t < 8 kB2; whole warps), 8 threads
+// per cell: all run the cell's chains, thread m writes the coefficients of order
+// m for every radial node; coef [QL][kH][kMP][2 halves].
+__device__ __forceinline__ void coefs(const float* cells, float* coef, const float* consts,
+                                      const SodGeom& g, const SodTables<float>& tb, int t) {
+  const int c = t >> 3, mine = t & 7;
+  float D[kMP], E[kMP];
+  const AeqCell<float> cell{cells[c], cells[kB2 + c], cells[2 * kB2 + c], cells[3 * kB2 + c]};
+  const AeqScalars<float> o =
+      aeq_cell<float, kMP>(cell, g.nm, 0xffffffffu, tb.gl_t, tb.gl_w, D, E);
+  float d = 0.f, e = 0.f, um = 0.f, bm = 1.f;
+#pragma unroll
+  for (int m = 0; m < kMP; ++m) {
+    if (m == mine) {
+      d = aeq_scale<float>(false, m) * D[m];
+      e = aeq_scale<float>(true, m) * E[m];
+      um = m < g.nm ? (m + 0.5f) * bm : 0.f;
+    }
+    bm *= o.q;
+  }
+  const float p3 = um * (o.A3 * d), pd = p3 - um * (o.A4 * e);
+  const int h = c / kH, i = c - h * kH;
+  float* dst = coef + ((size_t)i * kMP + mine) * 2 + h;
+  for (int k = 0; k < g.QL; ++k) dst[k * kH * kMP * 2] = fmaf(consts[k], pd, p3);
+}
 
+// Constants of the phases above in shared memory: L_1^{(2)}(x_k) (8), then
+// p_k as hi, lo pairs.
+constexpr int kConsts = 32 + 8;
 __device__ __forceinline__ void load_consts(float* cst, const SodTables<float>& tb, int QL, int t,
                                             int nt) {
-  for (int e = t; e < 32 + QL; e += nt)
-    cst[e] = e < 16 ? float(tb.gl_t[kAeqNodes + e])
-                    : (e < 32 ? float(tb.gl_w[kAeqNodes + e - 16]) : tb.L1k[e - 32]);
+  for (int e = t; e < 3 * QL; e += nt) cst[e < QL ? e : 8 + e - QL] = e < QL ? tb.L1k[e] : tb.pk[e - QL];
 }
 
-// f^eq coefficients of the tile: thread t (0 <= t < 8 kB2), 8 threads per cell
-// share the 16 nodes of the a_{l,m} rule; after an xor butterfly every thread
-// of a cell holds all the integrals, and thread q writes the coefficients of
-// order m = q for every radial node; coef [QL][kH][kMP][2 halves].
-__device__ __forceinline__ void coefs(const float* cellf, float* coef, const SodGeom& g,
-                                      const float* cst, int t) {
-  static_assert(kMP == 8, "one thread per order m");
-  const int c = t >> 3, q = t & 7;  // 8 threads per cell
-  const float ud = cellf[2 * kB2 + c];
-  const float A = cellf[3 * kB2 + c], sh2 = cellf[5 * kB2 + c];
-  const float uinv = (ud > 0.f) ? 1.f / ud : 0.f;
-  const bool at_rest = !(ud > 0.f);
-  float J3[kMaxM], J4[kMaxM];
-#pragma unroll
-  for (int m = 0; m < kMaxM; ++m) { J3[m] = 0.f; J4[m] = 0.f; }
-#pragma unroll
-  for (int i = 0; i < kAeqNodesF32 / 8; ++i)  // the 16-node rule (N_Omega <= 7 here)
-    aeq_node<float>(cst[q + 8 * i], cst[16 + q + 8 * i], A, sh2, uinv, at_rest, g.nm, J3, J4);
-#pragma unroll
-  for (int o = 4; o >= 1; o >>= 1)
-#pragma unroll
-    for (int m = 0; m < kMaxM; ++m)
-      if (m < g.nm) {
-        J3[m] += __shfl_xor_sync(0xffffffffu, J3[m], o);
-        J4[m] += __shfl_xor_sync(0xffffffffu, J4[m], o);
-      }
-  const int m = q;
-  float j3 = 0.f, j4 = 0.f;
-#pragma unroll
-  for (int mm = 0; mm < kMP; ++mm)
-    if (mm == m) {
-      j3 = J3[mm];
-      j4 = J4[mm];
-    }
-  const float fac = cellf[7 * kB2 + c] * cellf[0 * kB2 + c] * cellf[4 * kB2 + c] * 0.25f;
-  const float theta = cellf[1 * kB2 + c];
-  const float sgn = cellf[6 * kB2 + c];
-  const int h = c / kH, i = c - h * kH;
-  const float sm = ((m & 1) && sgn < 0.f) ? -fac : fac;  // fac sgn^m (sgn = +-1)
-  const float hh = sm * (float(m) + 0.5f);                // (2m + 1)/2, exact
-  const float d = j3 - theta * j4;
-  for (int k = 0; k < g.QL; ++k)
-    coef[(((size_t)k * kH + i) * kMP + m) * 2 + h] =
-        m < g.nm ? hh * (j3 + cst[32 + k] * d) : 0.f;
-}
-
-// Row sweeps: rows ir = first, first + stride, ... (negative-xi rows first,
-// so the upwind direction is uniform within a warp).
+// Row sweeps: rows ir = first, first + stride, ... (negative-xi rows first and
+// padded to whole warps, so the upwind direction is uniform within a warp;
+// stride a multiple of 32).
 __device__ __forceinline__ void sweep_rows(float* tile, const float* coef, const float* gco,
                                            const SodGeom& g, const SodTables<float>& tb,
                                            const int* __restrict__ rowv, int nneg, int first,
                                            int stride) {
-  const float inv_dz = float(g.inv_dz), dt = float(g.dt);
-  const int V = g.V;
-  for (int ir = first; ir < V; ir += stride) {
+  const float c1 = float(g.inv_dz * g.dt);
+  const int V = g.V, pad = (32 - nneg % 32) % 32;
+  for (int u = first; u < V + pad; u += stride) {
+    if (u >= nneg && u < nneg + pad) continue;
+    const int ir = u >= nneg ? u - pad : u;
     const int v = rowv[ir];
     const float xi = tb.xi[v];
     const int k = tb.kidx[v];
@@ -493,8 +494,8 @@ __device__ __forceinline__ void sweep_rows(float* tile, const float* coef, const
 #pragma unroll
     for (int m = 0; m < kMP; ++m) wp2[m] = splat((m < g.nm) ? tb.wp[m * V + v] : 0.f);
     const float* ck = coef + (size_t)k * kH * kMP * 2;
-    if (ir >= nneg) sweep_row2<true>(tile + v * kP, xi, wp2, g.nm, ck, gco, inv_dz, dt);
-    else sweep_row2<false>(tile + v * kP, xi, wp2, g.nm, ck, gco, inv_dz, dt);
+    if (ir >= nneg) sweep_row2<true>(tile + v * kP, xi, wp2, g.nm, ck, gco, c1 * xi);
+    else sweep_row2<false>(tile + v * kP, xi, wp2, g.nm, ck, gco, c1 * xi);
   }
 }
 
@@ -525,9 +526,11 @@ __device__ __forceinline__ void load_row_tables(const RowTables& rt, const SodGe
 __device__ __forceinline__ void sweep_rows_tab(float* tile, const float* coef, const float* gco,
                                                const SodGeom& g, const RowTables& rt, int nneg,
                                                int first, int stride) {
-  const float inv_dz = float(g.inv_dz), dt = float(g.dt);
-  const int V = g.V;
-  for (int ir = first; ir < V; ir += stride) {
+  const float c1 = float(g.inv_dz * g.dt);
+  const int V = g.V, pad = (32 - nneg % 32) % 32;
+  for (int u = first; u < V + pad; u += stride) {
+    if (u >= nneg && u < nneg + pad) continue;
+    const int ir = u >= nneg ? u - pad : u;
     const int v = rt.v[ir];
     const float xi = rt.xi[ir];
     const int k = rt.k[ir];
@@ -535,8 +538,8 @@ __device__ __forceinline__ void sweep_rows_tab(float* tile, const float* coef, c
 #pragma unroll
     for (int m = 0; m < kMP; ++m) wp2[m] = splat(rt.wp[m * V + ir]);
     const float* ck = coef + (size_t)k * kH * kMP * 2;
-    if (ir >= nneg) sweep_row2<true>(tile + v * kP, xi, wp2, g.nm, ck, gco, inv_dz, dt);
-    else sweep_row2<false>(tile + v * kP, xi, wp2, g.nm, ck, gco, inv_dz, dt);
+    if (ir >= nneg) sweep_row2<true>(tile + v * kP, xi, wp2, g.nm, ck, gco, c1 * xi);
+    else sweep_row2<false>(tile + v * kP, xi, wp2, g.nm, ck, gco, c1 * xi);
   }
 }
 
@@ -550,32 +553,37 @@ __device__ __forceinline__ void store(const float* tile, const float* __restrict
   const float b = (stage == 1) ? 0.25f : 2.f / 3.f;
   if (s0 + kB2 <= g.Z) {
     // full tile: kB2/4 chunks of 4 cells per row, 16-byte accesses, INFL loads
-    // of f_n in flight per thread
-    for (int base_i = t; base_i < V * (kB2 / 4); base_i += INFL * nt) {
+    // of f_n in flight per thread.  The first nt - nt % (kB2/4) threads each keep
+    // one chunk column and step over the rows, so no index is divided; the
+    // others have no rows (the caller's barrier needs whole warps, so they do
+    // not leave early).
+    constexpr int CQ = kB2 / 4;
+    const int dv = nt / CQ, v0 = t / CQ, q4 = 4 * (t - v0 * CQ);
+    const int ve = v0 < dv ? V : 0;
+    const size_t gs = (size_t)dv * g.ldz;
+    const float* pn = fn + (size_t)v0 * g.ldz + s0 + q4;
+    float* po = fout + (size_t)v0 * g.ldz + s0 + q4;
+    const float* pt = tile + v0 * kP + 4 + q4;
+    for (int v = v0; v < ve; v += INFL * dv) {
       float4 fo[INFL];
 #pragma unroll
-      for (int u = 0; u < INFL; ++u) {
-        const int idx = base_i + u * nt;
-        if (stage != 0 && idx < V * (kB2 / 4)) {
-          const int v = idx / (kB2 / 4), q = idx - v * (kB2 / 4);
-          fo[u] = __ldg(reinterpret_cast<const float4*>(fn + (size_t)v * g.ldz + s0 + 4 * q));
-        }
-      }
+      for (int u = 0; u < INFL; ++u)
+        if (stage != 0 && v + u * dv < V) fo[u] = __ldg(reinterpret_cast<const float4*>(pn + u * gs));
 #pragma unroll
-      for (int u = 0; u < INFL; ++u) {
-        const int idx = base_i + u * nt;
-        if (idx < V * (kB2 / 4)) {
-          const int v = idx / (kB2 / 4), q = idx - v * (kB2 / 4);
-          float4 r = *reinterpret_cast<const float4*>(tile + v * kP + 4 + 4 * q);
+      for (int u = 0; u < INFL; ++u)
+        if (v + u * dv < V) {
+          float4 r = *reinterpret_cast<const float4*>(pt + u * dv * kP);
           if (stage != 0) {
             r.x = a * fo[u].x + b * r.x;
             r.y = a * fo[u].y + b * r.y;
             r.z = a * fo[u].z + b * r.z;
             r.w = a * fo[u].w + b * r.w;
           }
-          *reinterpret_cast<float4*>(fout + (size_t)v * g.ldz + s0 + 4 * q) = r;
+          *reinterpret_cast<float4*>(po + u * gs) = r;
         }
-      }
+      pn += INFL * gs;
+      po += INFL * gs;
+      pt += INFL * dv * kP;
     }
   } else {
     for (int idx = t; idx < V * kB2; idx += nt) {
@@ -589,6 +597,7 @@ __device__ __forceinline__ void store(const float* tile, const float* __restrict
       }
     }
   }
+  __syncwarp();
 }
 
 }  // namespace p32

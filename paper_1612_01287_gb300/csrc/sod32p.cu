@@ -38,7 +38,6 @@ constexpr int kSweepWarps = 12;  // 600 rows in two rounds of 384
 constexpr int kCellT = 32 * kCellWarps;    // 128
 constexpr int kSweepT = 32 * kSweepWarps;  // 384
 constexpr int kThreads = kCellT + kSweepT;
-constexpr int kCellGroups = kB2 / 4;  // moments: 4 cells per warp pass
 constexpr int kStoreInflight = 12;    // f_n loads in flight per sweep thread in the store
 constexpr long long kWaitCycles = 4000000000ll;  // ~2 s at the maximum SM clock
 constexpr uint32_t kSuspendNs = 1000;
@@ -76,17 +75,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
   return true;
 }
 
+// The group barriers are the per-thread (not .aligned) forms, after a warp
+// barrier: a group's loops and per-cell branches leave lanes of one warp at
+// different places, and the aligned forms count a warp that arrives in two
+// parts twice.
 __device__ __forceinline__ void named_sync(int id, int n) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+  __syncwarp();
+  asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
 // Barrier among the n threads of named barrier id that returns whether any
 // of them passed pred != 0 (a group-uniform decision).
 __device__ __forceinline__ bool named_sync_or(int id, int n, int pred) {
   uint32_t r;
+  __syncwarp();
   asm volatile(
       "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n"
-      " bar.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}"
+      " barrier.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}"
       : "=r"(r)
       : "r"(pred), "r"(id), "r"(n)
       : "memory");
@@ -101,11 +106,10 @@ struct Smem {
   float* tile[2];
   float* coef[2];
   float* gco[2];
-  float* mws;
+  float2* part;
   float* cst;
   RowTables rt;
   double* msum;
-  float* cellf;
   uint64_t* full;
   uint64_t* ready;
   int* abort_flag;
@@ -127,11 +131,18 @@ __host__ __device__ __forceinline__ size_t rowtab_bytes(int V) {
   return 3 * al128(sizeof(int) * (size_t)V) + al128(sizeof(float) * kMP * (size_t)V);
 }
 
+// The moment slices' partial sums; like scratch_bytes, not smaller than the
+// weights and scalars they replaced (the size decides what fits).
+__host__ __device__ __forceinline__ size_t part_bytes(int V) {
+  const size_t part = al128(sizeof(float2) * kSlices * 5 * kB2);
+  const size_t old = al128(sizeof(float) * 5 * (size_t)V) + al128(sizeof(float) * 8 * kB2);
+  return old > part ? old : part;
+}
+
 __host__ __device__ __forceinline__ size_t smem_total(int V, int QL) {
   return 2 * tile_bytes(V) + 2 * coef_bytes(QL) + 2 * al128(sizeof(float) * kH * 4) +
-         al128(sizeof(float) * 5 * (size_t)V) + al128(sizeof(float) * kConsts) +
-         rowtab_bytes(V) + al128(sizeof(double) * 5 * kB2) + al128(sizeof(float) * 8 * kB2) +
-         128 + 128;
+         part_bytes(V) + al128(sizeof(float) * kConsts) + rowtab_bytes(V) +
+         al128(sizeof(double) * 5 * kB2) + 128 + 128;
 }
 
 __device__ __forceinline__ Smem carve(unsigned char* base, int V, int QL) {
@@ -149,8 +160,8 @@ __device__ __forceinline__ Smem carve(unsigned char* base, int V, int QL) {
     m.gco[b] = reinterpret_cast<float*>(base + o);
     o += al128(sizeof(float) * kH * 4);
   }
-  m.mws = reinterpret_cast<float*>(base + o);
-  o += al128(sizeof(float) * 5 * (size_t)V);
+  m.part = reinterpret_cast<float2*>(base + o);
+  o += part_bytes(V);
   m.cst = reinterpret_cast<float*>(base + o);
   o += al128(sizeof(float) * kConsts);
   m.rt.v = reinterpret_cast<int*>(base + o);
@@ -163,8 +174,6 @@ __device__ __forceinline__ Smem carve(unsigned char* base, int V, int QL) {
   o += al128(sizeof(float) * kMP * (size_t)V);
   m.msum = reinterpret_cast<double*>(base + o);
   o += al128(sizeof(double) * 5 * kB2);
-  m.cellf = reinterpret_cast<float*>(base + o);
-  o += al128(sizeof(float) * 8 * kB2);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + o);
   m.full = bars;
   m.ready = bars + 2;
@@ -230,7 +239,6 @@ sod32p_stage_kernel(const float* __restrict__ fin, const float* __restrict__ fn,
   int issued = 0;
   if (tid == issuer)
     for (; issued < 2 && issued < ntile_cta; ++issued) issue(issued);
-  for (int e = tid; e < 5 * V; e += kThreads) S.mws[e] = tb.mw[e];
   load_consts(S.cst, tb, g.QL, tid, kThreads);
   load_row_tables(S.rt, g, tb, rowv, tid, kThreads);
   __syncthreads();
@@ -256,18 +264,23 @@ sod32p_stage_kernel(const float* __restrict__ fin, const float* __restrict__ fn,
         named_sync(kBarCell, kCellT);
       }
       if (collide) {
-        for (int grp = warp; grp < kCellGroups; grp += kCellWarps)
-          moments(tile, S.mws, S.msum, V, grp, lane);
+        for (int sl = warp; sl < kSlices; sl += kCellWarps)
+          moments(tile, tb.m3, S.cst, S.part, V, g.Qx, sl, lane);
+        named_sync(kBarCell, kCellT);
+        for (int e = tid; e < 5 * kB2; e += kCellT) S.msum[e] = moment_total(S.part, e);
         named_sync(kBarCell, kCellT);
         // Landau matching: the cells spread over the warps, so that the FP64
         // work of the tile is shared by all four SM sub-partitions
         {
-          const int c = warp + kCellWarps * lane;
-          if (lane < (kB2 + kCellWarps - 1) / kCellWarps && c < kB2)
-            landau_cell(S.msum, S.cellf, S.gco[b], g, s0, c, err);
+          constexpr int CL = (kB2 + kCellWarps - 1) / kCellWarps;
+          static_assert(CL * kCellWarps == kB2, "whole cells per warp");
+          if (lane < CL)
+            landau_cell(S.msum, reinterpret_cast<float*>(S.part), S.gco[b], g, s0,
+                        warp + kCellWarps * lane, err);
         }
         named_sync(kBarCell, kCellT);
-        for (int q = tid; q < kCellThreads; q += kCellT) coefs(S.cellf, S.coef[b], g, S.cst, q);
+        for (int w = warp; w < kCellThreads / 32; w += kCellWarps)
+          coefs(reinterpret_cast<const float*>(S.part), S.coef[b], S.cst, g, tb, 32 * w + lane);
       } else {
         for (int e = tid; e < g.QL * kH * kMP * 2; e += kCellT) S.coef[b][e] = 0.f;
         for (int e = tid; e < kH * 4; e += kCellT) S.gco[b][e] = 0.f;
