@@ -536,6 +536,8 @@ struct rslb_bjorken {
   int ntc;
   size_t tc_smem;
   float* kimg;
+  float* npool32;  // FP32 constants of the stage kernel's epilogue
+  float* rad32;
   void* F1;
   void* F2;
   double* mp[2];
@@ -552,7 +554,7 @@ void bj_free(rslb_bjorken* b) {
   if (!b) return;
   void* ptrs[] = {b->state, b->kpool, b->npool, b->kpc, b->blocks, b->qtab, b->roff, b->xoff, b->rq,
                   b->tau_aw0, b->gas, b->user, b->xk, b->wk, b->KL, b->err, b->out_dev,
-                  b->tcblocks, b->kimg, b->F1, b->F2, b->mp[0], b->mp[1], b->ytmp,
+                  b->tcblocks, b->kimg, b->npool32, b->rad32, b->F1, b->F2, b->mp[0], b->mp[1], b->ytmp,
                   b->step_dev};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -649,7 +651,7 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
   b->tcblocks = nullptr;
   b->ntc = 0;
   b->tc_smem = 0;
-  b->kimg = nullptr;
+  b->kimg = b->npool32 = b->rad32 = nullptr;
   b->F1 = b->F2 = nullptr;
   b->mp[0] = b->mp[1] = nullptr;
   b->mp_cur = 0;
@@ -823,8 +825,17 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
     rc = set_error(RSLB_ERR_ALLOC, "rslb_bjorken_init: cudaMalloc failed");
   if (!rc && o->kp_mode == RSLB_KP_TF32X3) {
     rc = dev_upload(&b->tcblocks, tcb.data(), tcb.size());
+    std::vector<float> n32(npool.size());
+    for (size_t i = 0; i < qvals.size(); ++i)
+      for (int j = 0; j < qvals[i]; ++j) {
+        const size_t x = (size_t)qtab[i].xi_off + j;
+        n32[x] = (float)(npool[x] * npool[x]);
+        n32[x + qvals[i]] = (float)npool[x + qvals[i]];
+      }
+    if (!rc) rc = dev_upload(&b->npool32, n32.data(), n32.size());
     const size_t sb = sizeof(float) * (size_t)b->total_state;
     if (!rc && (cudaMalloc((void**)&b->kimg, sizeof(float) * (size_t)img_total) != cudaSuccess ||
+                cudaMalloc((void**)&b->rad32, sizeof(float) * QL * (QL + 3)) != cudaSuccess ||
                 cudaMalloc(&b->F1, sb) != cudaSuccess || cudaMalloc(&b->F2, sb) != cudaSuccess ||
                 cudaMalloc((void**)&b->ytmp, sb) != cudaSuccess ||
                 cudaMalloc((void**)&b->mp[0], sizeof(double) * 8 * nruns) != cudaSuccess ||
@@ -856,6 +867,7 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
       bj_tc_image_launch(qvals[i], b->npool + qtab[i].xi_off, b->kpc, b->kimg + img_off[i], st);
   }
   bj_kl_kernel<<<1, QL * QL, 0, st>>>(QL, b->xk, b->wk, b->KL);
+  if (o->kp_mode == RSLB_KP_TF32X3) bj_tc_radial_launch(QL, b->xk, b->wk, b->KL, b->rad32, st);
   if (b->precision == RSLB_F64)
     bj_init_kernel<double><<<nruns, 128, 0, st>>>(nruns, QL, b->rq, b->roff, b->xoff, b->npool,
                                                    b->wk, (double*)b->state);
@@ -893,10 +905,11 @@ namespace {
 
 // Steps of a graph of the tensor-core path: an even count, so that the moment
 // buffers are back in their starting roles at its end.
-constexpr int kTcGraphSteps = 2;
+constexpr int kTcGraphSteps = 8;
 
 // Enqueue nsteps RK3 steps of the tensor-core path: three stage launches each
-// (stage times from the device step counter, Tab. II) and the counter update.
+// (stage times from the device step counter and the step within the call, Tab.
+// II) and one update of the counter.
 cudaError_t bj_tc_enqueue(rslb_bjorken* b, int nsteps) {
   float* F[3] = {(float*)b->state, (float*)b->F1, (float*)b->F2};
   cudaError_t e = cudaSuccess;
@@ -905,12 +918,10 @@ cudaError_t bj_tc_enqueue(rslb_bjorken* b, int nsteps) {
       BjTcArgs a{};
       a.blocks = b->tcblocks;
       a.kimg = b->kimg;
-      a.npool = b->npool;
+      a.npool32 = b->npool32;
+      a.rad32 = b->rad32;
       a.tau_aw0 = b->tau_aw0;
       a.gas = b->gas;
-      a.xk = b->xk;
-      a.wk = b->wk;
-      a.KL = b->KL;
       a.QL = b->QL;
       a.stage = stage;
       a.Fin = F[stage];
@@ -920,14 +931,15 @@ cudaError_t bj_tc_enqueue(rslb_bjorken* b, int nsteps) {
       a.mp_out = b->mp[1 - b->mp_cur];
       a.dout = nullptr;
       a.step = b->step_dev;
+      a.step_off = n;
       a.tau0 = b->tau0;
       a.dtau = b->dtau;
       a.err = b->err;
       e = bj_tc_stage_launch(a, b->ntc, b->tc_smem, b->stream);
       b->mp_cur = 1 - b->mp_cur;
     }
-    if (e == cudaSuccess) e = bj_step_count_launch(b->step_dev, b->stream);
   }
+  if (e == cudaSuccess) e = bj_step_count_launch(b->step_dev, nsteps, b->stream);
   return e;
 }
 
@@ -1075,12 +1087,10 @@ extern "C" int rslb_bjorken_selftest_timeout(rslb_bjorken* b) {
   BjTcArgs a{};
   a.blocks = b->tcblocks;
   a.kimg = b->kimg;
-  a.npool = b->npool;
+  a.npool32 = b->npool32;
+  a.rad32 = b->rad32;
   a.tau_aw0 = b->tau_aw0;
   a.gas = b->gas;
-  a.xk = b->xk;
-  a.wk = b->wk;
-  a.KL = b->KL;
   a.QL = b->QL;
   a.stage = -1;
   a.Fin = (const float*)b->state;
@@ -1105,12 +1115,10 @@ extern "C" int rslb_bjorken_kp_apply(rslb_bjorken* b, void* y) {
   BjTcArgs a{};
   a.blocks = b->tcblocks;
   a.kimg = b->kimg;
-  a.npool = b->npool;
+  a.npool32 = b->npool32;
+  a.rad32 = b->rad32;
   a.tau_aw0 = b->tau_aw0;
   a.gas = b->gas;
-  a.xk = b->xk;
-  a.wk = b->wk;
-  a.KL = b->KL;
   a.QL = b->QL;
   a.stage = -1;
   a.Fin = (const float*)b->state;

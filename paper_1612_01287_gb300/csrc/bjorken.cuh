@@ -131,12 +131,10 @@ __host__ __device__ inline long long bj_tc_image_floats(int n) { return (long lo
 struct BjTcArgs {
   const BjTcBlock* blocks;
   const float* kimg;      // K^P images (FP32, tiles pre-swizzled)
-  const double* npool;    // [xi | w] per distinct Q
+  const float* npool32;   // [xi^2 | w] per distinct Q
+  const float* rad32;     // [x_k | w_k | 3 - x_k | K^L (QL x QL)]
   const double* tau_aw0;  // per run (sorted); <= 0 or inf: collisionless
   const int* gas;         // per run (sorted)
-  const double* xk;
-  const double* wk;
-  const double* KL;       // [QL][QL]
   int QL;
   int stage;              // 0, 1, 2 (Eq. rk3); -1: write K^P f to dout only
   const float* Fin;       // state the stage differentiates
@@ -146,8 +144,9 @@ struct BjTcArgs {
   double* mp_out;         // moments of Fout
   float* dout;            // stage -1 only
   double tau, dtau;       // stage time and step
-  const long long* step;  // if set: the stage time is tau0 + (*step + c_stage) dtau, with
-  double tau0;            // c = 0, 1, 1/2 (Tab. II), read on the device (graph replays)
+  const long long* step;  // if set: the stage time is tau0 + (*step + step_off + c_stage) dtau,
+  double tau0;            // with c = 0, 1, 1/2 (Tab. II), read on the device (graph replays)
+  int step_off;
   int* err;
   int withhold_ready;     // failure-handling self-test: the workers never
                           // signal that their operand tiles are ready
@@ -159,7 +158,9 @@ constexpr int kTcMaxCols = 80;
 cudaError_t bj_tc_set_attributes();
 size_t bj_tc_smem_bytes(int nc, int R);
 cudaError_t bj_tc_stage_launch(const BjTcArgs& a, int nblocks, size_t smem, cudaStream_t st);
-cudaError_t bj_step_count_launch(long long* step, cudaStream_t st);
+cudaError_t bj_step_count_launch(long long* step, int n, cudaStream_t st);
+cudaError_t bj_tc_radial_launch(int QL, const double* xk, const double* wk, const double* KL,
+                                float* rad32, cudaStream_t st);
 cudaError_t bj_tc_image_launch(int Q, const double* xw, const double* kc, float* img,
                                cudaStream_t st);
 cudaError_t bj_tc_moments_launch(int nruns, int QL, const int* rq, const long long* roff,

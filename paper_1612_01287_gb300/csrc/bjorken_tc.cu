@@ -35,7 +35,7 @@
 namespace rslb {
 namespace {
 
-constexpr int kTcThreads = 160;  // 4 worker warps + 1 issuer warp
+constexpr int kTcThreads = 192;  // 4 worker warps, the issuer's warp, the equilibrium's warp
 constexpr int kTcWorkers = 128;
 constexpr uint32_t kATile = 128 * 128;  // bytes: 128 rows x 32 FP32
 constexpr int kSpinLimit = 150000;       // try_wait rounds of at most kSuspendNs: ~0.3 s
@@ -203,7 +203,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) bj_tc_stage_kernel(BjTcArgs a) 
   uint64_t* ready = full + 2;                          // [2] workers filled the stage
   uint64_t* done = ready + 2;                          // [2] MMAs of the stage finished
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 2);
-  float* rs = reinterpret_cast<float*>(tail + 64);  // rate[R] | neq4[R] | omt[R]
+  float* s_itau = reinterpret_cast<float*>(tmem_slot + 1);  // 1 / stage time
+  float* rs = reinterpret_cast<float*>(tail + 64);          // rate[R] | neq4[R] | omt[R]
   float* mp = rs + 3 * R;                           // [4 warps][R][2]
 
   // zero the rows of the A buffers that the copies of the shorter image (O,
@@ -279,12 +280,13 @@ __global__ void __launch_bounds__(kTcThreads, 2) bj_tc_stage_kernel(BjTcArgs a) 
     }
   }
 
-  // per-run equilibrium of the stage state from the moment partials, by the
-  // issuer's 31 idle lanes while the workers start on the K-loop (the
-  // epilogue reads it after the CTA barrier that ends the loop)
+  // per-run equilibrium of the stage state from the moment partials, and the
+  // stage time's reciprocal, by a warp of their own while the K-loop runs (the
+  // epilogue reads them after the CTA barrier that ends the loop): ~8k cycles of
+  // FP64 latency that the issuer's warp used to wait for before its first MMA
   const bool rk = a.stage >= 0;
-  if (rk && warp == 4 && lane > 0) {
-    for (int r = lane - 1; r < R; r += 31) {
+  if (rk && warp == 5) {
+    for (int r = lane; r < R; r += 32) {
       const int gr = blk.first + r;
       double N = 0.0, E = 0.0;
       for (int m = 0; m < blk.nmt; ++m) {
@@ -316,6 +318,14 @@ __global__ void __launch_bounds__(kTcThreads, 2) bj_tc_stage_kernel(BjTcArgs a) 
       rs[R + r] = float(neq4);
       rs[2 * R + r] = float(omt);
     }
+    if (lane == 0) {
+      const double tau_s =
+          a.step ? a.tau0 + ((double)(*a.step + a.step_off) +
+                             (a.stage == 1 ? 1.0 : (a.stage == 2 ? 0.5 : 0.0))) *
+                                a.dtau
+                 : a.tau;
+      *s_itau = float(1.0 / tau_s);
+    }
   }
 
   // what the epilogue needs from global memory, loaded before the K-loop so
@@ -328,22 +338,20 @@ __global__ void __launch_bounds__(kTcThreads, 2) bj_tc_stage_kernel(BjTcArgs a) 
   float KL[QL * QL], xk[QL], wk[QL], l1[QL];
   if (warp < 4) {
     if (okE) {
-      const double x = a.npool[blk.xoff + j1];
-      xi2a = float(x * x);
-      wja = float(a.npool[blk.xoff + Q + j1]);
+      xi2a = a.npool32[blk.xoff + j1];
+      wja = a.npool32[blk.xoff + Q + j1];
     }
     if (okO) {
-      const double x = a.npool[blk.xoff + j2];
-      xi2b = float(x * x);
-      wjb = float(a.npool[blk.xoff + Q + j2]);
+      xi2b = a.npool32[blk.xoff + j2];
+      wjb = a.npool32[blk.xoff + Q + j2];
     }
 #pragma unroll
     for (int k = 0; k < QL; ++k) {
-      xk[k] = float(a.xk[k]);
-      wk[k] = float(a.wk[k]);
-      l1[k] = float(3.0 - a.xk[k]);
+      xk[k] = a.rad32[k];
+      wk[k] = a.rad32[QL + k];
+      l1[k] = a.rad32[2 * QL + k];
 #pragma unroll
-      for (int q = 0; q < QL; ++q) KL[k * QL + q] = float(a.KL[k * QL + q]);
+      for (int q = 0; q < QL; ++q) KL[k * QL + q] = a.rad32[(3 + k) * QL + q];
     }
   }
 
@@ -470,11 +478,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) bj_tc_stage_kernel(BjTcArgs a) 
   // ---- epilogue (worker warps): rows j1 = i and j2 = Q-1-i per thread ----
   // (K f)_{j1} = (Y_E + Y_O)/2, (K f)_{j2} = (Y_E - Y_O)/2 (Y_O = 0 past h)
   if (warp < 4) {
-    const double tau_s =
-        a.step ? a.tau0 + ((double)*a.step + (a.stage == 1 ? 1.0 : (a.stage == 2 ? 0.5 : 0.0))) *
-                              a.dtau
-               : a.tau;
-    const float itau = float(1.0 / tau_s), dt = float(a.dtau);
+    const float itau = *s_itau, dt = float(a.dtau);
     const float ca = a.stage == 1 ? 0.75f : 1.f / 3.f, cb = a.stage == 1 ? 0.25f : 2.f / 3.f;
     const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
     const float* Fin = a.Fin + blk.soff;
@@ -605,6 +609,19 @@ __global__ void __launch_bounds__(kTcThreads, 2) bj_tc_stage_kernel(BjTcArgs a) 
   }
 }
 
+// The epilogue's radial constants in FP32: [x_k | w_k | 3 - x_k | K^L].
+__global__ void bj_tc_radial_kernel(int QL, const double* __restrict__ xk,
+                                    const double* __restrict__ wk, const double* __restrict__ KL,
+                                    float* rad32) {
+  const int e = threadIdx.x;
+  if (e < QL) {
+    rad32[e] = float(xk[e]);
+    rad32[QL + e] = float(wk[e]);
+    rad32[2 * QL + e] = float(3.0 - xk[e]);
+  }
+  if (e < QL * QL) rad32[3 * QL + e] = float(KL[e]);
+}
+
 // Images of one Q, split for 3xTF32: the even matrix E (qh x qh) at img and
 // the odd matrix O (h x h) after it (see BjTcBlock).  Tile (mt, kb) of an
 // n x n matrix = rows i in M-tile mt (rows(mt) of them) x columns
@@ -674,10 +691,10 @@ cudaError_t bj_tc_set_attributes() {
   return cudaSuccess;
 }
 
-__global__ void bj_step_count_kernel(long long* step) { *step += 1; }
+__global__ void bj_step_count_kernel(long long* step, int n) { *step += n; }
 
-cudaError_t bj_step_count_launch(long long* step, cudaStream_t st) {
-  bj_step_count_kernel<<<1, 1, 0, st>>>(step);
+cudaError_t bj_step_count_launch(long long* step, int n, cudaStream_t st) {
+  bj_step_count_kernel<<<1, 1, 0, st>>>(step, n);
   return cudaGetLastError();
 }
 
@@ -696,6 +713,12 @@ cudaError_t bj_tc_image_launch(int Q, const double* xw, const double* kc, float*
                                cudaStream_t st) {
   const int n = (Q - Q / 2) * (Q - Q / 2);
   bj_tc_image_kernel<<<(n + 127) / 128, 128, 0, st>>>(Q, xw, kc, img);
+  return cudaGetLastError();
+}
+
+cudaError_t bj_tc_radial_launch(int QL, const double* xk, const double* wk, const double* KL,
+                                float* rad32, cudaStream_t st) {
+  bj_tc_radial_kernel<<<1, 64, 0, st>>>(QL, xk, wk, KL, rad32);
   return cudaGetLastError();
 }
 
