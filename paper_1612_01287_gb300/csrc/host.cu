@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdint>
 #include <cstdlib>
 #include <cstring>
 #include <vector>
@@ -477,8 +478,8 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   if (!rc) rc = upload<double>((void**)&h->d_wp, wp);
   if (!rc) rc = upload<double>((void**)&h->d_L1k, L1k);
   if (!rc) {
-    std::vector<unsigned char> mom(sod_moment_weights(fp64, V, xiv.data(), pv.data(), nullptr));
-    sod_moment_weights(fp64, V, xiv.data(), pv.data(), mom.data());
+    std::vector<unsigned char> mom(sod_moment_weights(fp64, V, Qx, xiv.data(), pv.data(), nullptr));
+    sod_moment_weights(fp64, V, Qx, xiv.data(), pv.data(), mom.data());
     if (cudaMalloc(&h->d_mom, mom.size()) != cudaSuccess)
       rc = set_error(RSLB_ERR_ALLOC, "cudaMalloc of a table failed");
     else if (cudaMemcpy(h->d_mom, mom.data(), mom.size(), cudaMemcpyHostToDevice) != cudaSuccess)
@@ -664,17 +665,26 @@ extern "C" int rslb_sync(rslb_handle* h) {
 extern "C" int rslb_moments(rslb_handle* h, double* out, int out_on_device) {
   clear_error();
   if (!h || !out) return set_error(RSLB_ERR_ARG, "rslb_moments: NULL argument");
-  cudaError_t e = h->fp64 ? sod_moments_launch<double>(h->geom, h->d_mom,
-                                                       (const double*)h->F[0], h->d_fields,
-                                                       h->d_err, h->stream)
-                          : sod_moments_launch<float>(h->geom, h->d_mom,
-                                                      (const float*)h->F[0], h->d_fields,
-                                                      h->d_err, h->stream);
+  // into plain device memory of this GPU the kernel writes by itself; any other
+  // destination gets a copy
+  bool direct = false;
+  if (out_on_device && reinterpret_cast<uintptr_t>(out) % sizeof(double) == 0) {
+    cudaPointerAttributes at;
+    int dev = -1;
+    direct = cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, out) == cudaSuccess &&
+             at.type == cudaMemoryTypeDevice && at.device == dev;
+    if (!direct) cudaGetLastError();
+  }
+  double* dst = direct ? out : h->d_fields;
+  cudaError_t e = h->fp64 ? sod_moments_launch<double>(h->geom, h->d_mom, (const double*)h->F[0],
+                                                       dst, h->d_err, h->stream)
+                          : sod_moments_launch<float>(h->geom, h->d_mom, (const float*)h->F[0],
+                                                      dst, h->d_err, h->stream);
   if (e != cudaSuccess) return cuda_error(e, "rslb_moments: launch");
-  const size_t bytes = sizeof(double) * RSLB_NFIELDS * (size_t)h->cfg.Z;
-  e = cudaMemcpyAsync(out, h->d_fields, bytes,
-                      out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                      h->stream);
+  if (!direct)
+    e = cudaMemcpyAsync(out, h->d_fields, sizeof(double) * RSLB_NFIELDS * (size_t)h->cfg.Z,
+                        out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                        h->stream);
   if (e != cudaSuccess) return cuda_error(e, "rslb_moments: copy");
   return check_device_error(h);
 }

@@ -145,11 +145,9 @@ template <typename T>
 cudaError_t sod_moments_launch(const SodGeom& g, const void* w, const T* f, double* out,
                                int* err, cudaStream_t st);
 
-// Host: the moment weight table, for velocity v w_q = (1+xi), (1-xi),
-// p(1+xi)^2, p(1-xi)^2, p(1-xi^2): FP32 populations get 12 floats per
-// velocity {hi0..hi3}{hi4 lo0 lo1 lo2}{lo3 lo4 0 0} with w = hi + lo; FP64
-// populations get 6 doubles {w0..w4 0}.  With out == NULL only the byte
-// size is returned.
-size_t sod_moment_weights(bool fp64, int V, const double* xi, const double* p, void* out);
+// Host: the output-moment weight table (layouts at the kernels in moments.cu)
+// of velocities v = k Qx + j with nodes xi[v] and p[v].  With out == NULL only
+// the byte size is returned.
+size_t sod_moment_weights(bool fp64, int V, int Qx, const double* xi, const double* p, void* out);
 
 }  // namespace rslb
