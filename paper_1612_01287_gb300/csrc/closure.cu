@@ -17,16 +17,26 @@
 //    would take more than half of a positive population (a positivity
 //    limiter that keeps the conservation).
 //
-// Training: one CTA holds up to 128 samples; each thread runs forward and
-// backward for its sample out of shared memory, then the CTA reduces the
-// weight gradients over its samples into a per-CTA partial; a second kernel
-// sums the partials in a fixed order (deterministic), a third applies Adam.
+// The network's kernels use four threads per sample (64 samples per CTA; training
+// 128), each with a quarter of every layer's outputs in packed FP32x2
+// accumulators; activations pass between layers through shared memory, and a
+// warp's lanes share the weights they read (broadcasts).  What bounds them is
+// the FMA pipe and the shared-memory broadcasts, about equal; one thread per
+// sample (64 scalar accumulators) left the chip with one warp per scheduler.
+// 65536 cells, 73-64-64-24: 69 us per application, cold (173 before); a
+// minibatch of 8192: 72 us for the gradient (279).
+//
+// Training: forward and backward of the CTA's samples, then the CTA reduces the
+// weight gradients over its samples into a per-CTA partial (a thread holds a
+// tile of 4 rows x 3 columns of a layer's gradient); a second kernel sums the
+// partials in a fixed order (deterministic) and applies Adam.
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <initializer_list>
 #include <type_traits>
 #include <vector>
 
@@ -38,7 +48,7 @@ namespace {
 
 constexpr int kMaxD = 128;
 constexpr int kMaxO = 32;
-constexpr int kSmemLimit = 232448;
+constexpr int kSmemLimit = 232448 - 2048;  // dynamic; the rest holds the static arrays
 constexpr float kLimitTheta = 0.5f;  // positivity limiter of the correction
 
 struct MlpShape {
@@ -61,39 +71,62 @@ MlpShape make_shape(int D, int H, int O) {
   return s;
 }
 
-// Shared-memory weight block: W1T [D][H], W2 [H][H], W3 [O][H] (BF16 values
-// widened to FP32), b1 [H], b2 [H], b3 [O], then the fixed normalisation
-// mu [D], inv_sd [D], out_sd [O] (the network sees (x - mu) * inv_sd, its
-// output is scaled by out_sd).
-__host__ __device__ inline int wblock_floats(const MlpShape& s) {
-  return s.D * s.H + s.H * s.H + s.O * s.H + 2 * s.H + s.O + 2 * s.D + s.O;
-}
+constexpr int kNS = 64;                // samples per CTA
+constexpr int kParts = 4;              // threads per sample
+constexpr int kNetThreads = kNS * kParts;
+constexpr int kMaxV4 = kMaxO / kParts;  // populations per thread of a cell
 
-__host__ __device__ inline int norm_offset(const MlpShape& s) {
-  return s.D * s.H + s.H * s.H + s.O * s.H + 2 * s.H + s.O;
-}
+__host__ __device__ inline int o_pad(const MlpShape& s) { return (s.O + 7) & ~7; }
 
-__device__ inline void load_weights(const MlpShape& s, const __nv_bfloat16* __restrict__ wb,
+// Shared-memory weight block (BF16 values widened to FP32): W1T [D][H], W2T [H][H]
+// (input-major), W3T [H][OP] (OP = O rounded up to 8, zero columns), b1 [H],
+// b2 [H], b3 [OP], then the fixed normalisation mu [D], inv_sd [D], out_sd [OP]
+// (the network sees (x - mu) * inv_sd, its output is scaled by out_sd).
+struct NetSmem {
+  int W1T, W2T, W3T, b1, b2, b3, mu, isd, osd, end;
+  __host__ __device__ NetSmem(const MlpShape& s) {
+    const int OP = o_pad(s);
+    W1T = 0;
+    W2T = W1T + s.D * s.H;
+    W3T = W2T + s.H * s.H;
+    b1 = W3T + s.H * OP;
+    b2 = b1 + s.H;
+    b3 = b2 + s.H;
+    mu = b3 + OP;
+    isd = mu + s.D;
+    osd = isd + s.D;
+    end = (osd + OP + 3) & ~3;
+  }
+};
+
+__device__ inline void load_weights(const MlpShape& s, const NetSmem& L,
+                                    const __nv_bfloat16* __restrict__ wb,
                                     const float* __restrict__ theta,
                                     const float* __restrict__ nrm, float* sw) {
-  for (int e = threadIdx.x; e < 2 * s.D + s.O; e += blockDim.x) sw[norm_offset(s) + e] = nrm[e];
-  float* W1T = sw;
-  float* W2 = W1T + s.D * s.H;
-  float* W3 = W2 + s.H * s.H;
-  float* b1 = W3 + s.O * s.H;
-  float* b2 = b1 + s.H;
-  float* b3 = b2 + s.H;
-  for (int e = threadIdx.x; e < s.H * s.D; e += blockDim.x) {
-    const int h = e / s.D, d = e - h * s.D;
-    W1T[d * s.H + h] = __bfloat162float(wb[s.oW1 + e]);
+  const int OP = o_pad(s), t = threadIdx.x, nt = blockDim.x;
+  // consecutive threads write consecutive shared words; the strided reads of the
+  // few KB of weights hit L1
+  for (int e = t; e < s.H * s.D; e += nt) {
+    const int d = e / s.H, h = e - d * s.H;
+    sw[L.W1T + e] = __bfloat162float(wb[s.oW1 + h * s.D + d]);
   }
-  for (int e = threadIdx.x; e < s.H * s.H; e += blockDim.x) W2[e] = __bfloat162float(wb[s.oW2 + e]);
-  for (int e = threadIdx.x; e < s.O * s.H; e += blockDim.x) W3[e] = __bfloat162float(wb[s.oW3 + e]);
-  for (int e = threadIdx.x; e < s.H; e += blockDim.x) {
-    b1[e] = theta[s.ob1 + e];
-    b2[e] = theta[s.ob2 + e];
+  for (int e = t; e < s.H * s.H; e += nt) {
+    const int i = e / s.H, h = e - i * s.H;
+    sw[L.W2T + e] = __bfloat162float(wb[s.oW2 + h * s.H + i]);
   }
-  for (int e = threadIdx.x; e < s.O; e += blockDim.x) b3[e] = theta[s.ob3 + e];
+  for (int e = t; e < OP * s.H; e += nt) {
+    const int i = e / OP, o = e - i * OP;
+    sw[L.W3T + e] = o < s.O ? __bfloat162float(wb[s.oW3 + o * s.H + i]) : 0.f;
+  }
+  for (int e = t; e < s.H; e += nt) {
+    sw[L.b1 + e] = theta[s.ob1 + e];
+    sw[L.b2 + e] = theta[s.ob2 + e];
+  }
+  for (int e = t; e < OP; e += nt) {
+    sw[L.b3 + e] = e < s.O ? theta[s.ob3 + e] : 0.f;
+    sw[L.osd + e] = e < s.O ? nrm[2 * s.D + e] : 1.f;
+  }
+  for (int e = t; e < 2 * s.D; e += nt) sw[L.mu + e] = nrm[e];
 }
 
 __device__ __forceinline__ float silu_f(float a, float* ds) {
@@ -102,246 +135,267 @@ __device__ __forceinline__ float silu_f(float a, float* ds) {
   return a * sg;
 }
 
-// Forward of one sample.  x(d) supplies input d; h1 and h2 (registers) receive
-// the hidden activations; with GRAD, s1[h] = silu'(a1_h) and s2[h] =
-// silu'(a2_h) are stored (shared memory); y(o) is handed to put_y.
-template <int H, bool GRAD, typename XF, typename YF>
-__device__ __forceinline__ void mlp_forward(const MlpShape& s, const float* __restrict__ sw,
-                                            XF x, float (&h1)[H], float (&h2)[H], float* s1,
-                                            float* s2, YF put_y) {
-  const float* W1T = sw;
-  const float* W2 = W1T + s.D * H;
-  const float* W3 = W2 + H * H;
-  const float* b1 = W3 + s.O * H;
-  const float* b2 = b1 + H;
-  const float* b3 = b2 + H;
+// acc += W^T x for N consecutive outputs (pairs in packed FP32x2): x is the
+// sample's input row, w the first of its N columns of the input-major weights.
+template <int N>
+__device__ __forceinline__ void dense(float2 (&acc)[N / 2], const float* x, int nin,
+                                      const float* w, int ldw) {
+#pragma unroll 4
+  for (int i = 0; i < nin; ++i) {
+    const float2 xi = make_float2(x[i], x[i]);
+    if constexpr (N % 4 == 0) {
 #pragma unroll
-  for (int h = 0; h < H; ++h) h1[h] = b1[h];
-  for (int d = 0; d < s.D; ++d) {
-    const float xd = x(d);
-    const float4* w = reinterpret_cast<const float4*>(W1T + d * H);
+      for (int q = 0; q < N / 4; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(w + i * ldw + 4 * q);
+        acc[2 * q] = __ffma2_rn(xi, make_float2(v.x, v.y), acc[2 * q]);
+        acc[2 * q + 1] = __ffma2_rn(xi, make_float2(v.z, v.w), acc[2 * q + 1]);
+      }
+    } else {
 #pragma unroll
-    for (int q = 0; q < H / 4; ++q) {
-      const float4 wv = w[q];
-      h1[4 * q] = fmaf(wv.x, xd, h1[4 * q]);
-      h1[4 * q + 1] = fmaf(wv.y, xd, h1[4 * q + 1]);
-      h1[4 * q + 2] = fmaf(wv.z, xd, h1[4 * q + 2]);
-      h1[4 * q + 3] = fmaf(wv.w, xd, h1[4 * q + 3]);
+      for (int q = 0; q < N / 2; ++q)
+        acc[q] = __ffma2_rn(xi, *reinterpret_cast<const float2*>(w + i * ldw + 2 * q), acc[q]);
     }
   }
+}
+
+// One hidden layer of the CTA's samples: this thread's quarter of the outputs of
+// its sample; with ds, silu' goes there.
+template <int H>
+__device__ __forceinline__ void hidden(const float* x, int nin, const float* w, const float* b,
+                                       int part, float* out, float* ds) {
+  constexpr int N = H / kParts;
+  float2 acc[N / 2];
 #pragma unroll
-  for (int h = 0; h < H; ++h) {
-    float ds;
-    h1[h] = silu_f(h1[h], &ds);
-    if (GRAD) s1[h] = ds;
+  for (int q = 0; q < N / 2; ++q) acc[q] = *reinterpret_cast<const float2*>(b + part * N + 2 * q);
+  dense<N>(acc, x, nin, w + part * N, H);
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    float d;
+    out[part * N + q] = silu_f((q & 1) ? acc[q / 2].y : acc[q / 2].x, &d);
+    if (ds) ds[part * N + q] = d;
   }
+}
+
+// The output layer: put(o, y) for this thread's quarter of the OP outputs.
+template <typename Put>
+__device__ __forceinline__ void outputs(const float* x, int nin, const float* w, const float* b,
+                                        int OP, int O, int part, Put put) {
+  auto run = [&](auto Nc) {
+    constexpr int N = decltype(Nc)::value;
+    float2 acc[N / 2];
 #pragma unroll
-  for (int h = 0; h < H; ++h) {
-    const float4* w = reinterpret_cast<const float4*>(W2 + h * H);
-    float acc = b2[h];
+    for (int q = 0; q < N / 2; ++q) acc[q] = *reinterpret_cast<const float2*>(b + part * N + 2 * q);
+    dense<N>(acc, x, nin, w + part * N, OP);
 #pragma unroll
-    for (int q = 0; q < H / 4; ++q) {
-      const float4 wv = w[q];
-      acc = fmaf(wv.x, h1[4 * q], acc);
-      acc = fmaf(wv.y, h1[4 * q + 1], acc);
-      acc = fmaf(wv.z, h1[4 * q + 2], acc);
-      acc = fmaf(wv.w, h1[4 * q + 3], acc);
-    }
-    float ds;
-    h2[h] = silu_f(acc, &ds);
-    if (GRAD) s2[h] = ds;
-  }
-  for (int o = 0; o < s.O; ++o) {
-    const float4* w = reinterpret_cast<const float4*>(W3 + o * H);
-    float acc = b3[o];
-#pragma unroll
-    for (int q = 0; q < H / 4; ++q) {
-      const float4 wv = w[q];
-      acc = fmaf(wv.x, h2[4 * q], acc);
-      acc = fmaf(wv.y, h2[4 * q + 1], acc);
-      acc = fmaf(wv.z, h2[4 * q + 2], acc);
-      acc = fmaf(wv.w, h2[4 * q + 3], acc);
-    }
-    put_y(o, acc);
+    for (int q = 0; q < N; ++q)
+      if (part * N + q < O) put(part * N + q, (q & 1) ? acc[q / 2].y : acc[q / 2].x);
+  };
+  switch (OP) {
+    case 8: run(std::integral_constant<int, 2>()); break;
+    case 16: run(std::integral_constant<int, 4>()); break;
+    case 24: run(std::integral_constant<int, 6>()); break;
+    default: run(std::integral_constant<int, 8>()); break;
   }
 }
 
 // ---------------------------------------------------------------------------
-// Training: forward + backward of NS samples per CTA, per-CTA partial gradient
+// Training: forward + backward of NS (128, 64 or 32) samples per CTA of 4 NS threads,
+// per-CTA partial gradient
 // ---------------------------------------------------------------------------
 // Sample row in shared memory (pitch odd): [x (D) | h1 (H) | ga1 (H) | h2 (H) |
 // ga2 (H) | gy (O)].
+
+// Gradient tile of one layer: rows r0 .. r0 + NR - 1 (activations at column ca of
+// the sample rows) x columns lane, lane + 32, ... < ncol (at column cb), and the
+// bias gradient (the plain sum of the rows) of those rows.
+template <int NR>
+__device__ __forceinline__ void grad_tile(const float* act, int pitch, int cnt, int ca, int cb,
+                                          int ncol, int r0, int nrow, int lane, float* out,
+                                          float* outb) {
+  for (int c0 = 0; c0 < ncol; c0 += 96) {
+    float acc[NR][3], sum[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      sum[r] = 0.f;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) acc[r][j] = 0.f;
+    }
+    // lanes past the last column read column 0 and write nothing
+    int cj[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) cj[j] = cb + (c0 + lane + 32 * j < ncol ? c0 + lane + 32 * j : 0);
+#pragma unroll 2
+    for (int n = 0; n < cnt; ++n) {
+      const float* row = act + n * pitch;
+      float bv[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) bv[j] = c0 + 32 * j < ncol ? row[cj[j]] : 0.f;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const float av = row[ca + min(r0 + r, nrow - 1)];
+        sum[r] += av;
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          if (c0 + 32 * j < ncol) acc[r][j] = fmaf(av, bv[j], acc[r][j]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (r0 + r < nrow) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          if (c0 + lane + 32 * j < ncol) out[(size_t)(r0 + r) * ncol + c0 + lane + 32 * j] = acc[r][j];
+        if (c0 == 0 && lane == 0) outb[r0 + r] = sum[r];
+      }
+  }
+}
+
+// This thread's quarter of the gradient with respect to a layer's inputs, times
+// silu': sum over the layer's n outputs (in order) of their gradients g times
+// the input-major weights' row of the input.
+template <int H, int NMAX>
+__device__ __forceinline__ void back_layer(const float* g, int n, const float* wT, int ldw,
+                                           int part, float* ds) {
+  constexpr int N = H / kParts;
+  float gr[NMAX];
+#pragma unroll
+  for (int h = 0; h < NMAX; ++h) gr[h] = h < n ? g[h] : 0.f;
+#pragma unroll 4
+  for (int q = 0; q < N; ++q) {
+    const float4* w = reinterpret_cast<const float4*>(wT + (part * N + q) * ldw);
+    float acc = 0.f;
+#pragma unroll
+    for (int h = 0; h < NMAX; h += 4)
+      if (h < n) {  // zero weights and gradients past n add nothing
+        const float4 v = w[h / 4];
+        acc = fmaf(v.x, gr[h], acc);
+        acc = fmaf(v.y, gr[h + 1], acc);
+        acc = fmaf(v.z, gr[h + 2], acc);
+        acc = fmaf(v.w, gr[h + 3], acc);
+      }
+    ds[part * N + q] *= acc;
+  }
+}
+
 template <int H>
-__global__ void __launch_bounds__(128) mlp_train_kernel(MlpShape s, const float* __restrict__ theta,
-                                                        const __nv_bfloat16* __restrict__ wb,
-                                                        const float* __restrict__ nrm,
-                                                        const float* __restrict__ X,
-                                                        const float* __restrict__ T,
-                                                        const int* __restrict__ perm, int n0,
-                                                        int nb, float inv_norm, int pitch,
-                                                        float* part, double* lossp) {
+__global__ void __launch_bounds__(512)
+mlp_train_kernel(MlpShape s, const float* __restrict__ theta, const __nv_bfloat16* __restrict__ wb,
+                 const float* __restrict__ nrm, const float* __restrict__ X,
+                 const float* __restrict__ T, const int* __restrict__ perm, int n0, int nb,
+                 float inv_norm, int pitch, float* part_out, double* lossp) {
   extern __shared__ __align__(16) float smem_f[];
+  const NetSmem L(s);
   float* sw = smem_f;
-  float* act = sw + ((wblock_floats(s) + 3) & ~3);
-  __shared__ double red[128];
-  const int NS = blockDim.x;
-  const int tid = threadIdx.x;
+  float* act = sw + L.end;
+  __shared__ double red[512 / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int NS = blockDim.x / kParts;
+  const int smp = tid % NS, part = tid / NS;
   const int base = blockIdx.x * NS;
   const int cnt = min(NS, nb - base);
-  load_weights(s, wb, theta, nrm, sw);
+  load_weights(s, L, wb, theta, nrm, sw);
   __syncthreads();
-  const float* mu = sw + norm_offset(s);
-  const float* isd = mu + s.D;
-  const float* osd = isd + s.D;
-  // stage the normalised inputs of the CTA's samples (coalesced)
-  for (int e = tid; e < NS * s.D; e += NS) {
-    const int r = e / s.D, c = e - r * s.D;
-    float v = 0.f;
-    if (r < cnt) {
-      const int n = n0 + base + r;
-      const int src = perm ? perm[n] : n;
-      v = (X[(size_t)src * s.D + c] - mu[c]) * isd[c];
-    }
-    act[r * pitch + c] = v;
+  // stage the normalised inputs of the CTA's samples, a warp per row (coalesced)
+  for (int r = warp; r < NS; r += nw) {
+    int src = 0;
+    if (r < cnt) src = perm ? perm[n0 + base + r] : n0 + base + r;
+    for (int c = lane; c < s.D; c += 32)
+      act[r * pitch + c] =
+          r < cnt ? (X[(size_t)src * s.D + c] - sw[L.mu + c]) * sw[L.isd + c] : 0.f;
   }
   __syncthreads();
-  float* row = act + tid * pitch;
+  float* row = act + smp * pitch;
   float* rh1 = row + s.D;
   float* rg1 = rh1 + H;
   float* rh2 = rg1 + H;
   float* rg2 = rh2 + H;
   float* rgy = rg2 + H;
-  double sq = 0.0;
-  if (tid < cnt) {
-    const int n = n0 + base + tid;
-    const int src = perm ? perm[n] : n;
-    const float* t = T + (size_t)src * s.O;
-    float h1[H], h2[H];
-    // silu'(a1) and silu'(a2) go to the ga1 and ga2 slots, overwritten below
-    mlp_forward<H, true>(s, sw, [&](int d) { return row[d]; }, h1, h2, rg1, rg2,
-                         [&](int o, float y) {
-                           const float r = y - t[o] / osd[o];
-                           sq += (double)r * r;
-                           rgy[o] = 2.f * r * inv_norm;
-                         });
-#pragma unroll
-    for (int i = 0; i < H; ++i) {
-      rh1[i] = h1[i];
-      rh2[i] = h2[i];
-    }
-    // backward through layer 3: gh2 = W3^T gy, ga2 = gh2 * silu'(a2)
-    const float* W3 = sw + s.D * H + H * H;
-    const float* W2 = sw + s.D * H;
-    float g[H];
-#pragma unroll
-    for (int i = 0; i < H; ++i) g[i] = 0.f;
-    for (int o = 0; o < s.O; ++o) {
-      const float go = rgy[o];
-      const float4* w = reinterpret_cast<const float4*>(W3 + o * H);
-#pragma unroll
-      for (int q = 0; q < H / 4; ++q) {
-        const float4 wv = w[q];
-        g[4 * q] = fmaf(wv.x, go, g[4 * q]);
-        g[4 * q + 1] = fmaf(wv.y, go, g[4 * q + 1]);
-        g[4 * q + 2] = fmaf(wv.z, go, g[4 * q + 2]);
-        g[4 * q + 3] = fmaf(wv.w, go, g[4 * q + 3]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < H; ++i) {
-      g[i] *= rg2[i];
-      rg2[i] = g[i];
-    }
-    // layer 2: gh1 = W2^T ga2, ga1 = gh1 * silu'(a1)
-#pragma unroll
-    for (int i = 0; i < H; ++i) h2[i] = 0.f;  // reused as gh1
-#pragma unroll
-    for (int h = 0; h < H; ++h) {
-      const float gh = g[h];
-      const float4* w = reinterpret_cast<const float4*>(W2 + h * H);
-#pragma unroll
-      for (int q = 0; q < H / 4; ++q) {
-        const float4 wv = w[q];
-        h2[4 * q] = fmaf(wv.x, gh, h2[4 * q]);
-        h2[4 * q + 1] = fmaf(wv.y, gh, h2[4 * q + 1]);
-        h2[4 * q + 2] = fmaf(wv.z, gh, h2[4 * q + 2]);
-        h2[4 * q + 3] = fmaf(wv.w, gh, h2[4 * q + 3]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < H; ++i) rg1[i] = h2[i] * rg1[i];
-  } else {
-    for (int c = s.D; c < s.D + 4 * H + s.O; ++c) row[c] = 0.f;
-  }
-  red[tid] = sq;
+  // silu'(a1) and silu'(a2) go to the ga1 and ga2 columns, overwritten below
+  hidden<H>(row, s.D, sw + L.W1T, sw + L.b1, part, rh1, rg1);
   __syncthreads();
-  // weight gradients summed over the CTA's samples
-  float* out = part + (size_t)blockIdx.x * s.P;
-  for (int e = tid; e < s.P; e += NS) {
-    int ca, cb = -1;
-    if (e < s.ob1) {
-      const int h = e / s.D, d = e - h * s.D;
-      ca = s.D + H + h;
-      cb = d;
-    } else if (e < s.oW2) {
-      ca = s.D + H + (e - s.ob1);
-    } else if (e < s.ob2) {
-      const int k = e - s.oW2, h = k / H, i = k - h * H;
-      ca = s.D + 3 * H + h;
-      cb = s.D + i;
-    } else if (e < s.oW3) {
-      ca = s.D + 3 * H + (e - s.ob2);
-    } else if (e < s.ob3) {
-      const int k = e - s.oW3, o = k / H, i = k - o * H;
-      ca = s.D + 4 * H + o;
-      cb = s.D + 2 * H + i;
-    } else {
-      ca = s.D + 4 * H + (e - s.ob3);
-    }
-    float acc = 0.f;
-    if (cb >= 0) {
-      for (int n = 0; n < cnt; ++n) acc = fmaf(act[n * pitch + ca], act[n * pitch + cb], acc);
-    } else {
-      for (int n = 0; n < cnt; ++n) acc += act[n * pitch + ca];
-    }
-    out[e] = acc;
+  hidden<H>(rh1, H, sw + L.W2T, sw + L.b2, part, rh2, rg2);
+  __syncthreads();
+  double sq = 0.0;
+  {
+    const int n = n0 + base + smp;
+    const int src = smp < cnt ? (perm ? perm[n] : n) : 0;
+    const float* t = T + (size_t)src * s.O;
+    outputs(rh2, H, sw + L.W3T, sw + L.b3, o_pad(s), s.O, part, [&](int o, float y) {
+      const float r = smp < cnt ? y - t[o] / sw[L.osd + o] : 0.f;
+      sq += (double)r * r;
+      rgy[o] = 2.f * r * inv_norm;
+    });
   }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if (lane == 0) red[warp] = sq;
+  __syncthreads();
+  // layer 3: gh2 = W3^T gy, ga2 = gh2 * silu'(a2); layer 2 likewise
+  back_layer<H, kMaxO>(rgy, s.O, sw + L.W3T, o_pad(s), part, rg2);
+  __syncthreads();
+  back_layer<H, H>(rg2, H, sw + L.W2T, H, part, rg1);
+  __syncthreads();
+  // weight gradients summed over the CTA's samples in their order: four rows per
+  // warp and pass
+  float* out = part_out + (size_t)blockIdx.x * s.P;
+  for (int r0 = 4 * warp; r0 < H; r0 += 4 * nw)
+    grad_tile<4>(act, pitch, cnt, s.D + H, 0, s.D, r0, H, lane, out + s.oW1, out + s.ob1);
+  for (int r0 = 4 * warp; r0 < H; r0 += 4 * nw)
+    grad_tile<4>(act, pitch, cnt, s.D + 3 * H, s.D, H, r0, H, lane, out + s.oW2, out + s.ob2);
+  for (int r0 = 2 * warp; r0 < s.O; r0 += 2 * nw)
+    grad_tile<2>(act, pitch, cnt, s.D + 4 * H, s.D + 2 * H, H, r0, s.O, lane, out + s.oW3,
+                 out + s.ob3);
   if (tid == 0) {
     double t = 0.0;
-    for (int i = 0; i < NS; ++i) t += red[i];
+    for (int i = 0; i < nw; ++i) t += red[i];
     lossp[blockIdx.x] = t;
   }
 }
 
-__global__ void mlp_reduce_kernel(const float* __restrict__ part, int nblk, int P, float* grad,
-                                  const double* __restrict__ lossp, double loss_scale,
-                                  double* loss_acc) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// Sum of the CTAs' partial gradients in their order (deterministic) and, with
+// adam, the parameter update.
+struct AdamStep {
+  float* theta;
+  float* m;
+  float* v;
+  __nv_bfloat16* wb;
+  float lr, c1, c2;
+};
+
+constexpr int kRedThreads = 64;  // few per CTA, so that every SM has some
+
+__global__ void __launch_bounds__(kRedThreads)
+mlp_reduce_kernel(const float* __restrict__ part, int nblk, int P, float* grad,
+                  const double* __restrict__ lossp, double loss_scale, double* loss_acc,
+                  AdamStep ad) {
+  const int e = blockIdx.x * kRedThreads + threadIdx.x;
   if (e < P) {
-    float acc = 0.f;
-    for (int b = 0; b < nblk; ++b) acc += part[(size_t)b * P + e];
-    grad[e] = acc;
+    float g = 0.f;
+    int b = 0;
+    for (; b + 16 <= nblk; b += 16) {
+      float x[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) x[u] = part[(size_t)(b + u) * P + e];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) g += x[u];
+    }
+    for (; b < nblk; ++b) g += part[(size_t)b * P + e];
+    grad[e] = g;
+    if (ad.theta) {
+      const float mm = 0.9f * ad.m[e] + 0.1f * g;
+      const float vv = 0.999f * ad.v[e] + 0.001f * g * g;
+      ad.m[e] = mm;
+      ad.v[e] = vv;
+      const float th = ad.theta[e] - ad.lr * (mm * ad.c1) / (sqrtf(vv * ad.c2) + 1e-8f);
+      ad.theta[e] = th;
+      ad.wb[e] = __float2bfloat16_rn(th);
+    }
   }
-  if (e == 0) {
+  if (e == P) {  // one thread past the parameters (the grid covers P + 1)
     double t = 0.0;
     for (int b = 0; b < nblk; ++b) t += lossp[b];
     *loss_acc += t * loss_scale;
   }
-}
-
-__global__ void mlp_adam_kernel(float* theta, const float* __restrict__ grad, float* m, float* v,
-                                int P, float lr, float c1, float c2, MlpShape s,
-                                __nv_bfloat16* wb) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= P) return;
-  const float g = grad[e];
-  const float mm = 0.9f * m[e] + 0.1f * g;
-  const float vv = 0.999f * v[e] + 0.001f * g * g;
-  m[e] = mm;
-  v[e] = vv;
-  const float th = theta[e] - lr * (mm * c1) / (sqrtf(vv * c2) + 1e-8f);
-  theta[e] = th;
-  wb[e] = __float2bfloat16_rn(th);
 }
 
 __global__ void mlp_round_kernel(const float* __restrict__ theta, int P, __nv_bfloat16* wb) {
@@ -349,35 +403,59 @@ __global__ void mlp_round_kernel(const float* __restrict__ theta, int P, __nv_bf
   if (e < P) wb[e] = __float2bfloat16_rn(theta[e]);
 }
 
-// Inference on given inputs: thread per sample, inputs staged through smem.
+// Sample row of the inference kernels (pitch odd): [x, then h2 (max(D, H)) | h1, then
+// the outputs (max(H, O))].
+__host__ __device__ inline int infer_h1(const MlpShape& s) { return s.D > s.H ? s.D : s.H; }
+__host__ __device__ inline int infer_pitch(const MlpShape& s) {
+  return (infer_h1(s) + (s.H > s.O ? s.H : s.O)) | 1;
+}
+__host__ __device__ inline size_t infer_smem(const MlpShape& s) {
+  return sizeof(float) * ((size_t)NetSmem(s).end + (size_t)kNS * infer_pitch(s));
+}
+
+// Forward of the CTA's staged samples.
+template <int H, typename Put>
+__device__ __forceinline__ void forward_rows(const MlpShape& s, const NetSmem& L, const float* sw,
+                                             float* row, int part, Put put) {
+  float* r1 = row + infer_h1(s);
+  hidden<H>(row, s.D, sw + L.W1T, sw + L.b1, part, r1, nullptr);
+  __syncthreads();
+  hidden<H>(r1, H, sw + L.W2T, sw + L.b2, part, row, nullptr);
+  __syncthreads();
+  outputs(row, H, sw + L.W3T, sw + L.b3, o_pad(s), s.O, part, put);
+  __syncthreads();
+}
+
+// Inference on given inputs.
 template <int H>
-__global__ void __launch_bounds__(128) mlp_infer_kernel(MlpShape s, const float* __restrict__ theta,
-                                                        const __nv_bfloat16* __restrict__ wb,
-                                                        const float* __restrict__ nrm,
-                                                        const float* __restrict__ X, int n,
-                                                        int pitch, float* Y) {
+__global__ void __launch_bounds__(kNetThreads)
+mlp_infer_kernel(MlpShape s, const float* __restrict__ theta, const __nv_bfloat16* __restrict__ wb,
+                 const float* __restrict__ nrm, const float* __restrict__ X, int n, float* Y) {
   extern __shared__ __align__(16) float smem_f[];
+  const NetSmem L(s);
   float* sw = smem_f;
-  float* xs = sw + ((wblock_floats(s) + 3) & ~3);
-  const int tid = threadIdx.x, NS = blockDim.x;
-  const int base = blockIdx.x * NS;
-  const int cnt = min(NS, n - base);
-  load_weights(s, wb, theta, nrm, sw);
+  float* act = sw + L.end;
+  const int pitch = infer_pitch(s);
+  const int tid = threadIdx.x;
+  load_weights(s, L, wb, theta, nrm, sw);
   __syncthreads();
-  const float* mu = sw + norm_offset(s);
-  const float* isd = mu + s.D;
-  const float* osd = isd + s.D;
-  for (int e = tid; e < NS * s.D; e += NS) {
-    const int r = e / s.D, c = e - r * s.D;
-    xs[r * pitch + c] = r < cnt ? (X[(size_t)(base + r) * s.D + c] - mu[c]) * isd[c] : 0.f;
+  for (int base = blockIdx.x * kNS; base < n; base += gridDim.x * kNS) {
+    const int cnt = min(kNS, n - base);
+    for (int r = tid >> 5; r < kNS; r += kNetThreads / 32)
+      for (int c = tid & 31; c < s.D; c += 32)
+        act[r * pitch + c] =
+            r < cnt ? (X[(size_t)(base + r) * s.D + c] - sw[L.mu + c]) * sw[L.isd + c] : 0.f;
+    __syncthreads();
+    float* row = act + (tid % kNS) * pitch;
+    const int oy = infer_h1(s);
+    forward_rows<H>(s, L, sw, row, tid / kNS,
+                    [&](int o, float y) { row[oy + o] = y * sw[L.osd + o]; });
+    for (int e = tid; e < cnt * s.O; e += kNetThreads) {
+      const int r = e / s.O, o = e - r * s.O;
+      Y[(size_t)base * s.O + e] = act[r * pitch + oy + o];
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  if (tid >= cnt) return;
-  const float* row = xs + tid * pitch;
-  float h1[H], h2[H];
-  float* y = Y + (size_t)(base + tid) * s.O;
-  mlp_forward<H, false>(s, sw, [&](int d) { return row[d]; }, h1, h2, nullptr, nullptr,
-                        [&](int o, float v) { y[o] = v * osd[o]; });
 }
 
 // ---------------------------------------------------------------------------
@@ -404,56 +482,98 @@ __device__ __forceinline__ void project_add(const ClosureConsts& cc, int V, cons
     out[v] = delta[v] - cc.w[v] * (c0 * cc.phi[v][0] + c1 * cc.phi[v][1] + c2 * cc.phi[v][2]);
 }
 
-// f_out = f_in + projected correction, thread per cell.
+// f_out = f_in + projected correction; four threads per cell.
 template <int H>
-__global__ void __launch_bounds__(128) closure_apply_kernel(MlpShape s, const float* __restrict__ theta,
-                                                            const __nv_bfloat16* __restrict__ wb,
-                                                            const float* __restrict__ nrm,
-                                                            const float* __restrict__ fin,
-                                                            float* fout, int Z, int ldz,
-                                                            float logtau, ClosureConsts cc) {
+__global__ void __launch_bounds__(kNetThreads)
+closure_apply_kernel(MlpShape s, const float* __restrict__ theta,
+                     const __nv_bfloat16* __restrict__ wb, const float* __restrict__ nrm,
+                     const float* __restrict__ fin, float* fout, int Z, int ldz, float logtau,
+                     ClosureConsts cc) {
   extern __shared__ __align__(16) float smem_f[];
+  __shared__ float lim[kParts][kNS];
+  const NetSmem L(s);
   float* sw = smem_f;
-  load_weights(s, wb, theta, nrm, sw);
+  float* act = sw + L.end;
+  const int pitch = infer_pitch(s);
+  const int V = s.O, part = threadIdx.x / kNS, smp = threadIdx.x % kNS;
+  load_weights(s, L, wb, theta, nrm, sw);
   __syncthreads();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= Z) return;
-  const int V = s.O;
-  const int cl = c > 0 ? c - 1 : 0, cr = c < Z - 1 ? c + 1 : Z - 1;
-  float n = 0.f;
-  for (int v = 0; v < V; ++v) n += fin[(size_t)v * ldz + c];
-  const float inv_n = 1.f / n;
-  const float* mu = sw + norm_offset(s);
-  const float* isd = mu + s.D;
-  const float* osd = isd + s.D;
-  // features: f_s, f_{s+1} - f_s, f_s - f_{s-1} (over n_s), log10 tau
-  auto x = [&](int d) {
-    float r;
-    if (d >= 3 * V) {
-      r = logtau;
-    } else {
-      const int blk = d / V, v = d - blk * V;
-      const float fc = fin[(size_t)v * ldz + c];
-      if (blk == 0) r = fc * inv_n;
-      else if (blk == 1) r = (fin[(size_t)v * ldz + cr] - fc) * inv_n;
-      else r = (fc - fin[(size_t)v * ldz + cl]) * inv_n;
+  const float* mu = sw + L.mu;
+  const float* isd = sw + L.isd;
+  for (int base = blockIdx.x * kNS; base < Z; base += gridDim.x * kNS) {
+    const bool live = base + smp < Z;
+    const int c = min(base + smp, Z - 1);
+    const int cl = c > 0 ? c - 1 : 0, cr = c < Z - 1 ? c + 1 : Z - 1;
+    float* row = act + smp * pitch;
+    // this thread's populations v = part + 4 j and their neighbours, all loads at
+    // once; kept for the limiter and the update
+    float fc[kMaxV4], fr[kMaxV4], fl[kMaxV4], np = 0.f;
+#pragma unroll
+    for (int j = 0; j < kMaxV4; ++j) {
+      const int v = part + kParts * j;
+      const float* f = fin + (size_t)v * ldz;
+      fc[j] = v < V ? f[c] : 0.f;
+      fr[j] = v < V ? f[cr] : 0.f;
+      fl[j] = v < V ? f[cl] : 0.f;
     }
-    return (r - mu[d]) * isd[d];
-  };
-  float h1[H], h2[H];
-  float delta[kMaxO], corr[kMaxO];
-  mlp_forward<H, false>(s, sw, x, h1, h2, nullptr, nullptr,
-                        [&](int o, float y) { delta[o] = n * osd[o] * y; });
-  project_add(cc, V, delta, corr);
-  // positivity limiter: scale the (conserving) correction so that no
-  // positive population loses more than kLimitTheta of itself
-  float alpha = 1.f;
-  for (int v = 0; v < V; ++v) {
-    const float f = fin[(size_t)v * ldz + c];
-    if (f > 0.f && corr[v] < 0.f) alpha = fminf(alpha, kLimitTheta * f / -corr[v]);
+#pragma unroll
+    for (int j = 0; j < kMaxV4; ++j) np += fc[j];
+    lim[part][smp] = np;
+    __syncthreads();
+    const float n = (lim[0][smp] + lim[1][smp]) + (lim[2][smp] + lim[3][smp]);
+    const float inv_n = 1.f / n;
+    // features: f_s, f_{s+1} - f_s, f_s - f_{s-1} (over n_s), log10 tau
+#pragma unroll
+    for (int j = 0; j < kMaxV4; ++j) {
+      const int v = part + kParts * j;
+      if (v < V) {
+        row[v] = (fc[j] * inv_n - mu[v]) * isd[v];
+        row[V + v] = ((fr[j] - fc[j]) * inv_n - mu[V + v]) * isd[V + v];
+        row[2 * V + v] = ((fc[j] - fl[j]) * inv_n - mu[2 * V + v]) * isd[2 * V + v];
+      }
+    }
+    if (part == 0) row[3 * V] = (logtau - mu[3 * V]) * isd[3 * V];
+    __syncthreads();
+    float* dl = row + infer_h1(s);
+    forward_rows<H>(s, L, sw, row, part,
+                    [&](int o, float y) { dl[o] = n * sw[L.osd + o] * y; });
+    // the correction without its component along the collision invariants
+    const float* delta = dl;
+    float b0 = 0.f, b1 = 0.f, b2 = 0.f;
+    for (int v = 0; v < V; ++v) {
+      b0 = fmaf(delta[v], cc.phi[v][0], b0);
+      b1 = fmaf(delta[v], cc.phi[v][1], b1);
+      b2 = fmaf(delta[v], cc.phi[v][2], b2);
+    }
+    const float c0 = cc.ginv[0] * b0 + cc.ginv[1] * b1 + cc.ginv[2] * b2;
+    const float c1 = cc.ginv[3] * b0 + cc.ginv[4] * b1 + cc.ginv[5] * b2;
+    const float c2 = cc.ginv[6] * b0 + cc.ginv[7] * b1 + cc.ginv[8] * b2;
+    auto corr = [&](int v) {
+      return delta[v] -
+             cc.w[v] * (c0 * cc.phi[v][0] + c1 * cc.phi[v][1] + c2 * cc.phi[v][2]);
+    };
+    // positivity limiter: scale the (conserving) correction so that no
+    // positive population loses more than kLimitTheta of itself
+    float alpha = 1.f;
+#pragma unroll
+    for (int j = 0; j < kMaxV4; ++j) {
+      const int v = part + kParts * j;
+      if (v < V) {
+        fr[j] = corr(v);
+        if (fc[j] > 0.f && fr[j] < 0.f) alpha = fminf(alpha, kLimitTheta * fc[j] / -fr[j]);
+      }
+    }
+    lim[part][smp] = alpha;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kParts; ++q) alpha = fminf(alpha, lim[q][smp]);
+#pragma unroll
+    for (int j = 0; j < kMaxV4; ++j) {
+      const int v = part + kParts * j;
+      if (live && v < V) fout[(size_t)v * ldz + c] = fc[j] + alpha * fr[j];
+    }
+    __syncthreads();
   }
-  for (int v = 0; v < V; ++v)
-    fout[(size_t)v * ldz + c] = fin[(size_t)v * ldz + c] + alpha * corr[v];
 }
 
 // Restriction, thread per cell: f_lo[k*Ql + i] = sum_j R[i][j] f_hi[k*Qh + j].
@@ -625,21 +745,31 @@ struct rslb_mlp {
 
 namespace {
 
+// CTAs of the inference kernels: each loads the weights once and walks groups of
+// kNS samples, so as many as fit the SMs at once.
+int net_grid(const MlpShape& s, int n) {
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
+    nsm = 152;
+  const int per = std::max(1, (int)(233472 / (infer_smem(s) + 2048)));  // 228 KB per SM
+  return std::min((n + kNS - 1) / kNS, per * nsm);
+}
+
 int mlp_pitch(const MlpShape& s) {
   int p = s.D + 4 * s.H + s.O;
   return (p % 2) ? p : p + 1;
 }
 
-int train_ns(const MlpShape& s) {
-  for (int ns = 128; ns >= 32; ns /= 2) {
-    const size_t b = sizeof(float) * (size_t)(((wblock_floats(s) + 3) & ~3) + ns * mlp_pitch(s));
-    if (b <= (size_t)kSmemLimit) return ns;
-  }
-  return 0;
+size_t train_smem(const MlpShape& s, int ns) {
+  return sizeof(float) * ((size_t)NetSmem(s).end + (size_t)ns * mlp_pitch(s));
 }
 
-size_t train_smem(const MlpShape& s, int ns) {
-  return sizeof(float) * (size_t)(((wblock_floats(s) + 3) & ~3) + ns * mlp_pitch(s));
+// Samples per CTA of the training kernel (0: the network does not fit).
+int train_ns(const MlpShape& s) {
+  for (int ns = 128; ns >= 32; ns /= 2)
+    if (train_smem(s, ns) <= (size_t)kSmemLimit) return ns;
+  return 0;
 }
 
 template <typename F>
@@ -662,26 +792,23 @@ void mlp_free(rslb_mlp* m) {
 }
 
 cudaError_t set_smem_attrs(const MlpShape& s) {
-  const int ns = train_ns(s);
-  const int tsm = (int)train_smem(s, ns);
   return dispatch_h(s.H, [&](auto Hc) {
     constexpr int H = decltype(Hc)::value;
-    cudaError_t e = cudaFuncSetAttribute(mlp_train_kernel<H>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, tsm);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(mlp_infer_kernel<H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmemLimit);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(closure_apply_kernel<H>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
-    return e;
+    for (const void* f : {(const void*)mlp_train_kernel<H>, (const void*)mlp_infer_kernel<H>,
+                          (const void*)closure_apply_kernel<H>}) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
   });
 }
 
 // Gradient of the mean-squared loss over samples [n0, n0 + nb) of the
-// (permuted) data into m->grad; adds loss * loss_scale to m->loss_acc.
+// (permuted) data into m->grad; adds loss * loss_scale to m->loss_acc; with adam,
+// the update follows in the same kernel as the sum of the partials.
 cudaError_t mlp_batch_grad(rslb_mlp* m, const float* X, const float* T, const int* perm, int n0,
-                           int nb, double loss_scale) {
+                           int nb, double loss_scale, const AdamStep& adam) {
   const MlpShape& s = m->s;
   const int ns = train_ns(s);
   const int nblk = (nb + ns - 1) / ns;
@@ -696,17 +823,16 @@ cudaError_t mlp_batch_grad(rslb_mlp* m, const float* X, const float* T, const in
     m->part_blocks = nblk;
   }
   const float inv_norm = 1.f / ((float)nb * (float)s.O);
-  const size_t smem = train_smem(s, ns);
   cudaError_t e = dispatch_h(s.H, [&](auto Hc) {
     constexpr int H = decltype(Hc)::value;
-    mlp_train_kernel<H><<<nblk, ns, smem, m->stream>>>(s, m->theta, m->wb, m->norm, X, T, perm,
-                                                       n0, nb,
-                                                       inv_norm, mlp_pitch(s), m->part, m->lossp);
+    mlp_train_kernel<H><<<nblk, ns * kParts, train_smem(s, ns), m->stream>>>(
+        s, m->theta, m->wb, m->norm, X, T, perm, n0, nb, inv_norm, mlp_pitch(s), m->part,
+        m->lossp);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
-  mlp_reduce_kernel<<<(s.P + 255) / 256, 256, 0, m->stream>>>(m->part, nblk, s.P, m->grad,
-                                                               m->lossp, loss_scale, m->loss_acc);
+  mlp_reduce_kernel<<<s.P / kRedThreads + 1, kRedThreads, 0, m->stream>>>(
+      m->part, nblk, s.P, m->grad, m->lossp, loss_scale, m->loss_acc, adam);
   return cudaGetLastError();
 }
 
@@ -850,14 +976,11 @@ extern "C" int rslb_mlp_forward(rslb_mlp* m, const float* X, int n, float* Y) {
   if (!m || !X || !Y || n < 0) return set_error(RSLB_ERR_ARG, "rslb_mlp_forward: bad arguments");
   if (n == 0) return RSLB_OK;
   const MlpShape& s = m->s;
-  const int ns = 128;
-  const int pitch = (s.D % 2) ? s.D : s.D + 1;
-  const size_t smem = sizeof(float) * (size_t)(((wblock_floats(s) + 3) & ~3) + ns * pitch);
+  const int grid = net_grid(s, n);
   cudaError_t e = dispatch_h(s.H, [&](auto Hc) {
     constexpr int H = decltype(Hc)::value;
-    mlp_infer_kernel<H><<<(n + ns - 1) / ns, ns, smem, m->stream>>>(s, m->theta, m->wb, m->norm,
-                                                                    X, n,
-                                                                    pitch, Y);
+    mlp_infer_kernel<H><<<grid, kNetThreads, infer_smem(s), m->stream>>>(s, m->theta, m->wb,
+                                                                        m->norm, X, n, Y);
     return cudaGetLastError();
   });
   return e == cudaSuccess ? RSLB_OK : cuda_error(e, "rslb_mlp_forward");
@@ -869,7 +992,7 @@ extern "C" int rslb_mlp_loss_grad(rslb_mlp* m, const float* X, const float* T, i
   if (!m || !X || !T || n < 1) return set_error(RSLB_ERR_ARG, "rslb_mlp_loss_grad: bad arguments");
   cudaError_t e = cudaMemsetAsync(m->loss_acc, 0, sizeof(double), m->stream);
   if (e == cudaSuccess)
-    e = mlp_batch_grad(m, X, T, nullptr, 0, n, 1.0 / ((double)n * m->s.O));
+    e = mlp_batch_grad(m, X, T, nullptr, 0, n, 1.0 / ((double)n * m->s.O), AdamStep{});
   double L = 0.0;
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(&L, m->loss_acc, sizeof(double), cudaMemcpyDeviceToHost, m->stream);
@@ -896,7 +1019,6 @@ extern "C" int rslb_mlp_train(rslb_mlp* m, const float* X, const float* T, int n
   std::vector<int> perm(n);
   uint64_t st = seed ^ 0x13198A2E03707344ull;
   cudaError_t e = cudaSuccess;
-  const int P = m->s.P;
   for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
     for (int i = 0; i < n; ++i) perm[i] = i;
     for (int i = n - 1; i > 0; --i) std::swap(perm[i], perm[splitmix(st) % (uint64_t)(i + 1)]);
@@ -905,15 +1027,11 @@ extern "C" int rslb_mlp_train(rslb_mlp* m, const float* X, const float* T, int n
     if (e == cudaSuccess) e = cudaMemsetAsync(m->loss_acc, 0, sizeof(double), m->stream);
     for (int n0 = 0; n0 < n && e == cudaSuccess; n0 += batch) {
       const int nb = std::min(batch, n - n0);
-      e = mlp_batch_grad(m, X, T, m->perm, n0, nb, 1.0 / ((double)n * m->s.O));
-      if (e != cudaSuccess) break;
       m->adam_t += 1;
       const double c1 = 1.0 / (1.0 - std::pow(0.9, (double)m->adam_t));
       const double c2 = 1.0 / (1.0 - std::pow(0.999, (double)m->adam_t));
-      mlp_adam_kernel<<<(P + 255) / 256, 256, 0, m->stream>>>(m->theta, m->grad, m->m, m->v, P,
-                                                              (float)lr, (float)c1, (float)c2,
-                                                              m->s, m->wb);
-      e = cudaGetLastError();
+      e = mlp_batch_grad(m, X, T, m->perm, n0, nb, 1.0 / ((double)n * m->s.O),
+                         AdamStep{m->theta, m->m, m->v, m->wb, (float)lr, (float)c1, (float)c2});
     }
     if (e == cudaSuccess && epoch_loss) {
       // the stream-ordered copy lands before the host buffer is read at the sync below
@@ -1044,23 +1162,28 @@ extern "C" int rslb_closure_step(rslb_handle* lo, rslb_mlp* m, double tau, int n
   int rc = closure_consts(vl.Q_xi, vl.Q_L, &cc);
   if (rc) return set_error(rc, "rslb_closure_step: low-order set too large");
   const MlpShape& s = m->s;
-  const size_t smem = sizeof(float) * (size_t)((wblock_floats(s) + 3) & ~3);
-  const int TB = 128, G = (vl.Z + TB - 1) / TB;
+  const size_t smem = infer_smem(s);
+  const int G = net_grid(s, vl.Z);
   const float lt = (float)std::log10(tau);
-  for (int n = 0; n < nsteps; ++n) {
-    rc = rslb_step(lo, 1);
-    if (rc) return rc;
-    cudaError_t e = dispatch_h(s.H, [&](auto Hc) {
-      constexpr int H = decltype(Hc)::value;
-      closure_apply_kernel<H><<<G, TB, smem, vl.stream>>>(s, m->theta, m->wb, m->norm,
-                                                          (const float*)vl.F0, (float*)vl.F1,
-                                                          vl.Z, vl.ldz, lt, cc);
-      return cudaGetLastError();
-    });
+  // the correction reads its neighbours, so it writes the other buffer, which
+  // then holds the state: the two change roles every step and only an odd
+  // count ends with a copy
+  float* F[2] = {(float*)vl.F0, (float*)vl.F1};
+  int cur = 0;
+  cudaError_t e = cudaSuccess;
+  for (int n = 0; n < nsteps && e == cudaSuccess; ++n, cur ^= 1) {
+    e = sod_step_in(lo, cur);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(vl.F0, vl.F1, sizeof(float) * (size_t)vl.V * vl.ldz,
-                          cudaMemcpyDeviceToDevice, vl.stream);
-    if (e != cudaSuccess) return cuda_error(e, "rslb_closure_step");
+      e = dispatch_h(s.H, [&](auto Hc) {
+        constexpr int H = decltype(Hc)::value;
+        closure_apply_kernel<H><<<G, kNetThreads, smem, vl.stream>>>(
+            s, m->theta, m->wb, m->norm, F[cur], F[cur ^ 1], vl.Z, vl.ldz, lt, cc);
+        return cudaGetLastError();
+      });
   }
+  if (e == cudaSuccess && cur)
+    e = cudaMemcpyAsync(vl.F0, vl.F1, sizeof(float) * (size_t)vl.V * vl.ldz,
+                        cudaMemcpyDeviceToDevice, vl.stream);
+  if (e != cudaSuccess) return cuda_error(e, "rslb_closure_step");
   return RSLB_OK;
 }

@@ -717,6 +717,26 @@ extern "C" int rslb_set_state(rslb_handle* h, const void* f, int on_device) {
 }
 
 namespace rslb {
+// One RK3 step whose state is in buffer `cur` (0 or 1) instead of F0; the other of
+// the two and F2 hold the stages.
+cudaError_t sod_step_in(rslb_handle* h, int cur) {
+  float* A = (float*)h->F[cur];
+  float* B = (float*)h->F[1 - cur];
+  float* C = (float*)h->F[2];
+  const SodTables<float> tb = tables_of<float>(h);
+  const float* fin[3] = {A, B, C};
+  float* fout[3] = {B, C, A};
+  for (int stage = 0; stage < 3; ++stage) {
+    const cudaError_t e = sod_stage_launch<float>(h->launch, h->geom, tb, h->t_rowv, h->nneg,
+                                                  fin[stage], A, fout[stage], stage, h->d_err,
+                                                  h->stream);
+    if (e != cudaSuccess) return e;
+  }
+  h->steps += 1;
+  h->t = h->steps * h->cfg.dt;
+  return cudaSuccess;
+}
+
 int sod_view(rslb_handle* h, SodView* v) {
   if (!h || !v) return RSLB_ERR_ARG;
   v->Z = h->cfg.Z;

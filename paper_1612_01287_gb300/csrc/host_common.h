@@ -26,5 +26,6 @@ struct SodView {
   double dt;
 };
 int sod_view(rslb_handle* h, SodView* v);
+cudaError_t sod_step_in(rslb_handle* h, int cur);  // FP32 handles
 
 }  // namespace rslb
