@@ -336,11 +336,10 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   if ((long long)V * (((long long)c.Z + 31) / 32 * 32) >= (1LL << 31))
     return set_error(RSLB_ERR_UNSUPPORTED,
                      "rslb_init: V x Z = %d x %d populations per buffer (limit 2^31)", V, c.Z);
-  std::vector<double> xj(Qx), wj(Qx), xk(QL), wk(QL), glt(kAeqTable), glw(kAeqTable);
+  std::vector<double> xj(Qx), wj(Qx), xk(QL), wk(QL), glt(kAeqNodes), glw(kAeqNodes);
   gauss_legendre_host(Qx, xj.data(), wj.data());
   gauss_laguerre2_host(QL, xk.data(), wk.data());
   gauss_legendre_host(kAeqNodes, glt.data(), glw.data());
-  gauss_legendre_host(kAeqNodesF32, glt.data() + kAeqNodes, glw.data() + kAeqNodes);
   const double dz = (c.z_max - c.z_min) / c.Z;
   double ximax = 0.0;
   for (double v : xj) ximax = std::fmax(ximax, std::fabs(v));
