@@ -282,9 +282,9 @@ typedef struct rslb_sod_batch rslb_sod_batch;
  * dt = t_end / ceil(t_end / dt_max) with dt_max = min(cfl dz / max|xi|,
  * dt_over_tau * tau), i.e. it reaches t_end exactly after its own number of
  * steps; a run with dt > 0 takes round(t_end / dt) steps of dt.  Runs are grouped by velocity
- * count; each group is advanced by one persistent launch per RK stage that
- * walks the tiles of its runs (runs with fewer steps drop out as they
- * finish).  With autotune, the tile kernel and CTAs per SM of each group are
+ * count; each group is advanced by one launch per RK stage that walks the
+ * tiles of its runs (runs with fewer steps drop out as they finish), the
+ * groups side by side on streams that fork from and join the caller's.  With autotune, the tile kernel and CTAs per SM of each group are
  * chosen by timing the candidates on the actual state.
  * Errors: RSLB_ERR_ARG, RSLB_ERR_UNSUPPORTED, RSLB_ERR_ALLOC, RSLB_ERR_CUDA.
  */
