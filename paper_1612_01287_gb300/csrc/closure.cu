@@ -40,6 +40,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "mod_range.h"
 #include "../../include/rslb.h"
 #include "host_common.h"
 
@@ -1021,7 +1022,8 @@ extern "C" int rslb_mlp_train(rslb_mlp* m, const float* X, const float* T, int n
   cudaError_t e = cudaSuccess;
   for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
     for (int i = 0; i < n; ++i) perm[i] = i;
-    for (int i = n - 1; i > 0; --i) std::swap(perm[i], perm[splitmix(st) % (uint64_t)(i + 1)]);
+    for (int i = n - 1; i > 0; --i)
+      std::swap(perm[i], perm[mod_range(splitmix(st), (uint32_t)i + 1)]);
     e = cudaMemcpyAsync(m->perm, perm.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice,
                         m->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->loss_acc, 0, sizeof(double), m->stream);
