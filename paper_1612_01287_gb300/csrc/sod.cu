@@ -264,15 +264,14 @@ __device__ __forceinline__ void weno_scale(float& s1, float& s2, float& s3) {
 }
 __device__ __forceinline__ void weno_scale(double& s1, double& s2, double& s3) {
   // the same by subtracting the exponent of the maximum from the high words
-  // (the indicators are >= 0, so their high words order like integers); a
-  // word that would fall below zero becomes a subnormal, whose square is 0.
-  // Indicators all below ~1e-231 are left alone: their squares vanish.
+  // (the indicators are >= 0, so their high words order like integers).  Words that
+  // would fall below zero, zero indicators and subnormal ones become subnormal:
+  // their squares are 0.
   const int h1 = __double2hiint(s1), h2 = __double2hiint(s2), h3 = __double2hiint(s3);
-  const int em = max(h1, max(h2, h3)) & 0x7FF00000;
-  const int sh = em < 0x10000000 ? 0 : em - 0x3FF00000;
-  s1 = __hiloint2double(max(h1 - sh, 0), __double2loint(s1));
-  s2 = __hiloint2double(max(h2 - sh, 0), __double2loint(s2));
-  s3 = __hiloint2double(max(h3 - sh, 0), __double2loint(s3));
+  const int sh = (max(h1, max(h2, h3)) & 0x7FF00000) - 0x3FF00000, least = max(sh, 0x00100000);
+  s1 = __hiloint2double(h1 < least ? 0 : h1 - sh, __double2loint(s1));
+  s2 = __hiloint2double(h2 < least ? 0 : h2 - sh, __double2loint(s2));
+  s3 = __hiloint2double(h3 < least ? 0 : h3 - sh, __double2loint(s3));
 }
 // num/den, 0 where den is below the smallest normal number (the reciprocals
 // flush subnormal inputs, and a vanishing denominator means a vanishing correction)
