@@ -98,7 +98,8 @@ constexpr int kMomCells32 = 64;  // 32 lanes x 2 cells
 __global__ void __launch_bounds__(kMomThreads, 4)
 sod_moments32_kernel(int Z, int ldz, int V, int Qx, const float4* __restrict__ w,
                      const float* __restrict__ f, double* out, int* err) {
-  __shared__ float2 part[kMomChunks][5][kMomCells32];  // [chunk][sum][cell] (hi, lo)
+  // [chunk][sum][cell] (hi, lo); a lane's two cells are accessed as one float4
+  __shared__ __align__(16) float2 part[kMomChunks][5][kMomCells32];
   const int chunk = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c0 = blockIdx.x * kMomCells32 + 2 * lane;  // first cell of the pair
   const bool active = c0 < ldz;                        // ldz is even: the pair fits
