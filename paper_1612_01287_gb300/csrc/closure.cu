@@ -41,6 +41,7 @@
 #include <vector>
 
 #include "mod_range.h"
+#include "swap_steps.h"
 #include "../../include/rslb.h"
 #include "host_common.h"
 
@@ -1168,24 +1169,24 @@ extern "C" int rslb_closure_step(rslb_handle* lo, rslb_mlp* m, double tau, int n
   const int G = net_grid(s, vl.Z);
   const float lt = (float)std::log10(tau);
   // the correction reads its neighbours, so it writes the other buffer, which
-  // then holds the state: the two change roles every step and only an odd
-  // count ends with a copy
+  // then holds the state: the two change roles every step
   float* F[2] = {(float*)vl.F0, (float*)vl.F1};
-  int cur = 0;
-  cudaError_t e = cudaSuccess;
-  for (int n = 0; n < nsteps && e == cudaSuccess; ++n, cur ^= 1) {
-    e = sod_step_in(lo, cur);
-    if (e == cudaSuccess)
-      e = dispatch_h(s.H, [&](auto Hc) {
-        constexpr int H = decltype(Hc)::value;
-        closure_apply_kernel<H><<<G, kNetThreads, smem, vl.stream>>>(
-            s, m->theta, m->wb, m->norm, F[cur], F[cur ^ 1], vl.Z, vl.ldz, lt, cc);
-        return cudaGetLastError();
+  const cudaError_t e = swap_steps(
+      nsteps, cudaSuccess,
+      [&](int cur) {
+        const cudaError_t es = sod_step_in(lo, cur);
+        if (es != cudaSuccess) return es;
+        return dispatch_h(s.H, [&](auto Hc) {
+          constexpr int H = decltype(Hc)::value;
+          closure_apply_kernel<H><<<G, kNetThreads, smem, vl.stream>>>(
+              s, m->theta, m->wb, m->norm, F[cur], F[cur ^ 1], vl.Z, vl.ldz, lt, cc);
+          return cudaGetLastError();
+        });
+      },
+      [&]() {
+        return cudaMemcpyAsync(vl.F0, vl.F1, sizeof(float) * (size_t)vl.V * vl.ldz,
+                               cudaMemcpyDeviceToDevice, vl.stream);
       });
-  }
-  if (e == cudaSuccess && cur)
-    e = cudaMemcpyAsync(vl.F0, vl.F1, sizeof(float) * (size_t)vl.V * vl.ldz,
-                        cudaMemcpyDeviceToDevice, vl.stream);
   if (e != cudaSuccess) return cuda_error(e, "rslb_closure_step");
   return RSLB_OK;
 }
