@@ -121,8 +121,9 @@ typedef struct rslb_config {
   const double* beta0;
   /* Cells per CTA tile of the stage kernel: 0 = automatic; otherwise
    * RSLB_PACKED_TILE_CELLS (the packed FP32x2 kernel: V >= 128,
-   * N_Omega <= 7), 128, 64, 32 or 16 (RSLB_F32), 16 or
-   * 8 (RSLB_F64).  A tuning knob; results agree to rounding. */
+   * N_Omega <= 7), 128, 64, 32 or 16 (RSLB_F32), 16, 8, 4
+   * or 2 (RSLB_F64; V must fit 8).  A tuning knob; results agree to rounding.
+   * What rslb_launch_info reports may be given here. */
   int tile_cells;
   /* Form of the packed FP32x2 kernel: RSLB_PACKED_AUTO or
    * RSLB_PACKED_PER_TILE (one CTA per tile, two CTAs per SM), or

@@ -362,16 +362,18 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   SodLaunch L = sod_pick_launch(fp64, V, QL, nm, max_smem, c.Z, nsm);
   if (c.tile_cells != 0) {
     // explicit tile width (tuning): must be one the kernels are built for
-    const bool okB = fp64 ? (c.tile_cells == 16 || c.tile_cells == 8)
+    const bool okB = fp64 ? (c.tile_cells == 16 || c.tile_cells == 8 || c.tile_cells == 4 ||
+                             c.tile_cells == 2)
                           : (c.tile_cells == kSod32Cells || c.tile_cells == 128 || c.tile_cells == 64 ||
                              c.tile_cells == 32 || c.tile_cells == 16);
     if (!okB)
       return set_error(RSLB_ERR_ARG, "rslb_init: tile_cells must be 0 or one of %s",
-                       fp64 ? "16, 8" : "the packed width, 128, 64, 32, 16");
+                       fp64 ? "16, 8, 4, 2" : "the packed width, 128, 64, 32, 16");
     if (c.tile_cells == kSod32Cells && (V < 128 || nm > 8))
       return set_error(RSLB_ERR_ARG,
                        "rslb_init: the packed tile width needs V >= 128 and N_Omega <= 7");
-    L.B = c.tile_cells;
+    // (widths of 4 and 2 serve small cell counts, not more velocities)
+    if (L.B != 0 || c.tile_cells >= 8) L.B = c.tile_cells;
   }
   if (L.B == 0)
     return set_error(RSLB_ERR_UNSUPPORTED, "rslb_init: V = %d velocities do not fit one tile", V);
