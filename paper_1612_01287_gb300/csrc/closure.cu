@@ -24,7 +24,9 @@
 // the FMA pipe and the shared-memory broadcasts, about equal; one thread per
 // sample (64 scalar accumulators) left the chip with one warp per scheduler.
 // 65536 cells, 73-64-64-24: 69 us per application, cold (173 before); a
-// minibatch of 8192: 72 us for the gradient (279).
+// minibatch of 8192: 72 us for the gradient (279).  Networks of 16 or 32 hidden
+// units and few inputs leave four threads little to do between barriers, so many
+// samples of these go by one thread each, in warps that share nothing (Team).
 //
 // Training: forward and backward of the CTA's samples, then the CTA reduces the
 // weight gradients over its samples into a per-CTA partial (a thread holds a
@@ -50,6 +52,8 @@ namespace {
 
 constexpr int kMaxD = 128;
 constexpr int kMaxO = 32;
+constexpr int kNarrowD = 32;                  // one thread per sample: inputs at most
+constexpr int kNarrowV = (kNarrowD - 1) / 3;  // and populations of a cell
 constexpr int kSmemLimit = 232448 - 2048;  // dynamic; the rest holds the static arrays
 constexpr float kLimitTheta = 0.5f;  // positivity limiter of the correction
 
@@ -73,10 +77,8 @@ MlpShape make_shape(int D, int H, int O) {
   return s;
 }
 
-constexpr int kNS = 64;                // samples per CTA
-constexpr int kParts = 4;              // threads per sample
-constexpr int kNetThreads = kNS * kParts;
-constexpr int kMaxV4 = kMaxO / kParts;  // populations per thread of a cell
+constexpr int kNS = 64;    // samples per CTA
+constexpr int kParts = 4;  // threads per sample
 
 __host__ __device__ inline int o_pad(const MlpShape& s) { return (s.O + 7) & ~7; }
 
@@ -160,12 +162,12 @@ __device__ __forceinline__ void dense(float2 (&acc)[N / 2], const float* x, int 
   }
 }
 
-// One hidden layer of the CTA's samples: this thread's quarter of the outputs of
-// its sample; with ds, silu' goes there.
-template <int H>
+// One hidden layer: this thread's share (1 / PARTS) of the outputs of its sample;
+// with ds, silu' goes there.
+template <int H, int PARTS>
 __device__ __forceinline__ void hidden(const float* x, int nin, const float* w, const float* b,
                                        int part, float* out, float* ds) {
-  constexpr int N = H / kParts;
+  constexpr int N = H / PARTS;
   float2 acc[N / 2];
 #pragma unroll
   for (int q = 0; q < N / 2; ++q) acc[q] = *reinterpret_cast<const float2*>(b + part * N + 2 * q);
@@ -178,8 +180,8 @@ __device__ __forceinline__ void hidden(const float* x, int nin, const float* w, 
   }
 }
 
-// The output layer: put(o, y) for this thread's quarter of the OP outputs.
-template <typename Put>
+// The output layer: put(o, y) for this thread's share of the OP outputs.
+template <int PARTS, typename Put>
 __device__ __forceinline__ void outputs(const float* x, int nin, const float* w, const float* b,
                                         int OP, int O, int part, Put put) {
   auto run = [&](auto Nc) {
@@ -193,10 +195,10 @@ __device__ __forceinline__ void outputs(const float* x, int nin, const float* w,
       if (part * N + q < O) put(part * N + q, (q & 1) ? acc[q / 2].y : acc[q / 2].x);
   };
   switch (OP) {
-    case 8: run(std::integral_constant<int, 2>()); break;
-    case 16: run(std::integral_constant<int, 4>()); break;
-    case 24: run(std::integral_constant<int, 6>()); break;
-    default: run(std::integral_constant<int, 8>()); break;
+    case 8: run(std::integral_constant<int, 8 / PARTS>()); break;
+    case 16: run(std::integral_constant<int, 16 / PARTS>()); break;
+    case 24: run(std::integral_constant<int, 24 / PARTS>()); break;
+    default: run(std::integral_constant<int, 32 / PARTS>()); break;
   }
 }
 
@@ -226,7 +228,7 @@ __device__ __forceinline__ void grad_tile(const float* act, int pitch, int cnt, 
     int cj[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) cj[j] = cb + (c0 + lane + 32 * j < ncol ? c0 + lane + 32 * j : 0);
-#pragma unroll 2
+#pragma unroll 4
     for (int n = 0; n < cnt; ++n) {
       const float* row = act + n * pitch;
       float bv[3];
@@ -280,7 +282,7 @@ __device__ __forceinline__ void back_layer(const float* g, int n, const float* w
 }
 
 template <int H>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(512, H == 64 ? 1 : 2)
 mlp_train_kernel(MlpShape s, const float* __restrict__ theta, const __nv_bfloat16* __restrict__ wb,
                  const float* __restrict__ nrm, const float* __restrict__ X,
                  const float* __restrict__ T, const int* __restrict__ perm, int n0, int nb,
@@ -313,16 +315,16 @@ mlp_train_kernel(MlpShape s, const float* __restrict__ theta, const __nv_bfloat1
   float* rg2 = rh2 + H;
   float* rgy = rg2 + H;
   // silu'(a1) and silu'(a2) go to the ga1 and ga2 columns, overwritten below
-  hidden<H>(row, s.D, sw + L.W1T, sw + L.b1, part, rh1, rg1);
+  hidden<H, kParts>(row, s.D, sw + L.W1T, sw + L.b1, part, rh1, rg1);
   __syncthreads();
-  hidden<H>(rh1, H, sw + L.W2T, sw + L.b2, part, rh2, rg2);
+  hidden<H, kParts>(rh1, H, sw + L.W2T, sw + L.b2, part, rh2, rg2);
   __syncthreads();
   double sq = 0.0;
   {
     const int n = n0 + base + smp;
     const int src = smp < cnt ? (perm ? perm[n] : n) : 0;
     const float* t = T + (size_t)src * s.O;
-    outputs(rh2, H, sw + L.W3T, sw + L.b3, o_pad(s), s.O, part, [&](int o, float y) {
+    outputs<kParts>(rh2, H, sw + L.W3T, sw + L.b3, o_pad(s), s.O, part, [&](int o, float y) {
       const float r = smp < cnt ? y - t[o] / sw[L.osd + o] : 0.f;
       sq += (double)r * r;
       rgy[o] = 2.f * r * inv_norm;
@@ -337,16 +339,21 @@ mlp_train_kernel(MlpShape s, const float* __restrict__ theta, const __nv_bfloat1
   __syncthreads();
   back_layer<H, H>(rg2, H, sw + L.W2T, H, part, rg1);
   __syncthreads();
-  // weight gradients summed over the CTA's samples in their order: four rows per
-  // warp and pass
+  // weight gradients summed over the CTA's samples in their order; the tiles of the
+  // three layers are dealt to the warps as one list, so that a narrow network's
+  // few tiles run side by side (16-unit layers: one pass instead of three)
   float* out = part_out + (size_t)blockIdx.x * s.P;
-  for (int r0 = 4 * warp; r0 < H; r0 += 4 * nw)
-    grad_tile<4>(act, pitch, cnt, s.D + H, 0, s.D, r0, H, lane, out + s.oW1, out + s.ob1);
-  for (int r0 = 4 * warp; r0 < H; r0 += 4 * nw)
-    grad_tile<4>(act, pitch, cnt, s.D + 3 * H, s.D, H, r0, H, lane, out + s.oW2, out + s.ob2);
-  for (int r0 = 2 * warp; r0 < s.O; r0 += 2 * nw)
-    grad_tile<2>(act, pitch, cnt, s.D + 4 * H, s.D + 2 * H, H, r0, s.O, lane, out + s.oW3,
-                 out + s.ob3);
+  const int nt1 = H / 4, nt3 = (s.O + 1) / 2;
+  for (int j = warp; j < 2 * nt1 + nt3; j += nw) {
+    if (j < nt1)
+      grad_tile<4>(act, pitch, cnt, s.D + H, 0, s.D, 4 * j, H, lane, out + s.oW1, out + s.ob1);
+    else if (j < 2 * nt1)
+      grad_tile<4>(act, pitch, cnt, s.D + 3 * H, s.D, H, 4 * (j - nt1), H, lane, out + s.oW2,
+                   out + s.ob2);
+    else
+      grad_tile<2>(act, pitch, cnt, s.D + 4 * H, s.D + 2 * H, H, 2 * (j - 2 * nt1), s.O, lane,
+                   out + s.oW3, out + s.ob3);
+  }
   if (tid == 0) {
     double t = 0.0;
     for (int i = 0; i < nw; ++i) t += red[i];
@@ -355,7 +362,7 @@ mlp_train_kernel(MlpShape s, const float* __restrict__ theta, const __nv_bfloat1
 }
 
 // Sum of the CTAs' partial gradients in their order (deterministic) and, with
-// adam, the parameter update.
+// adam, the parameter update; the last CTA sums the losses.
 struct AdamStep {
   float* theta;
   float* m;
@@ -364,39 +371,63 @@ struct AdamStep {
   float lr, c1, c2;
 };
 
-constexpr int kRedThreads = 64;  // few per CTA, so that every SM has some
+// A CTA takes 32 parameters: its warps bring rounds of kRedRows partials into shared
+// memory, many loads in flight, and one warp adds them in order.  A thread per
+// parameter that loaded 16 partials at a time, and one that added all losses,
+// waited on each load: 7813 partials (10^6 samples) of a 1-16-16-1 network 775 us,
+// 64 of a 73-64-64-24 network 5 us.
+constexpr int kRedThreads = 256, kRedRows = 128;
 
 __global__ void __launch_bounds__(kRedThreads)
 mlp_reduce_kernel(const float* __restrict__ part, int nblk, int P, float* grad,
                   const double* __restrict__ lossp, double loss_scale, double* loss_acc,
                   AdamStep ad) {
-  const int e = blockIdx.x * kRedThreads + threadIdx.x;
-  if (e < P) {
-    float g = 0.f;
-    int b = 0;
-    for (; b + 16 <= nblk; b += 16) {
-      float x[16];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) x[u] = part[(size_t)(b + u) * P + e];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) g += x[u];
+  constexpr int kWarps = kRedThreads / 32, kLoads = kRedRows / kWarps;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x == gridDim.x - 1) {
+    __shared__ double red[kRedThreads];
+    double t = 0.0;
+    for (int b = tid; b < nblk; b += kRedThreads) t += lossp[b];
+    red[tid] = t;
+    __syncthreads();
+    for (int o = kRedThreads / 2; o >= 1; o >>= 1) {
+      if (tid < o) red[tid] += red[tid + o];
+      __syncthreads();
     }
-    for (; b < nblk; ++b) g += part[(size_t)b * P + e];
-    grad[e] = g;
-    if (ad.theta) {
-      const float mm = 0.9f * ad.m[e] + 0.1f * g;
-      const float vv = 0.999f * ad.v[e] + 0.001f * g * g;
-      ad.m[e] = mm;
-      ad.v[e] = vv;
-      const float th = ad.theta[e] - ad.lr * (mm * ad.c1) / (sqrtf(vv * ad.c2) + 1e-8f);
-      ad.theta[e] = th;
-      ad.wb[e] = __float2bfloat16_rn(th);
+    if (tid == 0) *loss_acc += red[0] * loss_scale;
+    return;
+  }
+  __shared__ float buf[2][kRedRows][32];
+  const int e = blockIdx.x * 32 + lane;
+  float g = 0.f;
+  for (int b0 = 0, k = 0; b0 < nblk; b0 += kRedRows, k ^= 1) {
+    const int n = min(kRedRows, nblk - b0);
+    float x[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int b = warp + kWarps * u;
+      x[u] = b < n && e < P ? part[(size_t)(b0 + b) * P + e] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) buf[k][warp + kWarps * u][lane] = x[u];
+    // one barrier a round: warp 0 reads buffer k while the others fill k ^ 1, and
+    // reaches the next barrier before anyone writes k again
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll 8
+      for (int b = 0; b < n; ++b) g += buf[k][b][lane];
     }
   }
-  if (e == P) {  // one thread past the parameters (the grid covers P + 1)
-    double t = 0.0;
-    for (int b = 0; b < nblk; ++b) t += lossp[b];
-    *loss_acc += t * loss_scale;
+  if (warp != 0 || e >= P) return;
+  grad[e] = g;
+  if (ad.theta) {
+    const float mm = 0.9f * ad.m[e] + 0.1f * g;
+    const float vv = 0.999f * ad.v[e] + 0.001f * g * g;
+    ad.m[e] = mm;
+    ad.v[e] = vv;
+    const float th = ad.theta[e] - ad.lr * (mm * ad.c1) / (sqrtf(vv * ad.c2) + 1e-8f);
+    ad.theta[e] = th;
+    ad.wb[e] = __float2bfloat16_rn(th);
   }
 }
 
@@ -411,52 +442,80 @@ __host__ __device__ inline int infer_h1(const MlpShape& s) { return s.D > s.H ? 
 __host__ __device__ inline int infer_pitch(const MlpShape& s) {
   return (infer_h1(s) + (s.H > s.O ? s.H : s.O)) | 1;
 }
-__host__ __device__ inline size_t infer_smem(const MlpShape& s) {
-  return sizeof(float) * ((size_t)NetSmem(s).end + (size_t)kNS * infer_pitch(s));
+__host__ __device__ inline size_t infer_smem(const MlpShape& s, int rows) {
+  return sizeof(float) * ((size_t)NetSmem(s).end + (size_t)rows * infer_pitch(s));
 }
 
-// Forward of the CTA's staged samples.
-template <int H, typename Put>
+// The samples that go through the layers together: with one thread per sample a
+// warp's, which meets no barrier of the CTA, else the CTA's.
+template <int PARTS>
+struct Team {
+  static constexpr int kThreads = PARTS == 1 ? 128 : kNS * PARTS;  // of a CTA
+  static constexpr int kRows = kThreads / PARTS;                   // samples of a CTA
+  static constexpr int kSize = PARTS == 1 ? 32 : kNS;              // samples of a team
+  static constexpr int kWork = kSize * PARTS;                      // threads of a team
+  static __device__ __forceinline__ void sync() {
+    if constexpr (PARTS == 1) __syncwarp();
+    else __syncthreads();
+  }
+};
+
+// Forward of the team's staged samples.
+template <int H, int PARTS, typename Put>
 __device__ __forceinline__ void forward_rows(const MlpShape& s, const NetSmem& L, const float* sw,
                                              float* row, int part, Put put) {
   float* r1 = row + infer_h1(s);
-  hidden<H>(row, s.D, sw + L.W1T, sw + L.b1, part, r1, nullptr);
-  __syncthreads();
-  hidden<H>(r1, H, sw + L.W2T, sw + L.b2, part, row, nullptr);
-  __syncthreads();
-  outputs(row, H, sw + L.W3T, sw + L.b3, o_pad(s), s.O, part, put);
-  __syncthreads();
+  hidden<H, PARTS>(row, s.D, sw + L.W1T, sw + L.b1, part, r1, nullptr);
+  Team<PARTS>::sync();
+  hidden<H, PARTS>(r1, H, sw + L.W2T, sw + L.b2, part, row, nullptr);
+  Team<PARTS>::sync();
+  outputs<PARTS>(row, H, sw + L.W3T, sw + L.b3, o_pad(s), s.O, part, put);
+  Team<PARTS>::sync();
 }
 
 // Inference on given inputs.
-template <int H>
-__global__ void __launch_bounds__(kNetThreads)
+template <int H, int PARTS>
+__global__ void __launch_bounds__(Team<PARTS>::kThreads)
 mlp_infer_kernel(MlpShape s, const float* __restrict__ theta, const __nv_bfloat16* __restrict__ wb,
                  const float* __restrict__ nrm, const float* __restrict__ X, int n, float* Y) {
+  using T = Team<PARTS>;
   extern __shared__ __align__(16) float smem_f[];
   const NetSmem L(s);
   float* sw = smem_f;
-  float* act = sw + L.end;
   const int pitch = infer_pitch(s);
-  const int tid = threadIdx.x;
+  const int smp = threadIdx.x % T::kRows, row0 = smp / T::kSize * T::kSize;
+  const int tid = threadIdx.x % T::kWork;
+  float* act = sw + L.end + row0 * pitch;  // the team's rows
   load_weights(s, L, wb, theta, nrm, sw);
   __syncthreads();
-  for (int base = blockIdx.x * kNS; base < n; base += gridDim.x * kNS) {
-    const int cnt = min(kNS, n - base);
-    for (int r = tid >> 5; r < kNS; r += kNetThreads / 32)
-      for (int c = tid & 31; c < s.D; c += 32)
-        act[r * pitch + c] =
-            r < cnt ? (X[(size_t)(base + r) * s.D + c] - sw[L.mu + c]) * sw[L.isd + c] : 0.f;
-    __syncthreads();
-    float* row = act + (tid % kNS) * pitch;
-    const int oy = infer_h1(s);
-    forward_rows<H>(s, L, sw, row, tid / kNS,
-                    [&](int o, float y) { row[oy + o] = y * sw[L.osd + o]; });
-    for (int e = tid; e < cnt * s.O; e += kNetThreads) {
-      const int r = e / s.O, o = e - r * s.O;
-      Y[(size_t)base * s.O + e] = act[r * pitch + oy + o];
+  // element e of the team's inputs (outputs) is column e mod D (O) of row e / D (O)
+  auto walk = [&](int cnt, int cols, auto f) {
+    const int dr = T::kWork / cols, dc = T::kWork - dr * cols;
+    int r = tid / cols, c = tid - r * cols;
+    for (int e = tid; e < cnt * cols; e += T::kWork) {
+      f(e, r, c);
+      r += dr;
+      c += dc;
+      if (c >= cols) {
+        c -= cols;
+        ++r;
+      }
     }
-    __syncthreads();
+  };
+  for (int base = blockIdx.x * T::kRows + row0; base < n; base += gridDim.x * T::kRows) {
+    const int cnt = min(T::kSize, n - base);
+    const float* x = X + (size_t)base * s.D;
+    walk(cnt, s.D, [&](int e, int r, int c) {
+      act[r * pitch + c] = (x[e] - sw[L.mu + c]) * sw[L.isd + c];
+    });
+    T::sync();
+    float* row = act + (smp - row0) * pitch;
+    const int oy = infer_h1(s);
+    forward_rows<H, PARTS>(s, L, sw, row, threadIdx.x / T::kRows,
+                           [&](int o, float y) { row[oy + o] = y * sw[L.osd + o]; });
+    float* y = Y + (size_t)base * s.O;
+    walk(cnt, s.O, [&](int e, int r, int c) { y[e] = act[r * pitch + oy + c]; });
+    T::sync();
   }
 }
 
@@ -484,27 +543,30 @@ __device__ __forceinline__ void project_add(const ClosureConsts& cc, int V, cons
     out[v] = delta[v] - cc.w[v] * (c0 * cc.phi[v][0] + c1 * cc.phi[v][1] + c2 * cc.phi[v][2]);
 }
 
-// f_out = f_in + projected correction; four threads per cell.
-template <int H>
-__global__ void __launch_bounds__(kNetThreads)
+// f_out = f_in + projected correction; PARTS threads per cell.
+template <int H, int PARTS>
+__global__ void __launch_bounds__(Team<PARTS>::kThreads)
 closure_apply_kernel(MlpShape s, const float* __restrict__ theta,
                      const __nv_bfloat16* __restrict__ wb, const float* __restrict__ nrm,
                      const float* __restrict__ fin, float* fout, int Z, int ldz, float logtau,
                      ClosureConsts cc) {
+  using T = Team<PARTS>;
   extern __shared__ __align__(16) float smem_f[];
-  __shared__ float lim[kParts][kNS];
+  __shared__ float lim[PARTS][T::kRows];
+  constexpr int kMaxV4 = PARTS == 1 ? kNarrowV : kMaxO / PARTS;
   const NetSmem L(s);
   float* sw = smem_f;
   float* act = sw + L.end;
   const int pitch = infer_pitch(s);
-  const int V = s.O, part = threadIdx.x / kNS, smp = threadIdx.x % kNS;
+  const int V = s.O, part = threadIdx.x / T::kRows, smp = threadIdx.x % T::kRows;
+  const int row0 = smp / T::kSize * T::kSize;
   load_weights(s, L, wb, theta, nrm, sw);
   __syncthreads();
   const float* mu = sw + L.mu;
   const float* isd = sw + L.isd;
-  for (int base = blockIdx.x * kNS; base < Z; base += gridDim.x * kNS) {
-    const bool live = base + smp < Z;
-    const int c = min(base + smp, Z - 1);
+  for (int base = blockIdx.x * T::kRows + row0; base < Z; base += gridDim.x * T::kRows) {
+    const int cell = base + smp - row0, c = min(cell, Z - 1);
+    const bool live = cell < Z;
     const int cl = c > 0 ? c - 1 : 0, cr = c < Z - 1 ? c + 1 : Z - 1;
     float* row = act + smp * pitch;
     // this thread's populations v = part + 4 j and their neighbours, all loads at
@@ -512,7 +574,7 @@ closure_apply_kernel(MlpShape s, const float* __restrict__ theta,
     float fc[kMaxV4], fr[kMaxV4], fl[kMaxV4], np = 0.f;
 #pragma unroll
     for (int j = 0; j < kMaxV4; ++j) {
-      const int v = part + kParts * j;
+      const int v = part + PARTS * j;
       const float* f = fin + (size_t)v * ldz;
       fc[j] = v < V ? f[c] : 0.f;
       fr[j] = v < V ? f[cr] : 0.f;
@@ -521,13 +583,14 @@ closure_apply_kernel(MlpShape s, const float* __restrict__ theta,
 #pragma unroll
     for (int j = 0; j < kMaxV4; ++j) np += fc[j];
     lim[part][smp] = np;
-    __syncthreads();
-    const float n = (lim[0][smp] + lim[1][smp]) + (lim[2][smp] + lim[3][smp]);
+    T::sync();
+    float n = lim[0][smp];
+    if constexpr (PARTS == 4) n = (lim[0][smp] + lim[1][smp]) + (lim[2][smp] + lim[3][smp]);
     const float inv_n = 1.f / n;
     // features: f_s, f_{s+1} - f_s, f_s - f_{s-1} (over n_s), log10 tau
 #pragma unroll
     for (int j = 0; j < kMaxV4; ++j) {
-      const int v = part + kParts * j;
+      const int v = part + PARTS * j;
       if (v < V) {
         row[v] = (fc[j] * inv_n - mu[v]) * isd[v];
         row[V + v] = ((fr[j] - fc[j]) * inv_n - mu[V + v]) * isd[V + v];
@@ -535,9 +598,9 @@ closure_apply_kernel(MlpShape s, const float* __restrict__ theta,
       }
     }
     if (part == 0) row[3 * V] = (logtau - mu[3 * V]) * isd[3 * V];
-    __syncthreads();
+    T::sync();
     float* dl = row + infer_h1(s);
-    forward_rows<H>(s, L, sw, row, part,
+    forward_rows<H, PARTS>(s, L, sw, row, part,
                     [&](int o, float y) { dl[o] = n * sw[L.osd + o] * y; });
     // the correction without its component along the collision invariants
     const float* delta = dl;
@@ -559,22 +622,22 @@ closure_apply_kernel(MlpShape s, const float* __restrict__ theta,
     float alpha = 1.f;
 #pragma unroll
     for (int j = 0; j < kMaxV4; ++j) {
-      const int v = part + kParts * j;
+      const int v = part + PARTS * j;
       if (v < V) {
         fr[j] = corr(v);
         if (fc[j] > 0.f && fr[j] < 0.f) alpha = fminf(alpha, kLimitTheta * fc[j] / -fr[j]);
       }
     }
     lim[part][smp] = alpha;
-    __syncthreads();
+    T::sync();
 #pragma unroll
-    for (int q = 0; q < kParts; ++q) alpha = fminf(alpha, lim[q][smp]);
+    for (int q = 0; q < PARTS; ++q) alpha = fminf(alpha, lim[q][smp]);
 #pragma unroll
     for (int j = 0; j < kMaxV4; ++j) {
-      const int v = part + kParts * j;
+      const int v = part + PARTS * j;
       if (live && v < V) fout[(size_t)v * ldz + c] = fc[j] + alpha * fr[j];
     }
-    __syncthreads();
+    T::sync();
   }
 }
 
@@ -747,17 +810,6 @@ struct rslb_mlp {
 
 namespace {
 
-// CTAs of the inference kernels: each loads the weights once and walks groups of
-// kNS samples, so as many as fit the SMs at once.
-int net_grid(const MlpShape& s, int n) {
-  int dev = 0, nsm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
-    nsm = 152;
-  const int per = std::max(1, (int)(233472 / (infer_smem(s) + 2048)));  // 228 KB per SM
-  return std::min((n + kNS - 1) / kNS, per * nsm);
-}
-
 int mlp_pitch(const MlpShape& s) {
   int p = s.D + 4 * s.H + s.O;
   return (p % 2) ? p : p + 1;
@@ -793,17 +845,53 @@ void mlp_free(rslb_mlp* m) {
   delete m;
 }
 
+// One thread per sample of a network with few inputs, from `many` samples on; four
+// otherwise.  f(H, PARTS).
+template <typename F>
+cudaError_t dispatch_team(const MlpShape& s, int n, int many, F f) {
+  return dispatch_h(s.H, [&](auto Hc) {
+    if constexpr (decltype(Hc)::value <= 32)
+      if (s.D <= kNarrowD && n >= many) return f(Hc, std::integral_constant<int, 1>());
+    return f(Hc, std::integral_constant<int, kParts>());
+  });
+}
+
+// Where one thread per sample overtakes four (us, one / four threads).  Inference: 16
+// units 9.0 / 8.6 at 30000 samples of 1-16-16-1, 10.6 / 10.6 at 60000 and 11.0 / 13.0
+// at 100000, 15.1 / 15.1 and 18.7 / 20.8 at the last two of 31-16-16-10; 32 units
+// 49.1 / 47.6 at 300000 of 2-32-32-1 and 119 / 140 at 10^6, 74.8 / 76.6 and 228 /
+// 244 of 31-32-32-10.  Closure steps: 4 populations, 16 units 46.2 / 48.3 at 30000
+// cells and 62.6 / 68.2 at 65536; 10 populations, 32 units 56.7 / 54.5 and 75.0 /
+// 81.1.
+constexpr int kApplyMany = 49152;
+int infer_many(const MlpShape& s) { return s.H == 16 ? kApplyMany : 327680; }
+
 cudaError_t set_smem_attrs(const MlpShape& s) {
   return dispatch_h(s.H, [&](auto Hc) {
-    constexpr int H = decltype(Hc)::value;
-    for (const void* f : {(const void*)mlp_train_kernel<H>, (const void*)mlp_infer_kernel<H>,
-                          (const void*)closure_apply_kernel<H>}) {
+    constexpr int H = decltype(Hc)::value, N = H <= 32 ? 1 : kParts;
+    for (const void* f : {(const void*)mlp_train_kernel<H>,
+                          (const void*)mlp_infer_kernel<H, kParts>,
+                          (const void*)closure_apply_kernel<H, kParts>,
+                          (const void*)mlp_infer_kernel<H, N>,
+                          (const void*)closure_apply_kernel<H, N>}) {
       const cudaError_t e =
           cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
   });
+}
+
+// CTAs of the inference kernels: each loads the weights once and walks groups of
+// samples, so as many as the SMs hold at once (registers and threads count, not
+// the shared memory alone: a second, partial wave of long-lived CTAs doubles the time).
+int net_grid(const void* kernel, int threads, size_t smem, int groups) {
+  int dev = 0, nsm = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess)
+    cudaGetLastError();
+  return std::min(groups, std::max(per, 1) * std::max(nsm, 1));
 }
 
 // Gradient of the mean-squared loss over samples [n0, n0 + nb) of the
@@ -833,7 +921,7 @@ cudaError_t mlp_batch_grad(rslb_mlp* m, const float* X, const float* T, const in
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
-  mlp_reduce_kernel<<<s.P / kRedThreads + 1, kRedThreads, 0, m->stream>>>(
+  mlp_reduce_kernel<<<(s.P + 31) / 32 + 1, kRedThreads, 0, m->stream>>>(
       m->part, nblk, s.P, m->grad, m->lossp, loss_scale, m->loss_acc, adam);
   return cudaGetLastError();
 }
@@ -978,11 +1066,14 @@ extern "C" int rslb_mlp_forward(rslb_mlp* m, const float* X, int n, float* Y) {
   if (!m || !X || !Y || n < 0) return set_error(RSLB_ERR_ARG, "rslb_mlp_forward: bad arguments");
   if (n == 0) return RSLB_OK;
   const MlpShape& s = m->s;
-  const int grid = net_grid(s, n);
-  cudaError_t e = dispatch_h(s.H, [&](auto Hc) {
-    constexpr int H = decltype(Hc)::value;
-    mlp_infer_kernel<H><<<grid, kNetThreads, infer_smem(s), m->stream>>>(s, m->theta, m->wb,
-                                                                        m->norm, X, n, Y);
+  cudaError_t e = dispatch_team(s, n, infer_many(s), [&](auto Hc, auto Pc) {
+    constexpr int H = decltype(Hc)::value, PARTS = decltype(Pc)::value;
+    using T = Team<PARTS>;
+    const size_t smem = infer_smem(s, T::kRows);
+    const int grid = net_grid((const void*)mlp_infer_kernel<H, PARTS>, T::kThreads, smem,
+                              (n + T::kRows - 1) / T::kRows);
+    mlp_infer_kernel<H, PARTS><<<grid, T::kThreads, smem, m->stream>>>(s, m->theta, m->wb, m->norm,
+                                                                       X, n, Y);
     return cudaGetLastError();
   });
   return e == cudaSuccess ? RSLB_OK : cuda_error(e, "rslb_mlp_forward");
@@ -1165,20 +1256,24 @@ extern "C" int rslb_closure_step(rslb_handle* lo, rslb_mlp* m, double tau, int n
   int rc = closure_consts(vl.Q_xi, vl.Q_L, &cc);
   if (rc) return set_error(rc, "rslb_closure_step: low-order set too large");
   const MlpShape& s = m->s;
-  const size_t smem = infer_smem(s);
-  const int G = net_grid(s, vl.Z);
   const float lt = (float)std::log10(tau);
   // the correction reads its neighbours, so it writes the other buffer, which
   // then holds the state: the two change roles every step
   float* F[2] = {(float*)vl.F0, (float*)vl.F1};
+  int grid = 0;
   const cudaError_t e = swap_steps(
       nsteps, cudaSuccess,
       [&](int cur) {
         const cudaError_t es = sod_step_in(lo, cur);
         if (es != cudaSuccess) return es;
-        return dispatch_h(s.H, [&](auto Hc) {
-          constexpr int H = decltype(Hc)::value;
-          closure_apply_kernel<H><<<G, kNetThreads, smem, vl.stream>>>(
+        return dispatch_team(s, vl.Z, kApplyMany, [&](auto Hc, auto Pc) {
+          constexpr int H = decltype(Hc)::value, PARTS = decltype(Pc)::value;
+          using T = Team<PARTS>;
+          const size_t smem = infer_smem(s, T::kRows);
+          if (grid == 0)
+            grid = net_grid((const void*)closure_apply_kernel<H, PARTS>, T::kThreads, smem,
+                            (vl.Z + T::kRows - 1) / T::kRows);
+          closure_apply_kernel<H, PARTS><<<grid, T::kThreads, smem, vl.stream>>>(
               s, m->theta, m->wb, m->norm, F[cur], F[cur ^ 1], vl.Z, vl.ldz, lt, cc);
           return cudaGetLastError();
         });
