@@ -126,7 +126,7 @@ typedef struct rslb_config {
    * What rslb_launch_info reports may be given here. */
   int tile_cells;
   /* Form of the packed FP32x2 kernel: RSLB_PACKED_AUTO or
-   * RSLB_PACKED_PER_TILE (one CTA per tile, two CTAs per SM), or
+   * RSLB_PACKED_PER_TILE (one CTA per tile, two or three per SM), or
    * RSLB_PACKED_PERSISTENT (one CTA per SM walking the tiles with two tile
    * buffers and warp-specialised cell and sweep groups; RSLB_ERR_ARG where it
    * does not fit: it needs V <= ~700, Z >= RSLB_PACKED_TILE_CELLS + 8).  Both
@@ -282,11 +282,12 @@ typedef struct rslb_sod_batch rslb_sod_batch;
  * Set up nruns shock tubes.  A run with dt = 0 (constant tau only) gets
  * dt = t_end / ceil(t_end / dt_max) with dt_max = min(cfl dz / max|xi|,
  * dt_over_tau * tau), i.e. it reaches t_end exactly after its own number of
- * steps; a run with dt > 0 takes round(t_end / dt) steps of dt.  Runs are grouped by velocity
- * count; each group is advanced by one launch per RK stage that walks the
- * tiles of its runs (runs with fewer steps drop out as they finish), the
- * groups side by side on streams that fork from and join the caller's.  With autotune, the tile kernel and CTAs per SM of each group are
- * chosen by timing the candidates on the actual state.
+ * steps; a run with dt > 0 takes round(t_end / dt) steps of dt.  Runs are grouped by
+ * velocity count; each group is advanced by one launch per RK stage that walks
+ * the tiles of its runs (runs with fewer steps drop out as they finish), the
+ * groups side by side on streams that fork from and join the caller's.  With
+ * autotune, the tile kernel of each group is chosen by timing the candidates on
+ * the actual state, once per velocity set and power of two of cells.
  * Errors: RSLB_ERR_ARG, RSLB_ERR_UNSUPPORTED, RSLB_ERR_ALLOC, RSLB_ERR_CUDA.
  */
 int rslb_sod_batch_init(rslb_sod_batch** b, const rslb_sod_run* runs, int nruns,
@@ -307,8 +308,8 @@ int rslb_sod_batch_info(const rslb_sod_batch* b, long long* max_steps, long long
 /* Per-run step count and time step. */
 int rslb_sod_batch_run_info(const rslb_sod_batch* b, int run, long long* nsteps, double* dt);
 
-/* The tuner's choice for velocity group g (groups in ascending V): tile
- * width (cells per CTA) and CTAs per SM; returns RSLB_ERR_ARG past the last. */
+/* The tile width (cells per CTA) of velocity group g (groups in ascending V) and
+ * the CTAs of it that an SM holds; returns RSLB_ERR_ARG past the last. */
 int rslb_sod_batch_tuning(const rslb_sod_batch* b, int g, int* V, int* tile_cells,
                           int* ctas_per_sm);
 

@@ -857,11 +857,18 @@ void batch_free(rslb_sod_batch* b) {
   delete b;
 }
 
-// Tiles of one class per resident CTA and launch, at most, when classes run side
-// by side: a CTA that holds its place for a few tiles only lets the block
-// scheduler fill in other classes; the cap keeps the launches of finished
-// runs (whose CTAs return at once) short.
+// CTAs of a class's launches: a place on the GPU each when the class is alone, up to
+// kBatchWaves for every place when classes run side by side.  A CTA that holds its
+// place for a few tiles only lets the block scheduler fill in other classes; the
+// cap keeps the launches of finished runs (whose CTAs return at once) short.
+// Alone, one wave is the faster: 16 tubes of 1000 x 150 122 us per step against
+// 134 with up to four waves, 64 of 4000 x 150 1086 against 1109.
 constexpr int kBatchWaves = 4;
+
+int batch_grid(int ctas_per_sm, int nsm, int ntasks, bool alone) {
+  return (int)std::min((long long)ntasks,
+                       (long long)ctas_per_sm * nsm * (alone ? 1 : kBatchWaves));
+}
 
 // nsteps steps of every class.  The classes share nothing, so each is a chain of
 // its own on its own stream: a class whose tiles do not fill the GPU, or whose
@@ -880,7 +887,7 @@ cudaError_t batch_enqueue(rslb_sod_batch* b, int nsteps) {
     for (int n = 0; n < nsteps; ++n)
       for (int stage = 0; stage < 3 && e == cudaSuccess; ++stage)
         e = sod_batch_stage_launch<T>(
-            c.B, c.smem, std::min(c.ntasks, c.ctas_per_sm * b->nsm * (fork ? kBatchWaves : 1)),
+            c.B, c.smem, batch_grid(c.ctas_per_sm, b->nsm, c.ntasks, b->cls.size() == 1),
             (const SodRunDesc<T>*)c.runs_dev, c.tasks_dev, c.ntasks, b->step_dev, n, stage,
             b->err, c.V, c.QL, c.nm, st, c.B == kSod32Cells ? c.maps_dev : nullptr);
     if (st != b->stream) {
@@ -898,15 +905,18 @@ cudaError_t batch_enqueue(rslb_sod_batch* b, int nsteps) {
   return cudaGetLastError();
 }
 
-// Tuning results of this process: (device, FP64, V, Q_L, N_Omega + 1) ->
-// (tile cells, CTAs per SM).
+// Tuning results of this process: (device, FP64, V, Q_L, N_Omega + 1, log2 of the
+// class's cells) -> tile cells.  The width that fills the GPU with few cells is not
+// the fastest with many: 64 tubes of 4000 x 300 ran 2.27 ms per step on the 32
+// cells that 16 tubes of 1000 had chosen, 1.60 on the packed kernel.
 struct TuneKey {
-  int dev, fp64, V, QL, nm;
+  int dev, fp64, V, QL, nm, size;
   bool operator<(const TuneKey& o) const {
-    return std::tie(dev, fp64, V, QL, nm) < std::tie(o.dev, o.fp64, o.V, o.QL, o.nm);
+    return std::tie(dev, fp64, V, QL, nm, size) <
+           std::tie(o.dev, o.fp64, o.V, o.QL, o.nm, o.size);
   }
 };
-std::map<TuneKey, std::pair<int, int>> g_tune;
+std::map<TuneKey, int> g_tune;
 std::mutex g_tune_mu;
 
 template <typename T>
@@ -928,6 +938,7 @@ int batch_build_classes(rslb_sod_batch* b, int autotune) {
     const int V = b->h[order[i]]->V, nm = b->h[order[i]]->nm;
     size_t j = i;
     while (j < order.size() && b->h[order[j]]->V == V && b->h[order[j]]->nm == nm) ++j;
+    const bool alone = i == 0 && j == order.size();
     SodClass c{};
     c.V = V;
     c.QL = QL;
@@ -977,15 +988,14 @@ int batch_build_classes(rslb_sod_batch* b, int autotune) {
     // candidate tile kernels for this V (the automatic choice first); a
     // choice already timed in this process for the same device, precision
     // and velocity set is reused
-    const TuneKey key{dev, b->fp64 ? 1 : 0, V, QL, nm};
-    int cachedB = 0, cachedK = 0;
+    long long cells = 0;
+    for (size_t q = i; q < j; ++q) cells += b->h[order[q]]->cfg.Z;
+    const TuneKey key{dev, b->fp64 ? 1 : 0, V, QL, nm, std::ilogb((double)cells)};
+    int cachedB = 0;
     if (autotune) {
       std::lock_guard<std::mutex> lk(g_tune_mu);
       auto it = g_tune.find(key);
-      if (it != g_tune.end()) {
-        cachedB = it->second.first;
-        cachedK = it->second.second;
-      }
+      if (it != g_tune.end()) cachedB = it->second;
     }
     std::vector<int> cands = {cachedB ? cachedB : c.B};
     if (autotune && !cachedB) {
@@ -996,55 +1006,49 @@ int batch_build_classes(rslb_sod_batch* b, int autotune) {
             !(B == kSod32Cells && (V < 128 || nm > 8)))
           cands.push_back(B);
     }
+    // each candidate as it would be launched
+    const bool timing = autotune && !cachedB;
     float best = 1e30f;
-    int bestB = c.B, bestK = 1;
-    for (int B : cands) {
+    int bestB = cands[0];
+    for (size_t ic = 0; ic < cands.size() && timing; ++ic) {
+      const int B = cands[ic];
       make_tasks(B);
       SodTask* td = nullptr;
       if (cudaMalloc((void**)&td, sizeof(SodTask) * tasks.size()) != cudaSuccess)
         return set_error(RSLB_ERR_ALLOC, "rslb_sod_batch_init: cudaMalloc failed");
       cudaMemcpy(td, tasks.data(), sizeof(SodTask) * tasks.size(), cudaMemcpyHostToDevice);
       const size_t smem = sod_stage_smem_bytes(b->fp64, B, V, QL, nm);
-      const int maxk = (smem * 2 + 4096 <= (size_t)max_smem + 1024) ? 2 : 1;
-      const bool timing = autotune && !cachedB;
-      for (int k = 1; k <= (timing ? maxk : 1); ++k) {
-        float ms = 0.f;
-        if (timing) {
-          cudaEvent_t e0, e1;
-          cudaEventCreate(&e0);
-          cudaEventCreate(&e1);
-          // stage 0 reads F0 and writes F1 only: safe to repeat
-          sod_batch_stage_launch<T>(B, smem, k * b->nsm, (const SodRunDesc<T>*)c.runs_dev, td,
-                                    (int)tasks.size(), b->step_dev, 0, 0, b->err, V, QL, nm,
-                                    b->stream,
-                                    B == kSod32Cells ? c.maps_dev : nullptr);
-          cudaEventRecord(e0, b->stream);
-          for (int rep = 0; rep < 3; ++rep)
-            sod_batch_stage_launch<T>(B, smem, k * b->nsm, (const SodRunDesc<T>*)c.runs_dev, td,
-                                      (int)tasks.size(), b->step_dev, 0, 0, b->err, V, QL, nm,
-                                      b->stream,
-                                      B == kSod32Cells ? c.maps_dev : nullptr);
-          cudaEventRecord(e1, b->stream);
-          cudaEventSynchronize(e1);
-          cudaEventElapsedTime(&ms, e0, e1);
-          cudaEventDestroy(e0);
-          cudaEventDestroy(e1);
-        }
-        if (!timing || ms < best) {
-          best = ms;
-          bestB = B;
-          bestK = cachedB ? cachedK : k;
-        }
+      const int grid =
+          batch_grid(sod_batch_resident(b->fp64, B, smem), b->nsm, (int)tasks.size(), alone);
+      float ms = 0.f;
+      cudaEvent_t e0, e1;
+      cudaEventCreate(&e0);
+      cudaEventCreate(&e1);
+      // stage 0 reads F0 and writes F1 only: safe to repeat
+      for (int rep = 0; rep < 4; ++rep) {
+        if (rep == 1) cudaEventRecord(e0, b->stream);
+        sod_batch_stage_launch<T>(B, smem, grid, (const SodRunDesc<T>*)c.runs_dev, td,
+                                  (int)tasks.size(), b->step_dev, 0, 0, b->err, V, QL, nm,
+                                  b->stream, B == kSod32Cells ? c.maps_dev : nullptr);
+      }
+      cudaEventRecord(e1, b->stream);
+      cudaEventSynchronize(e1);
+      cudaEventElapsedTime(&ms, e0, e1);
+      cudaEventDestroy(e0);
+      cudaEventDestroy(e1);
+      if (ms < best) {
+        best = ms;
+        bestB = B;
       }
       cudaFree(td);
     }
-    if (autotune && !cachedB) {
+    if (timing) {
       std::lock_guard<std::mutex> lk(g_tune_mu);
-      g_tune[key] = {bestB, bestK};
+      g_tune[key] = bestB;
     }
     c.B = bestB;
-    c.ctas_per_sm = bestK;
     c.smem = sod_stage_smem_bytes(b->fp64, bestB, V, QL, nm);
+    c.ctas_per_sm = sod_batch_resident(b->fp64, bestB, c.smem);
     make_tasks(bestB);
     c.ntasks = (int)tasks.size();
     if (cudaMalloc((void**)&c.tasks_dev, sizeof(SodTask) * tasks.size()) != cudaSuccess)

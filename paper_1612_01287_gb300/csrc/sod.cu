@@ -914,6 +914,32 @@ cudaError_t sod32_batch_launch(size_t smem, int grid, const SodRunDesc<float>* r
                                const SodTask* tasks, int ntasks, const long long* step, int step_off,
                                int stage, int* err, const void* maps, cudaStream_t st);
 
+const void* sod32_batch_function(size_t smem);
+
+int sod_batch_resident(bool fp64, int B, size_t smem) {
+  const void* f = nullptr;
+  int nt = kNT;
+  if (fp64) {
+    if (B == 16) f = (const void*)sod_batch_kernel<double, 16, kNT>;
+    if (B == 8) f = (const void*)sod_batch_kernel<double, 8, kNT>;
+  } else {
+    if (B == 128) f = (const void*)sod_batch_kernel<float, 128, kNT>;
+    if (B == 64) f = (const void*)sod_batch_kernel<float, 64, kNT>;
+    if (B == 32) f = (const void*)sod_batch_kernel<float, 32, kNT>;
+    if (B == 16) f = (const void*)sod_batch_kernel<float, 16, kNT>;
+    if (B == kSod32Cells) {
+      f = sod32_batch_function(smem);
+      nt = kSod32Threads;
+    }
+  }
+  int n = 0;
+  if (!f || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, nt, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  return std::max(n, 1);
+}
+
 // Batched stages: all runs of a class share V (so nseg and the tile width).
 template <typename T, int B>
 static cudaError_t batch_b(size_t smem, int grid, const SodRunDesc<T>* runs, const SodTask* tasks,

@@ -130,6 +130,8 @@ cudaError_t sod_batch_stage_launch(int B, size_t smem, int grid, const SodRunDes
                                    const SodTask* tasks, int ntasks, const long long* step,
                                    int step_off, int stage, int* err, int V, int QL, int nm, cudaStream_t st,
                                    const void* maps = nullptr);
+// CTAs of the batched stage kernel of tile width B that an SM holds at once.
+int sod_batch_resident(bool fp64, int B, size_t smem);
 size_t sod_stage_smem_bytes(bool fp64, int B, int V, int QL, int nm);
 
 // Per-cell coefficients c''_{k,m} (FP64) of f^eq for given (n, T, beta) per

@@ -238,6 +238,10 @@ cudaError_t sod32_batch_launch(size_t smem, int grid, const SodRunDesc<float>* r
   return cudaGetLastError();
 }
 
+const void* sod32_batch_function(size_t smem) {
+  return three_ctas(smem) ? (const void*)sod32_batch_kernel<3> : (const void*)sod32_batch_kernel<2>;
+}
+
 size_t sod32_map_bytes() { return sizeof(CUtensorMap); }
 
 // The four tensor maps of one run (see sod32_batch_kernel); false if the
