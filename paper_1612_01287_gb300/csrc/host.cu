@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/rslb.h"
+#include "chains.h"
 #include "host_common.h"
 #include "rslb_device.cuh"
 #include "sod.cuh"
@@ -783,6 +784,7 @@ extern "C" void rslb_destroy(rslb_handle* h) {
 // ---------------------------------------------------------------------------
 struct SodClass {
   int V, QL, nm, B, ctas_per_sm;
+  int chain;  // 0: the caller's stream; c: side stream c - 1
   size_t smem;
   void* runs_dev;  // SodRunDesc<T>[nr]
   SodTask* tasks_dev;
@@ -804,8 +806,8 @@ struct rslb_sod_batch {
   int nsm;
   cudaGraphExec_t graph;
   bool graph_failed;
-  // one stream per class after the first (empty: all classes on `stream`), and
-  // the events that fork them from and join them to `stream`
+  // the streams of the chains after the first (empty: all classes on `stream`),
+  // and the events that fork them from and join them to `stream`
   std::vector<cudaStream_t> side;
   std::vector<cudaEvent_t> joined;
   cudaEvent_t forked;
@@ -824,11 +826,20 @@ void batch_free_streams(rslb_sod_batch* b) {
   b->forked = nullptr;
 }
 
-// The side streams; without them the classes run one after another.
+// Most chains of a batch: the SMs are shared by then, and a batch of many velocity
+// sets should not take a stream, an event and a graph branch for each.
+constexpr int kBatchChains = 16;
+
+// The classes (heaviest first) over the chains, and the side streams; without
+// streams the classes run one after another.
 void batch_make_streams(rslb_sod_batch* b) {
+  std::vector<double> load;
+  for (const SodClass& c : b->cls) load.push_back((double)c.V * c.ntasks * c.B);
+  const std::vector<int> chain = assign_chains(load, kBatchChains);
+  for (size_t i = 0; i < b->cls.size(); ++i) b->cls[i].chain = chain[i];
   if (b->cls.size() < 2) return;
   bool ok = cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming) == cudaSuccess;
-  for (size_t i = 1; i < b->cls.size() && ok; ++i) {
+  for (size_t i = 1; i < std::min<size_t>(b->cls.size(), kBatchChains) && ok; ++i) {
     cudaStream_t s = nullptr;
     cudaEvent_t e = nullptr;
     ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
@@ -871,33 +882,31 @@ int batch_grid(int ctas_per_sm, int nsm, int ntasks, bool alone) {
 }
 
 // nsteps steps of every class.  The classes share nothing, so each is a chain of
-// its own on its own stream: a class whose tiles do not fill the GPU, or whose
-// last wave is nearly empty, leaves the SMs to the others instead of holding
-// them up three times a step.  The step counter advances once, after all of
-// them; a launch knows its step within the call (step_off).
+// its own on its own stream (past kBatchChains, classes follow one another in a
+// chain): a class whose tiles do not fill the GPU, or whose last wave is nearly
+// empty, leaves the SMs to the others instead of holding them up three times a
+// step.  The step counter advances once, after all of them; a launch knows its
+// step within the call (step_off).
 template <typename T>
 cudaError_t batch_enqueue(rslb_sod_batch* b, int nsteps) {
   cudaError_t e = cudaSuccess;
   const bool fork = !b->side.empty();
   if (fork) e = cudaEventRecord(b->forked, b->stream);
-  for (size_t i = 0; i < b->cls.size() && e == cudaSuccess; ++i) {
-    const SodClass& c = b->cls[i];
-    cudaStream_t st = fork && i > 0 ? b->side[i - 1] : b->stream;
-    if (st != b->stream) e = cudaStreamWaitEvent(st, b->forked, 0);
+  for (size_t i = 0; i < b->side.size() && e == cudaSuccess; ++i)
+    e = cudaStreamWaitEvent(b->side[i], b->forked, 0);
+  for (const SodClass& c : b->cls) {
+    cudaStream_t st = fork && c.chain > 0 ? b->side[c.chain - 1] : b->stream;
     for (int n = 0; n < nsteps; ++n)
       for (int stage = 0; stage < 3 && e == cudaSuccess; ++stage)
         e = sod_batch_stage_launch<T>(
             c.B, c.smem, batch_grid(c.ctas_per_sm, b->nsm, c.ntasks, b->cls.size() == 1),
             (const SodRunDesc<T>*)c.runs_dev, c.tasks_dev, c.ntasks, b->step_dev, n, stage,
             b->err, c.V, c.QL, c.nm, st, c.B == kSod32Cells ? c.maps_dev : nullptr);
-    if (st != b->stream) {
-      // joined even after an error, so that a capture on `stream` can end
-      const cudaError_t j = cudaEventRecord(b->joined[i - 1], st);
-      if (e == cudaSuccess) e = j;
-    }
   }
-  for (size_t i = 0; i < b->joined.size() && fork; ++i) {
-    const cudaError_t j = cudaStreamWaitEvent(b->stream, b->joined[i], 0);
+  // joined even after an error, so that a capture on `stream` can end
+  for (size_t i = 0; i < b->side.size(); ++i) {
+    cudaError_t j = cudaEventRecord(b->joined[i], b->side[i]);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(b->stream, b->joined[i], 0);
     if (e == cudaSuccess) e = j;
   }
   if (e != cudaSuccess) return e;
