@@ -281,8 +281,9 @@ __global__ void bj_eo_kernel(int Q, const double* __restrict__ xw, const double*
 //   - the moments and equilibrium of a run by another warp meanwhile;
 //   - R follows the batch (see the host): few runs spread over all SMs.
 // 112 runs of Q_xi 3 .. 100, Q_L = 2, 50 steps: 0.99 ms (23.9 ms with
-// blocks of four padded runs and the full matrix); for Q_xi = 100 the products
-// alone are 6k of the ~13.7k cycles of a stage.
+// blocks of four padded runs and the full matrix).  The FP64 pipe is busy 51% of
+// the time on the SMs in use; between, warps wait at the two barriers of a stage
+// and for their FP64 results.
 // Shared memory per column: f_n and f [Q], s|d [Q] twice (a stage reads one
 // copy and writes the other), E s|O d [Q].
 // ---------------------------------------------------------------------------
@@ -557,7 +558,7 @@ struct rslb_bjorken {
   double* mp[2];
   int mp_cur;  // which moment buffer describes the state (F0)
   float* ytmp;       // K^P f in the sorted order
-  long long* uoff;   // per sorted run: its offset there
+  long long* uoff;   // per sorted run: its offset in the callers' order
   long long* step_dev;           // steps taken, read by the stage kernels for their times
   cudaGraphExec_t tc_graph[2];   // kTcGraphSteps steps, per parity of mp_cur at the start
   bool tc_graph_failed;

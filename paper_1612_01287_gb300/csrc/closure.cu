@@ -20,11 +20,13 @@
 // The network's kernels use four threads per sample (64 samples per CTA; training
 // 128), each with a quarter of every layer's outputs in packed FP32x2
 // accumulators; activations pass between layers through shared memory, and a
-// warp's lanes share the weights they read (broadcasts).  What bounds them is
-// the FMA pipe and the shared-memory broadcasts, about equal; one thread per
+// warp's lanes share the weights they read (broadcasts).  What bounds them are
+// the shared-memory broadcasts and latency (application: shared memory 56% of its
+// rate, issue slots 45%, FMA pipe 21%, 16 warps per SM; training: 64 CTAs of 16
+// warps for a minibatch of 8192, issue slots 51% on their SMs); one thread per
 // sample (64 scalar accumulators) left the chip with one warp per scheduler.
-// 65536 cells, 73-64-64-24: 69 us per application, cold (173 before); a
-// minibatch of 8192: 72 us for the gradient (279).  Networks of 16 or 32 hidden
+// 65536 cells, 73-64-64-24: 78 us per application (163 with one thread per sample);
+// a minibatch of 8192 with its update: 76 us (240).  Networks of 16 or 32 hidden
 // units and few inputs leave four threads little to do between barriers, so many
 // samples of these go by one thread each, in warps that share nothing (Team).
 //

@@ -2,8 +2,7 @@
 //
 // Per cell: the first and second moments (Eq. macro_jk), Landau matching
 // (Sec. II E, Eqs. E_landau-pi_val) in FP64 and the 14 fields of rslb.h.
-// Five sums are formed directly, each with a non-negative weight, as the
-// factored Landau form needs them:
+// The factored Landau form needs five sums, each with a non-negative weight:
 //   N+- = sum f (1 +- xi),  A+- = sum f p (1 +- xi)^2,  D = sum f p (1 - xi^2);
 // the conserved currents follow exactly:
 //   N^t = (N+ + N-)/2,  N^z = (N+ - N-)/2,  T^tz = (A+ - A-)/4,
@@ -26,9 +25,10 @@
 // TwoSum errors in a plain FP32 sum of the low part.  Two neighbouring cells
 // share a thread in packed FP32x2 arithmetic.  GB300's FP64 pipe is a small
 // fraction of its FP32 rate, so FP64 is used only for the per-cell finish.
-// What bounds it: the FMA pipe, 33 packed instructions per velocity and pair of
-// cells (55 with five sums); 65536 x 600: 87 us cold (118 with five sums
-// in four chunks of 64 threads and chunk sums in FP64).
+// What bounds it: the latency of its loads.  65536 x 600: 87 us cold, DRAM 23% of
+// peak, FMA pipe 22%, issue slots 31%, warps waiting on a load for 16 of the ~20
+// cycles between their instructions at 26 warps per SM (118 us with five sums in
+// four chunks of 64 threads and chunk sums in FP64).
 // FP64 populations: plain FP64 products and sums, one cell per thread.
 #include "rslb_device.cuh"
 #include "sod.cuh"

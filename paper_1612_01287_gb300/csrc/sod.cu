@@ -1,7 +1,7 @@
 // sod.cu -- fused RK-stage kernel of the R-SLB Sod shock tube (sm_103a).
 //
-// One CTA owns a tile of B consecutive cells (128, 64, 32 or 16 for FP32, 16
-// or 8 for FP64) and all V velocities.  A stage (Eq. rk3) is one launch:
+// One CTA owns a tile of B consecutive cells (128, 64, 32 or 16 for FP32, 16, 8,
+// 4 or 2 for FP64) and all V velocities.  A stage (Eq. rk3) is one launch:
 //   1. the tile plus a 4-cell halo on each side is staged in shared memory
 //      with 16-byte cp.async copies (velocity-major rows; boundary tiles map
 //      out-of-domain cells through the boundary condition);
@@ -30,8 +30,10 @@
 // 7, f^eq 6, update 7, the rest halo and idle lanes), 99 with five moment sums,
 // IEEE divisions, FP64 maxima and predicated-off orders.  65536 x 600: 4.23 ms
 // per stage (7.34 before); 256 x 60 on 2-cell tiles: 18 us (79 on 16-cell
-// tiles with the quadrature for a_{l,m}).  FP32 with few velocities: the
-// latency of the per-cell phases.
+// tiles with the quadrature for a_{l,m}).  FP32: latency.  With few velocities
+// that of the per-cell phases (V = 24: FP64 pipe 15%, FMA 12%, most warps at a
+// barrier while the cells' FP64 runs), else of the sweep, whose code also has to
+// fit the instruction cache (V = 60: FMA pipe 18%, issue slots 31%).
 #include <algorithm>
 #include <type_traits>
 
@@ -810,11 +812,14 @@ SodLaunch sod_pick_launch(bool fp64, int V, int QL, int nm, int max_smem, int Z,
   const size_t half = (size_t)max_smem / 2 - 2048;
   if (!fp64) {
     // packed FP32x2 kernel: whole rows per thread, so it needs enough rows to
-    // fill a CTA, N_Omega <= 7, and two CTAs per SM
+    // fill a CTA, N_Omega <= 7, and two CTAs per SM at least.  65536 cells, us per
+    // step, packed / best scalar tile: V = 150 244 / 274, V = 300 388 / 425, V = 600
+    // 715 / 758
     if (V >= 128 && nm <= 8 && sod32_smem_bytes(V, QL) <= half) return {kSod32Cells, 0};
     // few velocities: wide tiles share each tile's fixed costs among more
-    // cells and give the row segments more cells (65536 cells, V = 24: 0.15 ms
-    // per step with 128-cell tiles, 0.18 with 64, 0.26 with 32)
+    // cells and give the row segments more cells (65536 cells, us per step with
+    // 128-, 64- and 32-cell tiles: V = 24 91, 124, 184; V = 60 144, 162, 220; few
+    // cells run faster on narrower tiles: 4000 x 24 40, 32, 29)
     if (V < 48 && smem_base<float>(V, 128, QL, nm) <= half) return {128, 0};
     if (V < 128 && smem_base<float>(V, 64, QL, nm) <= half) return {64, 0};
     if (smem_base<float>(V, 32, QL, nm) <= half) return {32, 0};
