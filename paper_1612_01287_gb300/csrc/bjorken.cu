@@ -1052,42 +1052,51 @@ extern "C" int rslb_bjorken_read(rslb_bjorken* b, double* out, int out_on_device
   return bj_check_err(b);
 }
 
-// One value per population of the tensor-core path's buffer `src` (sorted order)
-// to host memory in the callers' order, through F1 (scratch between steps);
-// synchronises.
-static int bj_read_runs(rslb_bjorken* b, const float* src, void* out, const char* what) {
-  bj_gather_kernel<<<b->nruns, 256, 0, b->stream>>>(b->QL, b->rq, b->roff, b->uoff, src,
-                                                    (float*)b->F1);
-  cudaError_t e = cudaGetLastError();
+// One value per population (es bytes) of the buffer `src` (sorted order) to host
+// memory in the callers' order; synchronises.  The tensor-core path reorders on
+// the device, through F1 (scratch between steps), from kGatherBytes on; below, the
+// extra launch costs more than the host's pass (one run of Q_xi = 64 38 us through
+// the device, 30 without; 48 runs of 200, 115 KB, 42 and 41; 400 runs of 100, 480 KB,
+// 50 and 77).
+constexpr size_t kGatherBytes = 128 * 1024;
+
+static int bj_read_runs(rslb_bjorken* b, const void* src, size_t es, void* out, const char* what) {
+  const size_t bytes = es * (size_t)b->total_state;
+  bool sorted = true;  // the callers' order is the sorted one
+  for (int s = 0; s < b->nruns && sorted; ++s) sorted = b->user_of_sorted[s] == s;
+  std::vector<unsigned char> tmp;
+  cudaError_t e = cudaSuccess;
+  bool reorder = false;
+  if (!sorted && b->uoff && bytes >= kGatherBytes) {
+    bj_gather_kernel<<<b->nruns, 256, 0, b->stream>>>(b->QL, b->rq, b->roff, b->uoff,
+                                                      (const float*)src, (float*)b->F1);
+    e = cudaGetLastError();
+    src = b->F1;
+  } else if (!sorted) {
+    reorder = true;
+    tmp.resize(bytes);
+  }
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(out, b->F1, sizeof(float) * (size_t)b->total_state,
-                        cudaMemcpyDeviceToHost, b->stream);
+    e = cudaMemcpyAsync(reorder ? tmp.data() : out, src, bytes, cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return cuda_error(e, what);
+  if (reorder) {
+    std::vector<long long> uoff(b->nruns + 1, 0);
+    std::vector<int> uq(b->nruns);
+    for (int s = 0; s < b->nruns; ++s) uq[b->user_of_sorted[s]] = b->rq_h[s];
+    for (int r = 0; r < b->nruns; ++r) uoff[r + 1] = uoff[r] + (long long)b->QL * uq[r];
+    for (int s = 0; s < b->nruns; ++s)
+      std::memcpy((unsigned char*)out + es * uoff[b->user_of_sorted[s]], tmp.data() + es * b->roff_h[s],
+                  es * (size_t)b->QL * b->rq_h[s]);
+  }
   return bj_check_err(b);
 }
 
 extern "C" int rslb_bjorken_get_state(rslb_bjorken* b, void* f) {
   clear_error();
   if (!b || !f) return set_error(RSLB_ERR_ARG, "rslb_bjorken_get_state: NULL argument");
-  if (b->uoff) return bj_read_runs(b, (const float*)b->state, f, "rslb_bjorken_get_state");
   const size_t es = b->precision == RSLB_F64 ? sizeof(double) : sizeof(float);
-  std::vector<unsigned char> tmp(es * (size_t)b->total_state);
-  cudaError_t e = cudaMemcpyAsync(tmp.data(), b->state, tmp.size(), cudaMemcpyDeviceToHost,
-                                  b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  if (e != cudaSuccess) return cuda_error(e, "rslb_bjorken_get_state");
-  // sorted -> caller order
-  std::vector<long long> uoff(b->nruns + 1, 0);
-  std::vector<int> uq(b->nruns);
-  for (int s = 0; s < b->nruns; ++s) uq[b->user_of_sorted[s]] = b->rq_h[s];
-  for (int r = 0; r < b->nruns; ++r) uoff[r + 1] = uoff[r] + (long long)b->QL * uq[r];
-  for (int s = 0; s < b->nruns; ++s) {
-    const int r = b->user_of_sorted[s];
-    std::memcpy((unsigned char*)f + es * uoff[r], tmp.data() + es * b->roff_h[s],
-                es * (size_t)b->QL * b->rq_h[s]);
-  }
-  return bj_check_err(b);
+  return bj_read_runs(b, b->state, es, f, "rslb_bjorken_get_state");
 }
 
 extern "C" int rslb_bjorken_set_state(rslb_bjorken* b, const void* f) {
@@ -1169,7 +1178,7 @@ extern "C" int rslb_bjorken_kp_apply(rslb_bjorken* b, void* y) {
   a.err = b->err;
   cudaError_t e = bj_tc_stage_launch(a, b->ntc, b->tc_smem, b->stream);
   if (e != cudaSuccess) return cuda_error(e, "rslb_bjorken_kp_apply");
-  return bj_read_runs(b, b->ytmp, y, "rslb_bjorken_kp_apply");
+  return bj_read_runs(b, b->ytmp, sizeof(float), y, "rslb_bjorken_kp_apply");
 }
 
 extern "C" void rslb_bjorken_destroy(rslb_bjorken* b) {
