@@ -560,7 +560,8 @@ struct rslb_bjorken {
   float* ytmp;       // K^P f in the sorted order
   long long* uoff;   // per sorted run: its offset in the callers' order
   long long* step_dev;           // steps taken, read by the stage kernels for their times
-  cudaGraphExec_t tc_graph[2];   // kTcGraphSteps steps, per parity of mp_cur at the start
+  // kTcGraphSteps[i] steps, per parity of mp_cur at the start
+  cudaGraphExec_t tc_graph[2][2];
   bool tc_graph_failed;
 };
 
@@ -574,8 +575,9 @@ void bj_free(rslb_bjorken* b) {
                   b->step_dev};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  for (cudaGraphExec_t g : b->tc_graph)
-    if (g) cudaGraphExecDestroy(g);
+  for (auto& len : b->tc_graph)
+    for (cudaGraphExec_t g : len)
+      if (g) cudaGraphExecDestroy(g);
   delete b;
 }
 
@@ -924,9 +926,11 @@ extern "C" int rslb_bjorken_init(rslb_bjorken** out, const rslb_bjorken_run* run
 
 namespace {
 
-// Steps of a graph of the tensor-core path: an even count, so that the moment
-// buffers are back in their starting roles at its end.
-constexpr int kTcGraphSteps = 8;
+// Steps of the graphs of the tensor-core path: even counts, so that the moment
+// buffers are back in their starting roles at its end.  The short one takes short
+// calls and remainders: two steps of 400 runs of Q_xi = 100 154 us, 159 as plain
+// launches.
+constexpr int kTcGraphSteps[2] = {8, 2};
 
 // Enqueue nsteps RK3 steps of the tensor-core path: three stage launches each
 // (stage times from the device step counter and the step within the call, Tab.
@@ -964,17 +968,17 @@ cudaError_t bj_tc_enqueue(rslb_bjorken* b, int nsteps) {
   return e;
 }
 
-// Capture kTcGraphSteps steps for the current parity of mp_cur (non-default
+// Capture kTcGraphSteps[len] steps for the current parity of mp_cur (non-default
 // streams only: the legacy default stream cannot be captured).
-cudaError_t bj_tc_build_graph(rslb_bjorken* b) {
+cudaError_t bj_tc_build_graph(rslb_bjorken* b, int len) {
   const int par = b->mp_cur;
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  const cudaError_t le = bj_tc_enqueue(b, kTcGraphSteps);
+  const cudaError_t le = bj_tc_enqueue(b, kTcGraphSteps[len]);
   e = cudaStreamEndCapture(b->stream, &g);
   if (le != cudaSuccess) e = le;
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&b->tc_graph[par], g, 0);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&b->tc_graph[len][par], g, 0);
   if (g) cudaGraphDestroy(g);
   b->mp_cur = par;  // capture enqueued nothing
   return e;
@@ -991,21 +995,19 @@ extern "C" int rslb_bjorken_step(rslb_bjorken* b, int nsteps) {
   if (b->kp_mode == RSLB_KP_TF32X3) {
     e = cudaSuccess;
     int rest = nsteps;
-    if (b->stream != nullptr && nsteps >= kTcGraphSteps && !b->tc_graph_failed) {
-      if (!b->tc_graph[b->mp_cur]) {
-        e = bj_tc_build_graph(b);
-        if (e != cudaSuccess) {
-          // plain launches from here on (e.g. the caller's stream is being captured)
-          b->tc_graph[b->mp_cur] = nullptr;
-          b->tc_graph_failed = true;
-          cudaGetLastError();
-          e = cudaSuccess;
-        }
+    for (int len = 0; len < 2 && b->stream != nullptr; ++len) {
+      const int steps = kTcGraphSteps[len];
+      cudaGraphExec_t& graph = b->tc_graph[len][b->mp_cur];
+      if (rest >= steps && !graph && !b->tc_graph_failed &&
+          (e = bj_tc_build_graph(b, len)) != cudaSuccess) {
+        // plain launches from here on (e.g. the caller's stream is being captured)
+        graph = nullptr;
+        b->tc_graph_failed = true;
+        cudaGetLastError();
+        e = cudaSuccess;
       }
-      while (b->tc_graph[b->mp_cur] && rest >= kTcGraphSteps && e == cudaSuccess) {
-        e = cudaGraphLaunch(b->tc_graph[b->mp_cur], b->stream);
-        rest -= kTcGraphSteps;
-      }
+      for (; graph && !b->tc_graph_failed && rest >= steps && e == cudaSuccess; rest -= steps)
+        e = cudaGraphLaunch(graph, b->stream);
     }
     if (e == cudaSuccess && rest > 0) e = bj_tc_enqueue(b, rest);
     if (e != cudaSuccess) return cuda_error(e, "rslb_bjorken_step: launch");
