@@ -204,8 +204,7 @@ struct rslb_handle {
   SodLaunch launch;
   void* F[3];
   // tables in working precision
-  void* t_m3;
-  void* t_pk;
+  void* t_m3;  // the moment weights [V][4], then p_k [QL][2]
   void* t_xi;
   void* t_wp;
   void* t_L1k;
@@ -240,7 +239,7 @@ template <typename T>
 SodTables<T> tables_of(const rslb_handle* h) {
   SodTables<T> tb;
   tb.m3 = (const T*)h->t_m3;
-  tb.pk = (const T*)h->t_pk;
+  tb.pk = tb.m3 + 4 * (size_t)h->V;
   tb.xi = (const T*)h->t_xi;
   tb.wp = (const T*)h->t_wp;
   tb.kidx = h->t_kidx;
@@ -267,7 +266,7 @@ SodTablesF64 tables64_of(const rslb_handle* h) {
 void free_handle(rslb_handle* h) {
   if (!h) return;
   if (h->graph) cudaGraphExecDestroy(h->graph);
-  void* ptrs[] = {h->F[0], h->F[1], h->F[2], h->t_m3, h->t_pk, h->t_xi, h->t_wp, h->t_L1k, h->t_gL,
+  void* ptrs[] = {h->F[0], h->F[1], h->F[2], h->t_m3, h->t_xi, h->t_wp, h->t_L1k, h->t_gL,
                   h->t_gR, h->t_kidx, h->t_rowv, h->t_gl_t, h->t_gl_w, h->d_xi, h->d_p, h->d_wp,
                   h->d_L1k, h->d_mom, h->d_err, h->d_fields};
   for (void* p : ptrs)
@@ -457,15 +456,12 @@ extern "C" int rslb_init(rslb_handle** out, const rslb_config* cfg, void* stream
   auto up = [&](void** dst, const std::vector<double>& src) {
     return fp64 ? upload<double>(dst, src) : upload<float>(dst, src);
   };
-  if (!rc) rc = up(&h->t_m3, m3);
-  if (!rc) {
-    std::vector<double> pk(2 * (size_t)QL);  // p_k as hi + lo in the working precision
-    for (int k = 0; k < QL; ++k) {
-      pk[2 * k] = fp64 ? xk[k] : (double)(float)xk[k];
-      pk[2 * k + 1] = xk[k] - pk[2 * k];
-    }
-    rc = up(&h->t_pk, pk);
+  for (int k = 0; k < QL; ++k) {  // p_k as hi + lo in the working precision
+    const double hi = fp64 ? xk[k] : (double)(float)xk[k];
+    m3.push_back(hi);
+    m3.push_back(xk[k] - hi);
   }
+  if (!rc) rc = up(&h->t_m3, m3);
   if (!rc) rc = up(&h->t_xi, xiv);
   if (!rc) rc = up(&h->t_wp, wp);
   if (!rc) rc = up(&h->t_L1k, L1k);
