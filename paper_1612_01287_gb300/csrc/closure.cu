@@ -806,6 +806,8 @@ struct rslb_mlp {
   double* loss_acc;
   int* perm;
   int part_blocks;
+  int infer_places[2], apply_places[2];  // CTAs the GPU holds, [0]: four threads per
+                                         // sample, [1]: one
   int perm_n;
   long long adam_t;
 };
@@ -868,32 +870,47 @@ cudaError_t dispatch_team(const MlpShape& s, int n, int many, F f) {
 constexpr int kApplyMany = 49152;
 int infer_many(const MlpShape& s) { return s.H == 16 ? kApplyMany : 327680; }
 
-cudaError_t set_smem_attrs(const MlpShape& s) {
-  return dispatch_h(s.H, [&](auto Hc) {
-    constexpr int H = decltype(Hc)::value, N = H <= 32 ? 1 : kParts;
-    for (const void* f : {(const void*)mlp_train_kernel<H>,
-                          (const void*)mlp_infer_kernel<H, kParts>,
-                          (const void*)closure_apply_kernel<H, kParts>,
-                          (const void*)mlp_infer_kernel<H, N>,
-                          (const void*)closure_apply_kernel<H, N>}) {
-      const cudaError_t e =
-          cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-  });
+// CTAs of a kernel that the GPU holds at once.  The inference kernels' CTAs load the
+// weights once and walk groups of samples, so there are as many as this (registers
+// and threads count, not the shared memory alone: a second, partial wave of
+// long-lived CTAs doubles the time).
+cudaError_t places_of(const void* kernel, int threads, size_t smem, int* places) {
+  int dev = 0, nsm = 0, per = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+  *places = std::max(per, 1) * std::max(nsm, 1);
+  return e;
 }
 
-// CTAs of the inference kernels: each loads the weights once and walks groups of
-// samples, so as many as the SMs hold at once (registers and threads count, not
-// the shared memory alone: a second, partial wave of long-lived CTAs doubles the time).
-int net_grid(const void* kernel, int threads, size_t smem, int groups) {
-  int dev = 0, nsm = 0, per = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess)
-    cudaGetLastError();
-  return std::min(groups, std::max(per, 1) * std::max(nsm, 1));
+template <int H, int PARTS>
+cudaError_t prepare_team(rslb_mlp* m, int i) {
+  using T = Team<PARTS>;
+  const void* infer = (const void*)mlp_infer_kernel<H, PARTS>;
+  const void* apply = (const void*)closure_apply_kernel<H, PARTS>;
+  const size_t smem = infer_smem(m->s, T::kRows);
+  cudaError_t e = cudaSuccess;
+  for (const void* f : {infer, apply})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+  if (e == cudaSuccess) e = places_of(infer, T::kThreads, smem, &m->infer_places[i]);
+  if (e == cudaSuccess) e = places_of(apply, T::kThreads, smem, &m->apply_places[i]);
+  return e;
+}
+
+// Opts the network's kernels into large shared memory and counts their places.
+cudaError_t prepare_kernels(rslb_mlp* m) {
+  return dispatch_h(m->s.H, [&](auto Hc) {
+    constexpr int H = decltype(Hc)::value;
+    cudaError_t e =
+        cudaFuncSetAttribute((const void*)mlp_train_kernel<H>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    if (e == cudaSuccess) e = prepare_team<H, kParts>(m, 0);
+    if constexpr (H <= 32)
+      if (e == cudaSuccess && m->s.D <= kNarrowD) e = prepare_team<H, 1>(m, 1);
+    return e;
+  });
 }
 
 // Gradient of the mean-squared loss over samples [n0, n0 + nb) of the
@@ -972,7 +989,7 @@ extern "C" int rslb_mlp_create(rslb_mlp** out, int n_in, int n_hidden, int n_out
   }
   std::vector<float> nrm(2 * s.D + s.O, 1.f);
   for (int d = 0; d < s.D; ++d) nrm[d] = 0.f;  // mu = 0, inv_sd = 1, out_sd = 1
-  cudaError_t e = set_smem_attrs(m->s);
+  cudaError_t e = prepare_kernels(m);
   if (e == cudaSuccess)
     e = cudaMemcpy(m->norm, nrm.data(), sizeof(float) * nrm.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
@@ -1071,11 +1088,9 @@ extern "C" int rslb_mlp_forward(rslb_mlp* m, const float* X, int n, float* Y) {
   cudaError_t e = dispatch_team(s, n, infer_many(s), [&](auto Hc, auto Pc) {
     constexpr int H = decltype(Hc)::value, PARTS = decltype(Pc)::value;
     using T = Team<PARTS>;
-    const size_t smem = infer_smem(s, T::kRows);
-    const int grid = net_grid((const void*)mlp_infer_kernel<H, PARTS>, T::kThreads, smem,
-                              (n + T::kRows - 1) / T::kRows);
-    mlp_infer_kernel<H, PARTS><<<grid, T::kThreads, smem, m->stream>>>(s, m->theta, m->wb, m->norm,
-                                                                       X, n, Y);
+    const int grid = std::min((n + T::kRows - 1) / T::kRows, m->infer_places[PARTS == 1]);
+    mlp_infer_kernel<H, PARTS><<<grid, T::kThreads, infer_smem(s, T::kRows), m->stream>>>(
+        s, m->theta, m->wb, m->norm, X, n, Y);
     return cudaGetLastError();
   });
   return e == cudaSuccess ? RSLB_OK : cuda_error(e, "rslb_mlp_forward");
@@ -1262,7 +1277,6 @@ extern "C" int rslb_closure_step(rslb_handle* lo, rslb_mlp* m, double tau, int n
   // the correction reads its neighbours, so it writes the other buffer, which
   // then holds the state: the two change roles every step
   float* F[2] = {(float*)vl.F0, (float*)vl.F1};
-  int grid = 0;
   const cudaError_t e = swap_steps(
       nsteps, cudaSuccess,
       [&](int cur) {
@@ -1271,11 +1285,9 @@ extern "C" int rslb_closure_step(rslb_handle* lo, rslb_mlp* m, double tau, int n
         return dispatch_team(s, vl.Z, kApplyMany, [&](auto Hc, auto Pc) {
           constexpr int H = decltype(Hc)::value, PARTS = decltype(Pc)::value;
           using T = Team<PARTS>;
-          const size_t smem = infer_smem(s, T::kRows);
-          if (grid == 0)
-            grid = net_grid((const void*)closure_apply_kernel<H, PARTS>, T::kThreads, smem,
-                            (vl.Z + T::kRows - 1) / T::kRows);
-          closure_apply_kernel<H, PARTS><<<grid, T::kThreads, smem, vl.stream>>>(
+          const int grid =
+              std::min((vl.Z + T::kRows - 1) / T::kRows, m->apply_places[PARTS == 1]);
+          closure_apply_kernel<H, PARTS><<<grid, T::kThreads, infer_smem(s, T::kRows), vl.stream>>>(
               s, m->theta, m->wb, m->norm, F[cur], F[cur ^ 1], vl.Z, vl.ldz, lt, cc);
           return cudaGetLastError();
         });
