@@ -271,10 +271,11 @@ __device__ __forceinline__ void weno_scale(double& s1, double& s2, double& s3) {
   // would fall below zero, zero indicators and subnormal ones become subnormal:
   // their squares are 0.
   const int h1 = __double2hiint(s1), h2 = __double2hiint(s2), h3 = __double2hiint(s3);
-  const int sh = (max(h1, max(h2, h3)) & 0x7FF00000) - 0x3FF00000, least = max(sh, 0x00100000);
-  s1 = __hiloint2double(h1 < least ? 0 : h1 - sh, __double2loint(s1));
-  s2 = __hiloint2double(h2 < least ? 0 : h2 - sh, __double2loint(s2));
-  s3 = __hiloint2double(h3 < least ? 0 : h3 - sh, __double2loint(s3));
+  const int sh = (max(h1, max(h2, h3)) & 0x7FF00000) - 0x3FF00000;
+  auto shift = [&](int h) { return h < 0x00100000 ? 0 : max(h - sh, 0); };
+  s1 = __hiloint2double(shift(h1), __double2loint(s1));
+  s2 = __hiloint2double(shift(h2), __double2loint(s2));
+  s3 = __hiloint2double(shift(h3), __double2loint(s3));
 }
 // num/den, 0 where den is below the smallest normal number (the reciprocals
 // flush subnormal inputs, and a vanishing denominator means a vanishing correction)
